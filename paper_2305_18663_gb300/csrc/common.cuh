@@ -94,6 +94,7 @@ struct GraphDev {
 struct sbp_graph {
     int64_t n = 0, m = 0;
     int device = 0;
+    unsigned char *slab = nullptr;  // the one allocation behind the arrays below (but self_in)
     int32_t *op = nullptr, *ip = nullptr, *oc = nullptr, *ic = nullptr, *esrc = nullptr;
     int32_t *tw_oi = nullptr, *tw_io = nullptr;  // twin positions of each edge in the other CSR
     int32_t *self_in = nullptr;  // in-row positions of the self-loops
