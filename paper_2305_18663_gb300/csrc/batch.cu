@@ -267,6 +267,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
     __shared__ ModelOut sw;
     __shared__ SearchRec sr;
     __shared__ __int128 red[kBatchWarps];
+    __shared__ int2 mqueue[kBatchWarps][kMergeQueue];
     __shared__ unsigned s_job, s_nmov;
     __shared__ int s_stop, s_left, s_rounds, s_done, s_Bn, s_go, s_start, s_target, s_reload, s_slot;
     constexpr int V = 32 / G;  // movers per warp
@@ -353,7 +354,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                     for (int r = wid; r < B; r += kBatchWarps) {
                         int bs;
                         double bd;
-                        merge_best(md, sa.seed, rid, J.merge_x, r, bs, bd);
+                        merge_best(md, sa.seed, rid, J.merge_x, r, 0, 1, mqueue[wid], [](MergeSum &) {}, bs, bd);
                         if (lane == 0) {
                             J.best_s[r] = bs;
                             J.best_d[r] = bd;

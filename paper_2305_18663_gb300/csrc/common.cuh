@@ -482,6 +482,29 @@ __device__ __forceinline__ void Mat4(const ModelDev &md, int r, int s, int t, in
     Mts = sparse_probe_from(md, o_t, c_t, h4, s, k4);
 }
 
+// the four corner entries M[r][r], M[s][s], M[r][s], M[s][r]; on sparse rows
+// the two row offsets and then the four first probe slots are loaded
+// together (collisions continue one slot at a time)
+__device__ __forceinline__ void Mat4corner(const ModelDev &md, int r, int s, int &Mrr, int &Mss, int &Mrs, int &Msr) {
+    if (!md.sparse) {
+        const size_t B = (size_t)md.B;
+        Mrr = md.M[(size_t)r * B + r];
+        Mss = md.M[(size_t)s * B + s];
+        Mrs = md.M[(size_t)r * B + s];
+        Msr = md.M[(size_t)s * B + r];
+        return;
+    }
+    const uint32_t o_r = md.hoff[r], c_r = md.hoff[r + 1] - o_r;
+    const uint32_t o_s = md.hoff[s], c_s = md.hoff[s + 1] - o_s;
+    const uint32_t hr = sparse_hash(r), hs = sparse_hash(s);
+    const uint32_t h1 = hr & (c_r - 1), h2 = hs & (c_s - 1), h3 = hs & (c_r - 1), h4 = hr & (c_s - 1);
+    const int2 k1 = md.hkv[o_r + h1], k2 = md.hkv[o_s + h2], k3 = md.hkv[o_r + h3], k4 = md.hkv[o_s + h4];
+    Mrr = sparse_probe_from(md, o_r, c_r, h1, r, k1);
+    Mss = sparse_probe_from(md, o_s, c_s, h2, s, k2);
+    Mrs = sparse_probe_from(md, o_r, c_r, h3, s, k3);
+    Msr = sparse_probe_from(md, o_s, c_s, h4, r, k4);
+}
+
 // first i in a[lo, hi) with a[i] > t (one lane, binary search)
 __device__ __forceinline__ uint32_t lane_upper(const uint32_t *__restrict__ a, uint32_t lo, uint32_t hi, uint32_t t) {
     uint32_t n = hi - lo;
