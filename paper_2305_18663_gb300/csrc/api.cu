@@ -260,50 +260,9 @@ int upload_assignment(sbp_model *m, int32_t B, const int32_t *b) {
     return rebuild_blockmodel(m);
 }
 
-int64_t merge_key(double d) { return (int64_t)std::floor(d * 1048576.0 + 0.5); }
-
-// Alg. 1 "sort best_merges", "pop, merge c into c'": links in ascending
-// (key, r), pointer-based union (Section III-A (d)), stops at n_merges.
-// map[c] = new dense label, groups numbered by their smallest member.
-int64_t apply_merges(int32_t B, const std::vector<int32_t> &bs, const std::vector<double> &bd, int64_t n_merges,
-                     std::vector<int32_t> &map, int32_t &B_new) {
-    std::vector<std::pair<int64_t, int32_t>> it((size_t)B);
-    for (int32_t r = 0; r < B; ++r) it[(size_t)r] = {merge_key(bd[(size_t)r]), r};
-    std::sort(it.begin(), it.end());
-    std::vector<int32_t> parent((size_t)B);
-    std::iota(parent.begin(), parent.end(), 0);
-    auto find = [&](int32_t x) {
-        while (parent[(size_t)x] != x) {
-            parent[(size_t)x] = parent[(size_t)parent[(size_t)x]];
-            x = parent[(size_t)x];
-        }
-        return x;
-    };
-    int64_t done = 0;
-    for (size_t k = 0; k < it.size() && done < n_merges; ++k) {
-        const int32_t r = it[k].second, s = bs[(size_t)r];
-        if (s < 0) continue;
-        const int32_t a = find(r), c = find(s);
-        if (a == c) continue;
-        parent[(size_t)a] = c;
-        ++done;
-    }
-    std::vector<int32_t> label((size_t)B, -1);
-    map.assign((size_t)B, 0);
-    int32_t next = 0;
-    for (int32_t c = 0; c < B; ++c) {
-        const int32_t root = find(c);
-        if (label[(size_t)root] < 0) label[(size_t)root] = next++;
-        map[(size_t)c] = label[(size_t)root];
-    }
-    B_new = next;
-    return done;
-}
-
-int relabel_and_rebuild(sbp_model *m, const std::vector<int32_t> &map, int32_t B_new) {
-    SBP_CUDA(cudaMemcpyAsync(m->map, map.data(), map.size() * 4, cudaMemcpyHostToDevice, m->stream));
+// the labels through m->map, and the blockmodel of B_new blocks
+int relabel_and_rebuild(sbp_model *m, int32_t B_new) {
     SBP_TRY(launch_relabel(m, m->map));
-    SBP_CUDA(cudaStreamSynchronize(m->stream));
     SBP_TRY(ensure_capacity(m, B_new));  // dense or sparse for the new B
     m->B = B_new;
     return rebuild_blockmodel(m);
@@ -351,7 +310,7 @@ extern "C" void sbp_free_model(sbp_model_t *m) {
     void *ps[] = {m->b,        m->bnew,   m->M,        m->P,       m->Pc,     m->dout,  m->din,
                   m->rcp,      m->rcp32,  m->dsum,     m->dl,      m->partials, m->counters, m->status,
                   m->best_s,   m->best_d, m->map,      m->vcount,  m->movers, m->mcount, m->skip,
-                  m->items,    m->nbo,    m->nbi,      m->cta_tab};
+                  m->items,    m->nbo,    m->nbi,      m->cta_tab, m->merge_work};
     for (void *p : ps) model_free(p, st);
     for (int i = 0; i < 2; ++i) {
         if (m->side[i]) cudaStreamDestroy(m->side[i]);
@@ -504,21 +463,13 @@ extern "C" int sbp_merge_blocks(sbp_model_t *m, uint64_t round_id, int32_t n_mer
     if (!m) return fail(SBP_EINVAL, "sbp_merge_blocks: NULL model");
     if (n_merges < 1 || n_merges >= m->B) return fail(SBP_EINVAL, "sbp_merge_blocks: need 1 <= n_merges < B");
     int32_t rounds = 0;
-    int64_t left = n_merges;
-    std::vector<int32_t> bs, map;
-    std::vector<double> bd;
+    int32_t left = n_merges;
     while (left > 0 && m->B >= 2) {
-        const int32_t B = m->B;
         SBP_TRY(launch_merge_proposals(m, round_id + (uint64_t)rounds));
         ++rounds;
-        bs.resize((size_t)B);
-        bd.resize((size_t)B);
-        SBP_CUDA(cudaMemcpyAsync(bs.data(), m->best_s, (size_t)B * 4, cudaMemcpyDeviceToHost, m->stream));
-        SBP_CUDA(cudaMemcpyAsync(bd.data(), m->best_d, (size_t)B * 8, cudaMemcpyDeviceToHost, m->stream));
-        SBP_CUDA(cudaStreamSynchronize(m->stream));
-        int32_t Bn = B;
-        const int64_t done = apply_merges(B, bs, bd, left, map, Bn);
-        SBP_TRY(relabel_and_rebuild(m, map, Bn));
+        int32_t done = 0, Bn = m->B;
+        SBP_TRY(apply_merge_round(m, left, &done, &Bn));
+        SBP_TRY(relabel_and_rebuild(m, Bn));
         left -= done;
         if (done == 0) break;
     }
@@ -529,15 +480,9 @@ extern "C" int sbp_merge_blocks(sbp_model_t *m, uint64_t round_id, int32_t n_mer
 
 extern "C" int sbp_compact(sbp_model_t *m, int32_t *B_out) {
     if (!m) return fail(SBP_EINVAL, "sbp_compact: NULL model");
-    const int32_t B = m->B;
-    SBP_TRY(launch_vertex_count(m));
-    std::vector<int32_t> cnt((size_t)B), map((size_t)B, -1);
-    SBP_CUDA(cudaMemcpyAsync(cnt.data(), m->vcount, (size_t)B * 4, cudaMemcpyDeviceToHost, m->stream));
-    SBP_CUDA(cudaStreamSynchronize(m->stream));
-    int32_t next = 0;
-    for (int32_t c = 0; c < B; ++c)
-        if (cnt[(size_t)c] > 0) map[(size_t)c] = next++;
-    if (next != B) SBP_TRY(relabel_and_rebuild(m, map, next));
+    int32_t next = m->B;
+    SBP_TRY(compact_blocks(m, &next));
+    if (next != m->B) SBP_TRY(relabel_and_rebuild(m, next));
     if (B_out) *B_out = m->B;
     return SBP_OK;
 }

@@ -12,9 +12,9 @@
 //      no longer holds, and rebuilds the counts from it;
 //   1. (optional) the merge phase: per round, every block's best merge
 //      (one warp per block, the same scoring code as the per-graph kernel),
-//      the scores sorted in shared memory, the merges applied in order with
-//      a union-find until n_merges are done, the labels relabelled and the
-//      counts rebuilt; rounds repeat as the per-graph merge does;
+//      the merges applied (merge_apply.cuh, the per-graph code too) until
+//      n_merges are done, the labels relabelled and the counts rebuilt;
+//      rounds repeat as the per-graph merge does;
 //   2. the MCMC phase, per sweep:
 //      a. proposals, one thread per vertex (the same proposal as the
 //         per-graph pass), movers (s != r) appended to the graph's list;
@@ -45,7 +45,7 @@
 #include "sbp_check.h"
 #include "batch.h"
 #include "driver.h"
-#include "merge_dev.cuh"
+#include "merge_apply.cuh"
 #include "nodal_dev.cuh"
 
 namespace sbp {
@@ -211,39 +211,6 @@ __device__ void cta_rebuild(const GraphDev &g, const int32_t *b, const ModelOut 
     C = cta_sum_128(c, red);
 }
 
-// ascending sort of (key, idx) pairs, CTA-wide bitonic network (n a power
-// of two; the indices are distinct, so the order is total)
-__device__ void cta_sort_pairs(long long *key, int *idx, int n) {
-    for (int k = 2; k <= n; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < n; i += kBatchThreads) {
-                const int p = i ^ j;
-                if (p > i) {
-                    const bool up = (i & k) == 0;
-                    const bool gt = key[i] > key[p] || (key[i] == key[p] && idx[i] > idx[p]);
-                    if (gt == up) {
-                        const long long tk = key[i];
-                        key[i] = key[p];
-                        key[p] = tk;
-                        const int ti = idx[i];
-                        idx[i] = idx[p];
-                        idx[p] = ti;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
-__device__ __forceinline__ int uf_find(int *par, int x) {
-    while (par[x] != x) {
-        par[x] = par[par[x]];
-        x = par[x];
-    }
-    return x;
-}
-
 // b[v] = bnew[v] = map[b[v]] for every vertex
 __device__ void cta_relabel(int32_t *b, int32_t *bnew, int n, const int *map) {
     for (int v = threadIdx.x; v < n; v += kBatchThreads) {
@@ -268,6 +235,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
     __shared__ SearchRec sr;
     __shared__ __int128 red[kBatchWarps];
     __shared__ int2 mqueue[kBatchWarps][kMergeQueue];
+    __shared__ TeamShared tsh;
     __shared__ unsigned s_job, s_nmov;
     __shared__ int s_stop, s_left, s_rounds, s_done, s_Bn, s_go, s_start, s_target, s_reload, s_slot;
     constexpr int V = 32 / G;  // movers per warp
@@ -276,11 +244,16 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
     const unsigned gm = group_mask<G>();
     unsigned *cnt = reinterpret_cast<unsigned *>(bsm) + ((size_t)wid * V + gid) * group_words;
     // merge rounds and compaction (the same shared memory, used between
-    // sweeps only): sort keys and indices, union-find parents, labels
-    long long *skey = reinterpret_cast<long long *>(bsm);
-    int *sidx = reinterpret_cast<int *>(skey + blk_cap);
-    int *par = sidx + blk_cap;
-    int *smap = par + blk_cap;
+    // sweeps only): the merge application's work arrays, the label map
+    MergeApply mw;
+    mw.key = reinterpret_cast<unsigned long long *>(bsm);
+    mw.a0 = reinterpret_cast<int *>(mw.key + blk_cap);
+    mw.a1 = mw.a0 + blk_cap;
+    mw.x0 = mw.a1 + blk_cap;
+    mw.x1 = mw.x0 + blk_cap;
+    mw.mark = mw.x1 + blk_cap;
+    int *smap = mw.mark + blk_cap;
+    int *par = mw.a0;
     for (;;) {
         if (tid == 0) s_job = atomicAdd(queue, 1u);
         __syncthreads();
@@ -361,42 +334,16 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                         }
                     }
                     __syncthreads();
-                    int p2 = 1;
-                    while (p2 < B) p2 <<= 1;
-                    for (int i = tid; i < p2; i += kBatchThreads) {
-                        skey[i] = i < B ? score_key(J.best_d[i]) : LLONG_MAX;
-                        sidx[i] = i < B ? i : INT_MAX;
-                    }
-                    __syncthreads();
-                    cta_sort_pairs(skey, sidx, p2);
+                    CtaTeam team{tsh};
+                    int Bn;
+                    const int done = merge_apply(team, mw, B, J.best_s, J.best_d, s_left, smap, Bn);
                     if (tid == 0) {
-                        // ascending (score, block), pointer-based union, stop at
-                        // the merges still owed; groups numbered by their
-                        // smallest block
-                        for (int c = 0; c < B; ++c) par[c] = c;
-                        int done = 0;
-                        for (int q = 0; q < B && done < s_left; ++q) {
-                            const int r = sidx[q], s = J.best_s[r];
-                            if (s < 0) continue;
-                            const int a = uf_find(par, r), c = uf_find(par, s);
-                            if (a == c) continue;
-                            par[a] = c;
-                            ++done;
-                        }
-                        int *lab = reinterpret_cast<int *>(skey);
-                        for (int c = 0; c < B; ++c) lab[c] = -1;
-                        int next = 0;
-                        for (int c = 0; c < B; ++c) {
-                            const int root = uf_find(par, c);
-                            if (lab[root] < 0) lab[root] = next++;
-                            smap[c] = lab[root];
-                        }
                         s_done = done;
-                        s_Bn = next;
+                        s_Bn = Bn;
                         s_left -= done;
                         ++s_rounds;
-                        sa.md.B = next;
-                        sa.md.pstep = (2 * next + 31) / 32;
+                        sa.md.B = Bn;
+                        sa.md.pstep = (2 * Bn + 31) / 32;
                     }
                     __syncthreads();
                     cta_relabel(sw.b, md.bnew, n, smap);
@@ -550,12 +497,12 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
             __syncthreads();
             for (int v = tid; v < n; v += kBatchThreads) atomicAdd(&par[sw.b[v]], 1);
             __syncthreads();
+            CtaTeam team{tsh};
+            const int left = compact_map(team, B, par, smap);
             if (tid == 0) {
-                int next = 0;
-                for (int c = 0; c < B; ++c) smap[c] = par[c] > 0 ? next++ : -1;
-                s_Bn = next;
-                sa.md.B = next;
-                sa.md.pstep = (2 * next + 31) / 32;
+                s_Bn = left;
+                sa.md.B = left;
+                sa.md.pstep = (2 * left + 31) / 32;
                 s_slot = search_free_slot(sr);
             }
             __syncthreads();
@@ -726,7 +673,7 @@ int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, cons
     int V = tune.movers_per_warp == 4 ? 4 : tune.movers_per_warp == 2 ? 2 : 1;
     while (V > 1 && (size_t)kBatchWarps * V * group_words * 4 > kBatchSmemCap) V /= 2;
     // the merge rounds' and the compaction's arrays share that memory
-    const size_t smem = std::max((size_t)kBatchWarps * V * group_words * 4, (size_t)blk_cap * 20);
+    const size_t smem = std::max((size_t)kBatchWarps * V * group_words * 4, (size_t)blk_cap * (kMergeApplyBytes + 4));
     const int per_sm = tune.ctas_per_sm > 0 ? tune.ctas_per_sm : 2;
     const int grid = std::min(nj, sm_count_b() * per_sm);
     auto launch = [&](auto kern) -> int {

@@ -206,6 +206,8 @@ struct sbp_model {
     double *best_d = nullptr;
     int32_t *map = nullptr;
     int32_t *vcount = nullptr;
+    unsigned char *merge_work = nullptr;  // work arrays of the merge application
+    int32_t merge_work_B = 0;
     // nodal pass: proposals with s != r, in three lists by degree
     void *movers = nullptr;
     unsigned *mcount = nullptr;
@@ -594,6 +596,8 @@ int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_en
 int nb_rows_rebuild(sbp_model *m);       // block-labelled rows from m->b (nb_ok when there is memory)
 int nb_rows_after_commit(sbp_model *m);  // ... brought up to date after a commit
 int launch_merge_proposals(sbp_model *m, uint64_t round_id);
+int apply_merge_round(sbp_model *m, int32_t want, int32_t *done, int32_t *B_new);  // best proposals -> m->map
+int compact_blocks(sbp_model *m, int32_t *B_new);  // m->map dropping the empty blocks
 int launch_relabel(sbp_model *m, const int32_t *map_dev);
 int launch_vertex_count(sbp_model *m);
 int ensure_capacity(sbp_model *m, int32_t B);
