@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, SBP_DECIDE_MIN_BLOCKS) k_ev
             VertexCtx x;
             x.v = v; x.r = r; x.s = s;
             x.Kout = kout; x.Kin = kin; x.self = self; x.k = k;
-            evaluate_warp<DL32>(a, md, x, w2, [&](auto &&f) {
+            evaluate_warp<DL32, false>(a, md, x, w2, [&](auto &&f) {
                 for (int e = lane; e < D; e += 32) {
                     const int slot = list[e];
                     const unsigned cc = cnt[slot];
@@ -207,7 +207,7 @@ constexpr int kDirectChunks = 8;
 
 // one mover (v, s, w2) on the whole warp, counts in cnt[B] (all zero on entry
 // and on return), first touches in list
-template <bool DL32>
+template <bool DL32, bool EXACT>
 __device__ __forceinline__ void direct_mover(const DecideArgs &a, unsigned *cnt, int *list, int v, int s, uint64_t w2,
                                              Counts &c) {
     const int lane = threadIdx.x & 31;
@@ -250,7 +250,7 @@ __device__ __forceinline__ void direct_mover(const DecideArgs &a, unsigned *cnt,
     x.Kout = kout; x.Kin = kin; x.self = self; x.k = k;
     const int D = nl;
     if (lane == 0) c.entries += (unsigned)D;
-    evaluate_warp<DL32>(a, md, x, w2, [&](auto &&f) {
+    evaluate_warp<DL32, EXACT>(a, md, x, w2, [&](auto &&f) {
         for (int e = lane; e < D; e += 32) {
             const int t = list[e];
             const unsigned cc = cnt[t];
@@ -262,12 +262,48 @@ __device__ __forceinline__ void direct_mover(const DecideArgs &a, unsigned *cnt,
     __syncwarp();
 }
 
+// The proposals of vertices w, w + W, w + 2 W, ... of `count` (vertex(i) is
+// the i-th), drawn one per lane, and the evaluation of the movers among them,
+// one after another, on warp w of W.  Returns the lane's sum of its movers'
+// degrees.
+template <bool DL32, bool EXACT, class Vertex>
+__device__ __forceinline__ unsigned long long direct_vertices(const DecideArgs &a, unsigned *cnt, int *list, int64_t gw,
+                                                              int64_t nw, int64_t count, Vertex vertex, Counts &c) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long medges = 0;
+    for (int64_t j0 = 0; gw + j0 * nw < count; j0 += 32) {
+        const int64_t i = gw + (j0 + lane) * nw;
+        bool mover = false;
+        int pv = 0, ps = 0;
+        uint64_t pw = 0;
+        if (i < count) {
+            pv = vertex(i);
+            const Proposal p = propose_vertex(a.g, a.md, a.seed, a.sweep_id, pv);
+            if (p.s == p.r) {
+                c.proposed++;
+            } else {
+                mover = true;
+                ps = p.s;
+                pw = p.w2;
+                medges += (unsigned long long)p.k;
+            }
+        }
+        unsigned mask = __ballot_sync(0xffffffffu, mover);
+        while (mask) {
+            const int q = __ffs(mask) - 1;
+            mask &= mask - 1u;
+            const int v = __shfl_sync(0xffffffffu, pv, q), s = __shfl_sync(0xffffffffu, ps, q);
+            const uint64_t w2 = __shfl_sync(0xffffffffu, pw, q);
+            direct_mover<DL32, EXACT>(a, cnt, list, v, s, w2, c);
+        }
+    }
+    return medges;
+}
+
 // One warp per mover with direct-mapped counts.  FUSED = false: the movers
 // of list `bin`.  FUSED = true: the warps draw the proposals of the group's
-// vertices themselves, warp w taking the vertices w, w + W, w + 2W, ... of
-// the group (W warps in the grid; the group is sorted by descending degree,
-// so every warp gets a share of the largest rows), one per lane, then
-// evaluates its movers one after another.
+// vertices themselves (the group is sorted by descending degree, so every
+// warp gets a share of the largest rows).
 template <bool DL32, bool FUSED>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, SBP_DIRECT_MIN_BLOCKS) k_eval_warp_direct(DecideArgs a, int bin,
                                                                                            int warp_words) {
@@ -286,41 +322,43 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, SBP_DIRECT_MIN_BLOCKS) k_ev
         const int64_t count = *(volatile unsigned *)&a.mcount[bin];
         for (int64_t q = gw; q < count; q += nw) {
             const Mover mv = mlist[q];
-            direct_mover<DL32>(a, cnt, list, mv.v, mv.s, mv.w2, c);
+            direct_mover<DL32, false>(a, cnt, list, mv.v, mv.s, mv.w2, c);
         }
         if (lane == 0) flush_counts(md, c);
     } else {
         const int32_t *vl = a.vlist[bin];
-        const int64_t vcount = a.vcount[bin];
-        unsigned long long medges = 0;
-        for (int64_t j0 = 0; gw + j0 * nw < vcount; j0 += 32) {
-            const int64_t i = gw + (j0 + lane) * nw;
-            bool mover = false;
-            int pv = 0, ps = 0;
-            uint64_t pw = 0;
-            if (i < vcount) {
-                pv = vl[i];
-                const Proposal p = propose_vertex(a.g, md, a.seed, a.sweep_id, pv);
-                if (p.s == p.r) {
-                    c.proposed++;
-                } else {
-                    mover = true;
-                    ps = p.s;
-                    pw = p.w2;
-                    medges += (unsigned long long)p.k;
-                }
-            }
-            unsigned mask = __ballot_sync(0xffffffffu, mover);
-            while (mask) {
-                const int q = __ffs(mask) - 1;
-                mask &= mask - 1u;
-                const int v = __shfl_sync(0xffffffffu, pv, q), s = __shfl_sync(0xffffffffu, ps, q);
-                const uint64_t w2 = __shfl_sync(0xffffffffu, pw, q);
-                direct_mover<DL32>(a, cnt, list, v, s, w2, c);
-            }
-        }
+        const unsigned long long medges = direct_vertices<DL32, false>(
+            a, cnt, list, gw, nw, a.vcount[bin], [&](int64_t i) { return vl[i]; }, c);
         flush_counts_warp(md, c, medges);
     }
+}
+
+// ---------------------------------------------------------------------------
+// A small graph's whole pass in one launch: a warp per mover for every
+// degree, the moves the FP32 test cannot settle decided on the spot.  The
+// batches of 32 movers a warp (below) give a small graph too few warps, each
+// with a long serial aggregation: the three groups' kernels and the recheck
+// launch took 80 us at 1000 vertices and 107 us at 20,000 (16 edges out of
+// each), this takes 11 and 39 us.  It is bound by the chain of dependent
+// loads of a proposal and a move, a few of them per warp.
+template <bool DL32>
+__global__ void __launch_bounds__(kWarpsPerCta * 32, 2) k_eval_small(DecideArgs a, int warp_words) {
+    extern __shared__ unsigned smw[];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    const int B = a.md.B;
+    unsigned *cnt = smw + (size_t)wid * warp_words;
+    int *list = reinterpret_cast<int *>(cnt + B);
+    for (int i = lane; i < B; i += 32) cnt[i] = 0u;
+    __syncwarp();
+    Counts c;
+    const int64_t gw = (int64_t)blockIdx.x * nwarps + wid, nw = (int64_t)gridDim.x * nwarps;
+    // the largest rows first
+    const int64_t n2 = a.vcount[2], n1 = a.vcount[1];
+    const unsigned long long medges = direct_vertices<DL32, true>(
+        a, cnt, list, gw, nw, n2 + n1 + a.vcount[0], [&](int64_t i) {
+            return i < n2 ? a.vlist[2][i] : i < n2 + n1 ? a.vlist[1][i - n2] : a.vlist[0][i - n2 - n1];
+        }, c);
+    flush_counts_warp(a.md, c, medges);
 }
 
 // ---------------------------------------------------------------------------
@@ -1428,6 +1466,26 @@ int launch_recheck(sbp_model *m, const DecideArgs &a0, int sms) {
     return SBP_OK;
 }
 
+// Passes of at most this many vertices take k_eval_small.  Both sides, in us
+// (small pass, the groups' kernels; 16 edges out of each vertex / 20 with a
+// heavy tail): 40,000 vertices 64, 113 / 78, 150; 60,000 85, 103 / 106, 146;
+// 100,000 130, 126 / 174, 180; 200,000 246, 157 / 319, 223.
+constexpr int64_t kSmallPass = 60000;
+
+template <bool DL32>
+int launch_small(sbp_model *m, const DecideArgs &a, int sms) {
+    const int warp_words = 2 * m->B + 4;
+    const int nwarps = warp_words * 4 * kWarpsPerCta <= 64 * 1024 ? kWarpsPerCta : kWarpsPerCta / 2;
+    const size_t smem = (size_t)warp_words * 4 * nwarps;
+    SBP_TRY(ensure_dyn_smem((const void *)k_eval_small<DL32>, smem));
+    const int64_t n = a.vcount[0] + a.vcount[1] + a.vcount[2];
+    const int64_t ctas = (n + nwarps - 1) / nwarps;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ctas, sms * 2));
+    k_eval_small<DL32><<<grid, nwarps * 32, smem, m->stream>>>(a, warp_words);
+    SBP_LAUNCHED();
+    return SBP_OK;
+}
+
 template <bool DL32>
 int launch_evals(sbp_model *m, const DecideArgs &a, int sms, bool fused) {
     cudaStream_t st[3];
@@ -1500,8 +1558,6 @@ int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_en
     const int sms = sm_count();
     const int B = m->B;
     if (B >= (1 << 24)) return fail(SBP_ESTATE, "nodal pass: B must be below 2^24");
-    SBP_CUDA(cudaMemsetAsync(m->mcount, 0, 4 * sizeof(unsigned), m->stream));
-
     // hybrid pass: the sequential part first (full-range passes of a dense model)
     const int64_t h = std::min<int64_t>(m->p.hybrid_h, g->n);
     if (h > 0 && m->dense && v_begin == 0 && v_end == g->n) {
@@ -1541,6 +1597,9 @@ int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_en
     }
     const bool fused = SBP_FUSED_PROPOSALS && v_begin == 0 && v_end == g->n && !a.skip && !a.trace_on &&
                        B <= kDirectMaxB && g->max_deg < 65536;
+    if (fused && a.vcount[0] + a.vcount[1] + a.vcount[2] <= kSmallPass)
+        return m->p.dl_fp32 ? launch_small<true>(m, a, sms) : launch_small<false>(m, a, sms);
+    SBP_CUDA(cudaMemsetAsync(m->mcount, 0, 4 * sizeof(unsigned), m->stream));
     if (!fused) {
         int64_t blocks = (v_end - v_begin + 255) / 256;
         if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;

@@ -679,11 +679,12 @@ __device__ __forceinline__ void evaluate_group(const DecideArgs &a, const ModelD
     }
 }
 
-// the whole warp on one mover; unsettled moves go to the recheck list
-template <bool DL32, class EachEntry>
+// the whole warp on one mover; a move the FP32 test cannot settle goes to the
+// recheck list, or is decided on the spot (EXACT)
+template <bool DL32, bool EXACT, class EachEntry>
 __device__ __forceinline__ void evaluate_warp(const DecideArgs &a, const ModelDev &md, VertexCtx &x, uint64_t w2,
                                               EachEntry each_entry, Counts &c) {
-    evaluate_group<DL32, 32, false>(a, md, x, w2, each_entry, c);
+    evaluate_group<DL32, 32, EXACT>(a, md, x, w2, each_entry, c);
 }
 
 }  // namespace
