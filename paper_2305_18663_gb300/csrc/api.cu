@@ -121,17 +121,9 @@ int validate_params(const sbp_params &p) {
     return SBP_OK;
 }
 
-struct Stats {
-    DevCounters c;
-    double dl[2];
-    int32_t status;
-};
-
-int read_stats(sbp_model *m, sbp_sweep_stats *out) {
-    Stats *h = static_cast<Stats *>(m->pinned);
-    SBP_CUDA(cudaMemcpyAsync(&h->c, m->counters, sizeof(DevCounters), cudaMemcpyDeviceToHost, m->stream));
-    SBP_CUDA(cudaMemcpyAsync(h->dl, m->dl, 16, cudaMemcpyDeviceToHost, m->stream));
-    SBP_CUDA(cudaMemcpyAsync(&h->status, m->status, 4, cudaMemcpyDeviceToHost, m->stream));
+// the host's copy of a pass's report, once the stream has reached it
+int finish_stats(sbp_model *m, sbp_sweep_stats *out) {
+    const SweepReadback *h = static_cast<const SweepReadback *>(m->pinned);
     SBP_CUDA(cudaStreamSynchronize(m->stream));
     if (h->status != 0) {
         const int st = h->status;
@@ -148,6 +140,14 @@ int read_stats(sbp_model *m, sbp_sweep_stats *out) {
     out->dl_after = h->dl[0];
     out->dl_before = h->dl[1];
     return SBP_OK;
+}
+
+int read_stats(sbp_model *m, sbp_sweep_stats *out) {
+    SweepReadback *h = static_cast<SweepReadback *>(m->pinned);
+    SBP_CUDA(cudaMemcpyAsync(&h->c, m->counters, sizeof(DevCounters), cudaMemcpyDeviceToHost, m->stream));
+    SBP_CUDA(cudaMemcpyAsync(h->dl, m->dl, 16, cudaMemcpyDeviceToHost, m->stream));
+    SBP_CUDA(cudaMemcpyAsync(&h->status, m->status, 4, cudaMemcpyDeviceToHost, m->stream));
+    return finish_stats(m, out);
 }
 
 // labels outside [0, B): the slot keeps INT32_MAX - (smallest such vertex)
@@ -223,10 +223,15 @@ int upload_incremental(sbp_model *m, const int32_t *b) {
         return fail(SBP_EINVAL, "label out of [0, B) at vertex " + std::to_string((int64_t)INT32_MAX - *h));
     }
     std::swap(m->b, m->bnew);
-    SBP_CUDA(cudaMemcpyAsync(m->dl + 1, m->dl, 8, cudaMemcpyDeviceToDevice, m->stream));
     m->list_ok = true;  // the items list every change, once
     m->decided.clear();
     m->nb_in_commit = false;
+    if (commit_small_ok(m)) {
+        const int rs = commit_small(m, nullptr);
+        if (rs != SBP_OK) m->nb_ok = false;
+        return rs;
+    }
+    SBP_CUDA(cudaMemcpyAsync(m->dl + 1, m->dl, 8, cudaMemcpyDeviceToDevice, m->stream));
     int rc = commit_blockmodel(m);
     if (rc == SBP_OK) rc = nb_rows_after_commit(m);
     if (rc != SBP_OK) m->nb_ok = false;
@@ -429,6 +434,13 @@ extern "C" int sbp_set_pending(sbp_model_t *m, int64_t v_begin, int64_t v_end, c
 extern "C" int sbp_commit(sbp_model_t *m, sbp_sweep_stats *stats) {
     if (!m) return fail(SBP_EINVAL, "sbp_commit: NULL model");
     std::swap(m->b, m->bnew);
+    if (commit_small_ok(m)) {
+        const int rs = commit_small(m, stats ? static_cast<SweepReadback *>(m->pinned) : nullptr);
+        m->decided.clear();
+        if (rs != SBP_OK) m->nb_ok = false;
+        SBP_TRY(rs);
+        return stats ? finish_stats(m, stats) : SBP_OK;
+    }
     SBP_CUDA(cudaMemcpyAsync(m->dl + 1, m->dl, 8, cudaMemcpyDeviceToDevice, m->stream));
     m->nb_in_commit = false;
     int rc = commit_blockmodel(m);

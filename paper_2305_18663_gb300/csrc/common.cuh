@@ -120,6 +120,13 @@ struct DevCounters {
     unsigned long long entries;  // distinct neighbour blocks of the evaluated movers (sum of D_v)
 };
 
+// what a pass reports to the host
+struct SweepReadback {
+    DevCounters c;
+    double dl[2];
+    int32_t status;
+};
+
 // the accepted-move list: one (vertex, chunk) item per kMoveChunk edges of
 // every accepted mover, so the apply step's work units are all small
 constexpr int kMoveChunk = 256;
@@ -586,11 +593,53 @@ __device__ __forceinline__ int sparse_cdf_block(const ModelDev &md, int u, uint3
 }
 
 // ---------------------------------------------------------------------------
+// thread-block clusters
+
+__device__ __forceinline__ int cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return (int)r;
+}
+
+__device__ __forceinline__ int cluster_size() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return (int)r;
+}
+
+// barrier over the cluster's threads; what any of them wrote to global memory
+// before it is seen by all after it
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// one launch of one cluster of `size` blocks (1: a plain block)
+template <class... Args>
+int launch_cluster(void (*kern)(Args...), int size, int threads, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)size;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = size > 1 ? 1 : 0;
+    count_launch();
+    SBP_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
+    return SBP_OK;
+}
+
+// ---------------------------------------------------------------------------
 // host-side launch helpers implemented in the .cu files
 int rebuild_blockmodel(sbp_model *m);  // M, P, degrees, rcp, DL from m->b
 int count_cells(sbp_model *m, int32_t *cells);  // cells[r * B + t] = edges r -> t
 int update_cells(sbp_model *m, int32_t *cells);  // counts of m->bnew -> counts of m->b
 int launch_prefix(sbp_model *m);                 // P, Pc, degrees, reciprocals from a dense M
+bool commit_small_ok(const sbp_model *m);
+int commit_small(sbp_model *m, SweepReadback *host);  // the whole commit of a small dense model in one launch
 int commit_blockmodel(sbp_model *m);   // the same after a pass: m->b new labels, m->bnew the previous ones
 int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_end, const sbp_vertex_trace *trace);
 int nb_rows_rebuild(sbp_model *m);       // block-labelled rows from m->b (nb_ok when there is memory)

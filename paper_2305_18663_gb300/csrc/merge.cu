@@ -108,24 +108,6 @@ __global__ void __launch_bounds__(kApplyThreads) k_compact_map(uint32_t *words, 
     if (blockIdx.x == 0 && threadIdx.x == 0) res[1] = B_new;
 }
 
-// one block, or one cluster of kApplyCluster
-template <class... Args>
-int launch_team(void (*kern)(Args...), bool cluster, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cluster ? kApplyCluster : 1);
-    cfg.blockDim = dim3(kApplyThreads);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kApplyCluster;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = cluster ? 1 : 0;
-    count_launch();
-    SBP_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
-    return SBP_OK;
-}
-
 // the work arrays of both kernels, for B blocks
 int ensure_merge_work(sbp_model *m, int32_t B) {
     if (m->merge_work_B >= B) return SBP_OK;
@@ -200,7 +182,8 @@ int apply_merge_round(sbp_model *m, int32_t want, int32_t *done, int32_t *B_new)
     SBP_TRY(ensure_merge_work(m, m->B));
     const MergeWork x = merge_work(m);
     const bool cl = m->B > kOneCtaB;
-    SBP_TRY(launch_team(cl ? k_merge_apply<true> : k_merge_apply<false>, cl, m->stream, x.w, x.words, (int)m->B,
+    SBP_TRY(launch_cluster(cl ? k_merge_apply<true> : k_merge_apply<false>, cl ? kApplyCluster : 1, kApplyThreads, 0,
+                           m->stream, x.w, x.words, (int)m->B,
                         (const int32_t *)m->best_s, (const double *)m->best_d, (int)want, m->map, x.res));
     int32_t *h = static_cast<int32_t *>(m->pinned);
     SBP_CUDA(cudaMemcpyAsync(h, x.res, 8, cudaMemcpyDeviceToHost, m->stream));
@@ -216,7 +199,8 @@ int compact_blocks(sbp_model *m, int32_t *B_new) {
     SBP_TRY(ensure_merge_work(m, m->B));
     const MergeWork x = merge_work(m);
     const bool cl = m->B > kOneCtaB;
-    SBP_TRY(launch_team(cl ? k_compact_map<true> : k_compact_map<false>, cl, m->stream, x.words, (int)m->B,
+    SBP_TRY(launch_cluster(cl ? k_compact_map<true> : k_compact_map<false>, cl ? kApplyCluster : 1, kApplyThreads, 0,
+                           m->stream, x.words, (int)m->B,
                         (const int32_t *)m->vcount, m->map, x.res));
     int32_t *h = static_cast<int32_t *>(m->pinned);
     SBP_CUDA(cudaMemcpyAsync(h, x.res + 1, 4, cudaMemcpyDeviceToHost, m->stream));

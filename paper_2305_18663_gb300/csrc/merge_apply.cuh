@@ -99,19 +99,9 @@ struct ClusterTeam {
     TeamShared &sh;
     uint32_t *words;
     int turn = 0, turn_bins = 0;
-    __device__ int rank() const {
-        uint32_t r;
-        asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-        return (int)r;
-    }
-    __device__ int size() const {
-        uint32_t r;
-        asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-        return (int)r;
-    }
-    __device__ void sync() {
-        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-    }
+    __device__ int rank() const { return cluster_rank(); }
+    __device__ int size() const { return cluster_size(); }
+    __device__ void sync() { cluster_sync(); }
     __device__ uint32_t across(uint32_t v, uint32_t &before) {
         uint32_t *w = words + 8 * turn;
         turn ^= 1;
