@@ -621,7 +621,7 @@ int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, cons
             // on this stream, which runs the kernel that first uses them
             // the degree groups' lists and the recheck list of the per-graph pass
             if (model_alloc(&m->movers, (size_t)(m->g->n > 0 ? 2 * m->g->n : 1) * sizeof(Mover), st) != cudaSuccess ||
-                model_alloc((void **)&m->mcount, 4 * sizeof(unsigned), st) != cudaSuccess) {
+                model_alloc((void **)&m->mcount, kMoverLists * sizeof(unsigned), st) != cudaSuccess) {
                 cudaGetLastError();
                 cudaFreeAsync(buf, st);
                 return fail(SBP_ENOMEM, "device allocation failed for the mover lists");

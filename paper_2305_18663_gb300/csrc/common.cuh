@@ -65,7 +65,10 @@ __device__ __forceinline__ void record_status(int32_t *status, int32_t code) {
 constexpr int kWarp = 32;
 constexpr int kSmallDeg = 32;     // k <= 32: one neighbour per lane, no table
 constexpr int kWarpDeg = 128;     // k <= 128: one warp per vertex, per-warp table
-constexpr int kWarpCap = 256;     // per-warp table slots (>= 2 * kWarpDeg)
+constexpr int kMidDeg = 512;      // at large B, the classes above 128: up to 512, up to 1600, more
+constexpr int kWideDeg = 1600;
+constexpr int kMoverLists = 6;    // a pass's mover lists: five degree classes and the recheck list
+constexpr int kRecheck = 5;
 constexpr int kWarpsPerCta = 8;
 constexpr int kBigThreads = 256;  // threads of the CTA-per-vertex kernel
 constexpr int64_t kMaxTable = int64_t(1) << 22;  // largest x ln x table (entries)
@@ -102,6 +105,7 @@ struct sbp_graph {
     int32_t *order = nullptr;  // vertices grouped: k=0 | 1..32 | 33..128 | >128
     int32_t *by_degree = nullptr;  // all vertices by degree, descending (ties: lower id first)
     int64_t bin[5] = {0, 0, 0, 0, 0};
+    int64_t n_mid = 0, n_wide = 0;  // vertices of the top group up to kMidDeg, then up to kWideDeg
     int32_t max_deg = 0;
     sbp::GraphDev dev() const {
         sbp::GraphDev d;

@@ -50,7 +50,7 @@ int bits_for(uint64_t maxval) {
 // what the host needs to know of the graph
 struct Info {
     unsigned long long bad;  // the first edge with an id out of range (all ones: none)
-    unsigned long long cnt[4];  // vertices of the degree groups
+    unsigned long long cnt[6];  // vertices of the degree groups, the top one in its three classes
     unsigned long long n_self;
     int32_t maxk;
 };
@@ -140,32 +140,36 @@ __device__ __forceinline__ int degree_group(int32_t k) {
     return k == 0 ? 0 : k <= kSmallDeg ? 1 : k <= kWarpDeg ? 2 : 3;
 }
 
-// sizes of the degree groups and the largest degree
-__global__ void __launch_bounds__(kT) k_degree_groups(const int32_t *__restrict__ op, const int32_t *__restrict__ ip,
-                                                      int64_t n, Info *__restrict__ info) {
-    __shared__ unsigned cnt[4];
+__device__ __forceinline__ int degree_class(int32_t k) {
+    return k <= kWarpDeg ? degree_group(k) : k <= kMidDeg ? 3 : k <= kWideDeg ? 4 : 5;
+}
+
+// sizes of the degree classes and the largest degree
+__global__ void __launch_bounds__(kT) k_degree_classes(const int32_t *__restrict__ op, const int32_t *__restrict__ ip,
+                                                       int64_t n, Info *__restrict__ info) {
+    __shared__ unsigned cnt[6];
     __shared__ int mx;
-    if (threadIdx.x < 4) cnt[threadIdx.x] = 0;
+    if (threadIdx.x < 6) cnt[threadIdx.x] = 0;
     if (threadIdx.x == 0) mx = 0;
     __syncthreads();
     int m = 0;
-    unsigned c[4] = {0, 0, 0, 0};
+    unsigned c[6] = {0, 0, 0, 0, 0, 0};
     for (int64_t v = (int64_t)blockIdx.x * kT + threadIdx.x; v < n; v += (int64_t)gridDim.x * kT) {
         const int32_t k = (op[v + 1] - op[v]) + (ip[v + 1] - ip[v]);
         m = max(m, k);
-        const int q = degree_group(k);
+        const int q = degree_class(k);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) c[i] += q == i;
+        for (int i = 0; i < 6; ++i) c[i] += q == i;
     }
     m = __reduce_max_sync(0xffffffffu, m);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) c[i] = __reduce_add_sync(0xffffffffu, c[i]);
+    for (int i = 0; i < 6; ++i) c[i] = __reduce_add_sync(0xffffffffu, c[i]);
     if ((threadIdx.x & 31) == 0) {
         atomicMax(&mx, m);
-        for (int i = 0; i < 4; ++i) atomicAdd(&cnt[i], c[i]);
+        for (int i = 0; i < 6; ++i) atomicAdd(&cnt[i], c[i]);
     }
     __syncthreads();
-    if (threadIdx.x < 4 && cnt[threadIdx.x]) atomicAdd(&info->cnt[threadIdx.x], (unsigned long long)cnt[threadIdx.x]);
+    if (threadIdx.x < 6 && cnt[threadIdx.x]) atomicAdd(&info->cnt[threadIdx.x], (unsigned long long)cnt[threadIdx.x]);
     if (threadIdx.x == 0) atomicMax(&info->maxk, mx);
 }
 
@@ -259,7 +263,7 @@ int build_graph(sbp_graph *g, const int32_t *src, const int32_t *dst, const Scra
     }
     k_row_offsets<<<grid_of(n + 1), kT, 0, st>>>(g->esrc, *ikey, m, n, g->op, g->ip);
     SBP_LAUNCHED();
-    k_degree_groups<<<grid_of(n), kT, 0, st>>>(g->op, g->ip, n, x.info);
+    k_degree_classes<<<grid_of(n), kT, 0, st>>>(g->op, g->ip, n, x.info);
     SBP_LAUNCHED();
     SBP_CUDA(cudaMemcpyAsync(info, x.info, sizeof(Info), cudaMemcpyDeviceToHost, st));
     SBP_CUDA(cudaStreamSynchronize(st));
@@ -270,7 +274,10 @@ int build_graph(sbp_graph *g, const int32_t *src, const int32_t *dst, const Scra
 int finish_graph(sbp_graph *g, const Scratch &x, const Info &info, const uint32_t *ikey, cudaStream_t st) {
     g->max_deg = info.maxk;
     g->bin[0] = 0;
-    for (int i = 0; i < 4; ++i) g->bin[i + 1] = g->bin[i] + (int64_t)info.cnt[i];
+    for (int i = 0; i < 3; ++i) g->bin[i + 1] = g->bin[i] + (int64_t)info.cnt[i];
+    g->bin[4] = g->n;
+    g->n_mid = (int64_t)info.cnt[3];
+    g->n_wide = (int64_t)info.cnt[4];
     g->n_self = (int64_t)info.n_self;
     if (g->n_self > 0) {
         if (cudaMalloc((void **)&g->self_in, (size_t)g->n_self * 4) != cudaSuccess) {

@@ -4,7 +4,7 @@
 // above 128), each with its own evaluation kernel: k_eval_batch (32 movers
 // per warp; for 33..128 with direct-mapped counts while B is small),
 // k_eval_warp_direct (one warp per mover, direct-mapped counts) or, at
-// larger B, k_eval_warp (one warp per mover with a shared-memory table) and
+// larger B, k_eval_table (one warp per mover with a shared-memory table) and
 // k_eval_cta (one CTA per mover, very large tables).  In a pass over all
 // vertices without a trace the first two kinds draw the proposals of their
 // group's vertices themselves; otherwise k_propose (one lane per vertex)
@@ -59,13 +59,13 @@ __global__ void __launch_bounds__(256) k_propose(DecideArgs a) {
                 c.proposed++;
                 write_trace(a, v, p.r, 1, 0.0, 0.0);
             } else {
-                bin = p.k <= kSmallDeg ? 0 : p.k <= kWarpDeg ? 1 : 2;
+                bin = p.k <= kSmallDeg ? 0 : p.k <= kWarpDeg ? 1 : !a.split_top || p.k <= kMidDeg ? 2 : p.k <= kWideDeg ? 3 : 4;
                 w2 = p.w2;
                 medges += (unsigned long long)p.k;
             }
         }
 #pragma unroll
-        for (int bb = 0; bb < 3; ++bb) {
+        for (int bb = 0; bb < kRecheck; ++bb) {
             const unsigned msk = __ballot_sync(0xffffffffu, bin == bb);
             if (msk == 0) continue;
             const int leader = __ffs(msk) - 1;
@@ -84,40 +84,335 @@ __global__ void __launch_bounds__(256) k_propose(DecideArgs a) {
     flush_counts_warp(md, c, medges);
 }
 
-// One warp per mover of list `bin` (k >= 33).  Dynamic shared memory per
-// warp: cap int keys, cap 32-bit counts (ko | ki << 16, degrees below
-// 65536), cap 16-bit list entries, one list length.  Warps take chunks of
-// `chunk` movers and prefetch their records with one lane per mover.
+// ---------------------------------------------------------------------------
+// One warp per mover at large B (B > kDirectMaxB): the row's neighbour blocks
+// are counted in a shared-memory hash table of `cap` slots, then the entries
+// are evaluated.  Warp w of W takes the movers w, w + W, ... of list `bin`.
+//
+// On sparse rows most of what an entry needs of M is zero, and looking it up
+// costs two dependent loads of scattered sectors per count, four counts per
+// entry.  The counts of row r, row s, column r and column s are contiguous in
+// the CSR and CSC, so a row or column that is not much longer than the
+// mover's own entry list (kStreamRatio) is read through instead, each of its
+// entries looked up in the shared-memory table:
+//   - a hit is one changed cell of M: its term of Delta L and its share of the
+//     Hastings sums are added on the spot (all linear in the cells);
+//   - hits in row s and column s mark their slot; the entries left unmarked
+//     have a zero count there and get f(k) - f(0) in the pass over the
+//     entries.  (Every entry with edges out of v has its cell in row r, and
+//     every one with edges into v in column r.)
+//   - the corner entries are the hits on r and s themselves.
+// Longer rows (a hub's block) are probed entry by entry as before.
+// Bound by instruction issue and the latency of those loads (36% of the issue
+// slots, 4% of DRAM bandwidth).  A decision pass of 200k vertices, 4M edges
+// (30% of the labels redrawn), with the tables sized by degree class: 845 ->
+// 507 us at B = 4096 dense, 1679 -> 1231 us at B = 65,536 sparse.  The line
+// kStreamRatio, at B = 65,536 / 8192: rows never read through 1443 / 1104 us,
+// up to 2 entries per entry of the mover 1231 / 1061, 4 1233 / 1226, 8 1314 /
+// 1362.
+constexpr int kStreamRatio = 2;
+
+struct TableWarp {
+    int *keys;             // [cap] block, with the two mark bits; -1 empty
+    unsigned *cnt;         // [cap] ko | ki << 16 (degrees below 65536)
+    unsigned short *list;  // [cap] slots in order of appearance
+    int *corner;           // [4] M[r][r], M[s][s], M[r][s], M[s][r]
+    int2 *queue;           // [kTableQueue] changed cells waiting for their terms
+    int cap, cap_log2;
+};
+constexpr int kTableIn = 4;                      // 32-entry chunks in flight
+constexpr int kTableQueue = 31 + 32 * kTableIn;  // (an entry pushes at most four, too)
+constexpr int kMarkRow = 1 << 29, kMarkCol = 1 << 30;  // hit in row s / column s
+constexpr int kKeyMask = (1 << 24) - 1;
+
+// a key's slot, -1 when it is not in the table (marks ignored)
+__device__ __forceinline__ int table_find(const TableWarp &W, int key) {
+    unsigned h = hash_slot(key, W.cap_log2);
+    for (int p = 0; p < W.cap; ++p) {
+        const int x = W.keys[h];
+        if (x < 0) return -1;
+        if ((x & kKeyMask) == key) return (int)h;
+        h = (h + 1) & (unsigned)(W.cap - 1);
+    }
+    return -1;
+}
+
+// v's row into the table: the number of entries (in `list`), the self-loops
+__device__ __forceinline__ int table_row(const DecideArgs &a, const TableWarp &W, int v, int o0, int i0, int kout, int k,
+                                         int &self) {
+    const int lane = threadIdx.x & 31;
+    const ModelDev &md = a.md;
+    constexpr int kIn = kTableIn;
+    int nl = 0;
+    self = 0;
+    bool full = false;
+    for (int base = 0; base < k; base += 32 * kIn) {
+        int nb[kIn], tb[kIn];
+        bool sf[kIn];
+#pragma unroll
+        for (int c4 = 0; c4 < kIn; ++c4) {
+            const int idx = base + c4 * 32 + lane;
+            nb[c4] = idx < k ? nb_raw(a.g, md, o0, i0, kout, idx) : 0;
+        }
+#pragma unroll
+        for (int c4 = 0; c4 < kIn; ++c4) {
+            const int idx = base + c4 * 32 + lane;
+            sf[c4] = false;
+            tb[c4] = idx < k ? nb_block(md, nb[c4], v, sf[c4]) : -1;
+        }
+#pragma unroll
+        for (int c4 = 0; c4 < kIn; ++c4) {
+            if (base + c4 * 32 >= k) break;
+            const int idx = base + c4 * 32 + lane;
+            const bool is_out = idx < kout, is_self = idx < k && sf[c4];
+            self += __popc(__ballot_sync(0xffffffffu, is_self && is_out));
+            bool fresh = false;
+            unsigned h = 0;
+            if (tb[c4] >= 0 && !is_self) {
+                h = hash_slot(tb[c4], W.cap_log2);
+                bool done = false;
+                for (int p = 0; p < W.cap; ++p) {
+                    const int prev = atomicCAS(&W.keys[h], -1, tb[c4]);
+                    if (prev == -1 || prev == tb[c4]) {
+                        fresh = prev == -1;
+                        done = true;
+                        break;
+                    }
+                    h = (h + 1) & (unsigned)(W.cap - 1);
+                }
+                if (done) atomicAdd(&W.cnt[h], is_out ? 1u : 0x10000u);
+                else full = true;
+            }
+            const unsigned fm = __ballot_sync(0xffffffffu, fresh);
+            if (fresh) W.list[nl + __popc(fm & ((1u << lane) - 1u))] = (unsigned short)h;
+            nl += __popc(fm);
+        }
+    }
+    if (full) record_status(md.status, SBP_EHASHFULL);
+    __syncwarp();
+    return nl;
+}
+
+// the sums of a move's entries on one lane
+struct MoveSums {
+    __int128 dl = 0;
+    double fb = 0.0;
+    float dlf = 0.0f, am = 0.0f, pf = 0.0f, pb = 0.0f;
+};
+
+// Changed cells of a move wait in the warp's queue as (m, k) for their terms
+// f(m + k) - f(m) (bit 31 of m: subtracted, for the block degrees), so that
+// the terms are evaluated by full warps and by one copy of their code: inline
+// at every place that finds a cell, lanes without one idled and the kernel
+// stalled on instruction fetches (5 of 13 cycles between two issues).
+__device__ __forceinline__ void queue_cell(const TableWarp &W, int &nq, bool has, int m, int k) {
+    const unsigned hm = __ballot_sync(0xffffffffu, has);
+    if (has) W.queue[nq + __popc(hm & ((1u << (threadIdx.x & 31)) - 1u))] = make_int2(m, k);
+    nq += __popc(hm);
+}
+
 template <bool DL32>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, SBP_DECIDE_MIN_BLOCKS) k_eval_warp(DecideArgs a, int bin, int cap,
-                                                                                    int cap_log2, int chunk) {
+__device__ __forceinline__ void drain_cells(const ModelDev &md, const TableWarp &W, int &nq, int keep, MoveSums &S) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    while (nq > keep) {
+        const int take = nq < 32 ? nq : 32;
+        const int2 e = lane < take ? W.queue[nq - take + lane] : make_int2(0, 0);
+        nq -= take;
+        const int m = e.x & 0x7fffffff;
+        if (DL32) {
+            const float d = dxlogx32(m, e.y, S.am);
+            S.dlf += e.x < 0 ? -d : d;
+        } else {
+            double f2 = 0.0;
+            const __int128 d = dT(md.T, md.XT, m, e.y, f2);
+            S.dl += e.x < 0 ? -d : d;
+            S.fb += e.x < 0 ? -f2 : f2;
+        }
+    }
+    __syncwarp();
+}
+
+// the move of x (entries in the table, nl of them) on sparse rows
+template <bool DL32>
+__device__ __forceinline__ void table_move_sparse(const DecideArgs &a, const TableWarp &W, VertexCtx &x, int nl,
+                                                  uint64_t w2, Counts &c) {
+    const int lane = threadIdx.x & 31;
+    const ModelDev &md = a.md;
+    const int r = x.r, s = x.s;
+    // segments: row r, row s, column r, column s
+    const uint32_t r0 = md.rp[r], r1 = md.rp[r + 1], s0 = md.rp[s], s1 = md.rp[s + 1];
+    const uint32_t cr0 = md.cp[r], cr1 = md.cp[r + 1], cs0 = md.cp[s], cs1 = md.cp[s + 1];
+    const uint32_t most = (uint32_t)(kStreamRatio * nl + 32);
+    const bool st_r = r1 - r0 <= most, st_s = s1 - s0 <= most, st_cr = cr1 - cr0 <= most, st_cs = cs1 - cs0 <= most;
+    const uint32_t e0 = st_r ? r1 - r0 : 0u, e1 = e0 + (st_s ? s1 - s0 : 0u), e2 = e1 + (st_cr ? cr1 - cr0 : 0u),
+                   e3 = e2 + (st_cs ? cs1 - cs0 : 0u);
+    const int deg = (lane < 6 ? md.dout : md.din)[(lane & 1) ? s : r];  // lanes 4..7: the degrees
+    if (lane < 4) W.corner[lane] = 0;
+    __syncwarp();
+    MoveSums S;
+    int nq = 0;
+    constexpr int kIn = kTableIn;
+    for (uint32_t b0 = 0; b0 < e3; b0 += 32 * kIn) {
+        int key[kIn], val[kIn];
+#pragma unroll
+        for (int u = 0; u < kIn; ++u) {
+            const uint32_t i = b0 + 32 * u + lane;
+            const bool col = i >= e1;
+            const uint32_t p = i < e0 ? r0 + i : i < e1 ? s0 + (i - e0) : i < e2 ? cr0 + (i - e1) : cs0 + (i - e2);
+            key[u] = i < e3 ? (col ? md.cr : md.rc)[p] : -1;
+            val[u] = i < e3 ? (col ? md.cv : md.rv)[p] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < kIn; ++u) {
+            if (b0 + 32 * u >= e3) break;
+            const uint32_t i = b0 + 32 * u + lane;
+            const bool col = i >= e1, to = col ? i >= e2 : i >= e0;  // to: of s, which the edges reach
+            if (key[u] == r || key[u] == s) {
+                // from rows r and s (the columns hold the same four again)
+                if (!col) W.corner[!to ? (key[u] == r ? 0 : 2) : (key[u] == r ? 3 : 1)] = val[u];
+                key[u] = -1;
+            }
+            const int slot = key[u] >= 0 ? table_find(W, key[u]) : -1;
+            int kk = 0;
+            if (slot >= 0) {
+                const unsigned cc = W.cnt[slot];
+                const int ko = (int)(cc & 0xffffu), ki = (int)(cc >> 16);
+                kk = col ? ki : ko;  // rows change by ko, columns by ki
+                if (to) atomicOr(&W.keys[slot], col ? kMarkCol : kMarkRow);
+                const float cw = (float)(ko + ki) * md.rcp32[key[u]];
+                if (to) S.pf += cw * (float)val[u];
+                else S.pb += cw * (float)(val[u] - kk);
+            }
+            queue_cell(W, nq, kk != 0, val[u], to ? kk : -kk);
+        }
+        drain_cells<DL32>(md, W, nq, 31, S);
+    }
+    __syncwarp();
+    // the counts to r and to s, and the corner entries not read through
+    {
+        const int slot = lane < 2 ? table_find(W, lane == 0 ? r : s) : -1;
+        const unsigned cc = slot >= 0 ? W.cnt[slot] : 0u;
+        const unsigned cr = __shfl_sync(0xffffffffu, cc, 0), cs = __shfl_sync(0xffffffffu, cc, 1);
+        x.ko_r = (int)(cr & 0xffffu);
+        x.ki_r = (int)(cr >> 16);
+        x.ko_s = (int)(cs & 0xffffu);
+        x.ki_s = (int)(cs >> 16);
+    }
+    int val = deg;
+    if (lane < 4) {
+        const bool of_r = lane == 0 || lane == 2;  // Mrr, Mrs
+        val = (of_r ? st_r : st_s) ? W.corner[lane] : sparse_at(md, of_r ? r : s, (lane == 0 || lane == 3) ? r : s);
+    }
+    // the entries: what the hits left (an entry with ko > 0 has a cell in row
+    // r, one with ki > 0 in column r, so those are hits where they were read)
+    const bool all_read = st_r && st_s && st_cr && st_cs;
+    for (int e0i = 0; e0i < nl; e0i += 32) {
+        const int e = e0i + lane;
+        const int slot = e < nl ? W.list[e] : 0;
+        const int key = e < nl ? W.keys[slot] : r, t = key & kKeyMask;
+        const bool on = t != r && t != s;
+        const unsigned cc = on ? W.cnt[slot] : 0u;
+        const int ko = (int)(cc & 0xffffu), ki = (int)(cc >> 16);
+        const float cw = on ? (float)(ko + ki) * md.rcp32[t] : 0.0f;
+        int Mst = 0, Mts = 0;
+        if (!all_read) {
+            int Mrt = ko, Mtr = ki;
+            if (on) {
+                if (!st_r) Mrt = sparse_at(md, r, t);
+                if (!st_s) Mst = sparse_at(md, s, t);
+                if (!st_cr) Mtr = sparse_at(md, t, r);
+                if (!st_cs) Mts = sparse_at(md, t, s);
+            }
+            S.pf += cw * (float)(Mts + Mst);
+            S.pb += cw * (float)((Mtr - ki) + (Mrt - ko));
+            queue_cell(W, nq, !st_r && ko, Mrt, -ko);
+            queue_cell(W, nq, !st_cr && ki, Mtr, -ki);
+        }
+        S.pf += cw;
+        S.pb += cw;
+        queue_cell(W, nq, ko && (!st_s || !(key & kMarkRow)), Mst, ko);
+        queue_cell(W, nq, ki && (!st_cs || !(key & kMarkCol)), Mts, ki);
+        drain_cells<DL32>(md, W, nq, 31, S);
+    }
+    // corner and degrees
+    const int cr = x.ko_r + x.ki_r, cs = x.ko_s + x.ki_s;
+    const int kk = lane == 0   ? -(cr + x.self)
+                   : lane == 1 ? cs + x.self
+                   : lane == 2 ? x.ki_r - x.ko_s
+                   : lane == 3 ? x.ko_r - x.ki_s
+                   : lane == 4 ? -x.Kout
+                   : lane == 5 ? x.Kout
+                   : lane == 6 ? -x.Kin
+                               : x.Kin;
+    queue_cell(W, nq, lane < 8 && kk != 0, lane < 4 ? val : val | INT32_MIN, kk);
+    drain_cells<DL32>(md, W, nq, 0, S);
+    CornerVals cv;
+    cv.Mrr = __shfl_sync(0xffffffffu, val, 0);
+    cv.Mss = __shfl_sync(0xffffffffu, val, 1);
+    cv.Mrs = __shfl_sync(0xffffffffu, val, 2);
+    cv.Msr = __shfl_sync(0xffffffffu, val, 3);
+    cv.dr = md.dsum[r];
+    cv.ds = md.dsum[s];
+    float pf = warp_sum_f(S.pf), pb = warp_sum_f(S.pb);
+    corner_hastings_fast(x, cv, md.B, pf, pb);
+    // additions on a lane: one per 32 cells of the queue and one per 32
+    // entries read; at most e3 + 4 nl + 8 cells (bounds all the FP32 sums)
+    const int adds = (int)e3 + 4 * nl + 64;
+    int dec = -1;
+    if (DL32) {
+        const float dlf = warp_sum_f(S.dlf), am = warp_sum_f(S.am);
+        if (!a.trace_on) dec = fast_decision_f(a.beta32, dlf, 0.0f, pf, pb, w2, max(x.k, adds), dl32_error(am, adds));
+    } else {
+        const __int128 dl = warp_sum_128(S.dl);
+        const bool has_fb = __any_sync(0xffffffffu, __double_as_longlong(S.fb) != 0);
+        const double fb = has_fb ? warp_sum(S.fb) : 0.0;
+        if (!a.trace_on) dec = fast_decision(a.beta32, dl, has_fb, fb, pf, pb, w2, max(x.k, adds));
+    }
+    if (lane == 0) {
+        if (dec >= 0) {
+            if (dec) accept_move(md, x.v, s, x.k);
+            count_result(c, dec != 0, false, x.k);
+        } else {
+            push_recheck(a, x.v, s, w2);
+        }
+    }
+}
+
+template <bool DL32, bool SPARSE>
+__global__ void __launch_bounds__(kWarpsPerCta * 32, SBP_DECIDE_MIN_BLOCKS) k_eval_table(DecideArgs a, int bin, int cap,
+                                                                                     int cap_log2) {
     extern __shared__ int dsm[];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
     const ModelDev &md = a.md;
     const GraphDev &g = a.g;
-    int *keys = dsm + (size_t)wid * cap;
-    unsigned *cnt = reinterpret_cast<unsigned *>(dsm + (size_t)nwarps * cap) + (size_t)wid * cap;
-    int *nlist = dsm + (size_t)2 * nwarps * cap + wid;
-    unsigned short *list = reinterpret_cast<unsigned short *>(dsm + (size_t)2 * nwarps * cap + nwarps) + (size_t)wid * cap;
+    TableWarp W;
+    W.cap = cap;
+    W.cap_log2 = cap_log2;
+    __shared__ int2 queue[kWarpsPerCta][SPARSE ? kTableQueue : 1];
+    __shared__ int corner[kWarpsPerCta][4];
+    W.keys = dsm + (size_t)wid * cap;
+    W.cnt = reinterpret_cast<unsigned *>(dsm + (size_t)nwarps * cap) + (size_t)wid * cap;
+    W.list = reinterpret_cast<unsigned short *>(dsm + (size_t)2 * nwarps * cap) + (size_t)wid * cap;
+    W.corner = corner[wid];
+    W.queue = queue[wid];
     for (int i = lane; i < cap; i += 32) {
-        keys[i] = -1;
-        cnt[i] = 0;
+        W.keys[i] = -1;
+        W.cnt[i] = 0;
     }
-    if (lane == 0) *nlist = 0;
     __syncwarp();
 
     const Mover *mlist = a.movers + a.mbase[bin];
     const int64_t count = *(volatile unsigned *)&a.mcount[bin];
     Counts c;
-    const int64_t nw = (int64_t)gridDim.x * nwarps;
-    const int64_t nchunk = (count + chunk - 1) / chunk;
-    for (int64_t ch = (int64_t)blockIdx.x * nwarps + wid; ch < nchunk; ch += nw) {
-        const int64_t first = ch * chunk;
-        const int cnt_v = (int)(count - first < chunk ? count - first : chunk);
+    const int64_t gw = (int64_t)blockIdx.x * nwarps + wid, nw = (int64_t)gridDim.x * nwarps;
+    // 32 movers' records at a time, a lane each
+    for (int64_t j0 = 0; gw + j0 * nw < count; j0 += 32) {
+        const int64_t i = gw + (j0 + lane) * nw;
         int pv = 0, ps = 0, pr = 0, po = 0, pko = 0, pi = 0, pki = 0;
         uint64_t pw2 = 0;
-        if (lane < cnt_v) {
-            const Mover mv = mlist[first + lane];
+        if (i < count) {
+            const Mover mv = mlist[i];
             pv = mv.v;
             ps = mv.s;
             pw2 = mv.w2;
@@ -127,70 +422,36 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, SBP_DECIDE_MIN_BLOCKS) k_ev
             pi = g.ip[pv];
             pki = g.ip[pv + 1] - pi;
         }
-        for (int q = 0; q < cnt_v; ++q) {
-            const int v = __shfl_sync(0xffffffffu, pv, q);
-            const int s = __shfl_sync(0xffffffffu, ps, q);
-            const int r = __shfl_sync(0xffffffffu, pr, q);
-            const int o0 = __shfl_sync(0xffffffffu, po, q), kout = __shfl_sync(0xffffffffu, pko, q);
-            const int i0 = __shfl_sync(0xffffffffu, pi, q), kin = __shfl_sync(0xffffffffu, pki, q);
-            const uint64_t w2 = __shfl_sync(0xffffffffu, pw2, q);
-            const int k = kout + kin;
-            // aggregate the row: four 32-neighbour chunks per round
-            int self = 0;
-            bool ok = true;
-            for (int base = 0; base < k; base += 128) {
-                int nb[4], tb[4];
-                bool sf[4];
-#pragma unroll
-                for (int c4 = 0; c4 < 4; ++c4) {
-                    const int idx = base + c4 * 32 + lane;
-                    nb[c4] = idx < k ? nb_raw(g, md, o0, i0, kout, idx) : 0;
-                }
-#pragma unroll
-                for (int c4 = 0; c4 < 4; ++c4) {
-                    const int idx = base + c4 * 32 + lane;
-                    sf[c4] = false;
-                    tb[c4] = idx < k ? nb_block(md, nb[c4], v, sf[c4]) : -1;
-                }
-#pragma unroll
-                for (int c4 = 0; c4 < 4; ++c4) {
-                    const int cb = base + c4 * 32;
-                    if (cb >= k) break;
-                    const int idx = cb + lane;
-                    const bool valid = idx < k, is_out = idx < kout;
-                    const bool is_self = valid && sf[c4];
-                    self += __popc(__ballot_sync(0xffffffffu, is_self && is_out));
-                    const int key = (valid && !is_self) ? tb[c4] : -1;
-                    const unsigned peers = __match_any_sync(0xffffffffu, key);
-                    const unsigned outm = __ballot_sync(0xffffffffu, valid && !is_self && is_out);
-                    if (key >= 0 && lane == __ffs(peers) - 1) {
-                        const unsigned ko = __popc(peers & outm), ki = __popc(peers) - ko;
-                        ok &= table_add32(keys, cnt, list, nlist, cap, cap_log2, key, ko | (ki << 16));
-                    }
-                    __syncwarp();
-                }
-            }
-            if (!ok) record_status(md.status, SBP_EHASHFULL);
-            const int D = *nlist;
-            if (lane == 0) c.entries += (unsigned)D;
+        const int nq = __popc(__ballot_sync(0xffffffffu, i < count));
+        for (int q = 0; q < nq; ++q) {
             VertexCtx x;
-            x.v = v; x.r = r; x.s = s;
-            x.Kout = kout; x.Kin = kin; x.self = self; x.k = k;
-            evaluate_warp<DL32, false>(a, md, x, w2, [&](auto &&f) {
-                for (int e = lane; e < D; e += 32) {
-                    const int slot = list[e];
-                    const unsigned cc = cnt[slot];
-                    f(keys[slot], (int)(cc & 0xffffu), (int)(cc >> 16));
-                }
-            }, c);
+            x.v = __shfl_sync(0xffffffffu, pv, q);
+            x.s = __shfl_sync(0xffffffffu, ps, q);
+            x.r = __shfl_sync(0xffffffffu, pr, q);
+            const int o0 = __shfl_sync(0xffffffffu, po, q), i0 = __shfl_sync(0xffffffffu, pi, q);
+            x.Kout = __shfl_sync(0xffffffffu, pko, q);
+            x.Kin = __shfl_sync(0xffffffffu, pki, q);
+            const uint64_t w2 = __shfl_sync(0xffffffffu, pw2, q);
+            x.k = x.Kout + x.Kin;
+            const int D = table_row(a, W, x.v, o0, i0, x.Kout, x.k, x.self);
+            if (lane == 0) c.entries += (unsigned)D;
+            if constexpr (SPARSE) {
+                table_move_sparse<DL32>(a, W, x, D, w2, c);
+            } else {
+                evaluate_warp<DL32, false>(a, md, x, w2, [&](auto &&f) {
+                    for (int e = lane; e < D; e += 32) {
+                        const int slot = W.list[e];
+                        const unsigned cc = W.cnt[slot];
+                        f(W.keys[slot], (int)(cc & 0xffffu), (int)(cc >> 16));
+                    }
+                }, c);
+            }
             __syncwarp();
             for (int e = lane; e < D; e += 32) {
-                const int slot = list[e];
-                keys[slot] = -1;
-                cnt[slot] = 0;
+                const int slot = W.list[e];
+                W.keys[slot] = -1;
+                W.cnt[slot] = 0;
             }
-            __syncwarp();
-            if (lane == 0) *nlist = 0;
             __syncwarp();
         }
     }
@@ -1382,11 +1643,26 @@ template <bool DL32, bool FUSED>
 int launch_groups(sbp_model *m, const DecideArgs &a, int sms, const cudaStream_t st[3]) {
     const sbp_graph *g = m->g;
     const int B = m->B;
-    auto warp_smem = [](int cap, int nwarps) { return (size_t)nwarps * cap * 10 + (size_t)nwarps * 4 + 16; };
-    // movers with k > 128: per-warp direct-mapped counts while B is small,
-    // else per-warp tables sized for min(max degree, B) distinct blocks while
-    // they fit, one CTA per mover beyond that
-    if (g->bin[4] > g->bin[3] && B <= kDirectMaxB && g->max_deg < 65536) {
+    // one launch of k_eval_table over list `bin`, tables of 2^cap_log2 slots
+    auto tables = [&](int bin, int cap_log2, cudaStream_t on) -> int {
+        const int cap = 1 << cap_log2;
+        const size_t smem = (size_t)kWarpsPerCta * cap * 10;
+        const size_t fixed = (size_t)kWarpsPerCta * (kTableQueue * 8 + 16) + 1024;  // static, and the system's
+        const int per_sm = std::max(1, std::min(SBP_DECIDE_MIN_BLOCKS, (int)((size_t)228 * 1024 / (smem + fixed))));
+        auto go = [&](auto kern) -> int {
+            SBP_TRY(ensure_dyn_smem((const void *)kern, smem));
+            kern<<<sms * per_sm, kWarpsPerCta * 32, smem, on>>>(a, bin, cap, cap_log2);
+            SBP_LAUNCHED();
+            return SBP_OK;
+        };
+        return m->dense ? go(k_eval_table<DL32, false>) : go(k_eval_table<DL32, true>);
+    };
+    // movers with k > 128: per-warp direct-mapped counts while B is small; at
+    // larger B per-warp tables by degree class (each holds its class's
+    // distinct blocks at a load of at most 0.8), one CTA per mover above
+    // kWideDeg.  One table size for the whole group, set by the largest hub,
+    // had sent all of it to the CTA kernel.
+    if (g->bin[4] > g->bin[3] && !a.split_top) {
         const int warp_words = 2 * B + 4;
         const int nwarps = warp_words * 4 * kWarpsPerCta <= 64 * 1024 ? kWarpsPerCta : kWarpsPerCta / 2;
         const size_t smem = (size_t)warp_words * 4 * nwarps;
@@ -1394,26 +1670,21 @@ int launch_groups(sbp_model *m, const DecideArgs &a, int sms, const cudaStream_t
         k_eval_warp_direct<DL32, FUSED><<<sms * 4, nwarps * 32, smem, st[2]>>>(a, 2, warp_words);
         SBP_LAUNCHED();
     } else if (g->bin[4] > g->bin[3]) {
-        const int64_t dmax = g->max_deg < B ? g->max_deg : B;
-        const int64_t need = dmax + dmax / 4 + 2;
-        int cap_log2 = 6;
-        while ((int64_t(1) << cap_log2) < need) ++cap_log2;
-        const int cap = 1 << cap_log2;
-        if (cap <= 4096 && g->max_deg < 65536) {
-            const int nwarps = cap <= 2048 ? 8 : 4;
-            const size_t smem = warp_smem(cap, nwarps);
-            SBP_TRY(ensure_dyn_smem((const void *)k_eval_warp<DL32>, smem));
-            k_eval_warp<DL32><<<sms * 4, nwarps * 32, smem, st[2]>>>(a, 2, cap, cap_log2, 1);
-            SBP_LAUNCHED();
-        } else {
+        if (g->n - g->bin[3] > g->n_mid + g->n_wide) {
+            const int64_t dmax = g->max_deg < B ? g->max_deg : B;
+            const int64_t need = dmax + dmax / 4 + 2;
+            int cap_log2 = 6;
+            while ((int64_t(1) << cap_log2) < need) ++cap_log2;
             int grid;
             size_t smem;
             unsigned long long *gtab;
-            SBP_TRY(cta_table(m, cap, sms, &grid, &smem, &gtab));
+            SBP_TRY(cta_table(m, 1 << cap_log2, sms, &grid, &smem, &gtab));
             SBP_TRY(ensure_dyn_smem((const void *)k_eval_cta<DL32>, smem));
-            k_eval_cta<DL32><<<grid, kBigThreads, smem, st[2]>>>(a, 2, cap, cap_log2, gtab);
+            k_eval_cta<DL32><<<grid, kBigThreads, smem, st[2]>>>(a, 4, 1 << cap_log2, cap_log2, gtab);
             SBP_LAUNCHED();
         }
+        if (g->n_wide > 0) SBP_TRY(tables(3, 11, st[2]));
+        if (g->n_mid > 0) SBP_TRY(tables(2, 10, st[0]));
     }
     // movers with k <= 32: batches of 32 per warp
     if (g->bin[2] > g->bin[1]) {
@@ -1434,10 +1705,7 @@ int launch_groups(sbp_model *m, const DecideArgs &a, int sms, const cudaStream_t
             k_eval_batch<1, DL32, FUSED><<<sms * SBP_DECIDE_MIN_BLOCKS, nwarps * 32, smem, st[1]>>>(a, 1, wb);
             SBP_LAUNCHED();
         } else {
-            const size_t smem = warp_smem(kWarpCap, kWarpsPerCta);
-            SBP_TRY(ensure_dyn_smem((const void *)k_eval_warp<DL32>, smem));
-            k_eval_warp<DL32><<<sms * SBP_DECIDE_MIN_BLOCKS, kWarpsPerCta * 32, smem, st[1]>>>(a, 1, kWarpCap, 8, 32);
-            SBP_LAUNCHED();
+            SBP_TRY(tables(1, 8, st[1]));
         }
     }
     return SBP_OK;
@@ -1461,7 +1729,7 @@ int launch_recheck(sbp_model *m, const DecideArgs &a0, int sms) {
     unsigned long long *gtab;
     SBP_TRY(cta_table(m, cap, sms, &grid, &smem, &gtab));
     SBP_TRY(ensure_dyn_smem((const void *)k_eval_cta<DL32>, smem));
-    k_eval_cta<DL32><<<grid, kBigThreads, smem, m->stream>>>(a, 3, cap, cap_log2, gtab);
+    k_eval_cta<DL32><<<grid, kBigThreads, smem, m->stream>>>(a, kRecheck, cap, cap_log2, gtab);
     SBP_LAUNCHED();
     return SBP_OK;
 }
@@ -1504,7 +1772,7 @@ int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_en
     if (!m->movers) {
         // the degree groups' lists (n entries) and the recheck list (n more)
         if (model_alloc(&m->movers, (size_t)(g->n > 0 ? 2 * g->n : 1) * sizeof(Mover), m->stream) != cudaSuccess ||
-            model_alloc((void **)&m->mcount, 4 * sizeof(unsigned), m->stream) != cudaSuccess) {
+            model_alloc((void **)&m->mcount, kMoverLists * sizeof(unsigned), m->stream) != cudaSuccess) {
             cudaGetLastError();
             return fail(SBP_ENOMEM, "cudaMalloc failed for the mover lists");
         }
@@ -1546,7 +1814,9 @@ int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_en
     a.mbase[0] = 0;
     a.mbase[1] = g->bin[2] - g->bin[1];
     a.mbase[2] = a.mbase[1] + (g->bin[3] - g->bin[2]);
-    a.mbase[3] = g->n;  // the recheck list
+    a.mbase[3] = a.mbase[2] + g->n_mid;
+    a.mbase[4] = a.mbase[3] + g->n_wide;
+    a.mbase[kRecheck] = g->n;
     a.force_exact = 0;
     a.seed = m->p.seed;
     a.sweep_id = sweep_id;
@@ -1557,6 +1827,7 @@ int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_en
     a.trace_on = (a.tr.s || a.tr.flags || a.tr.dH || a.tr.logA) ? 1 : 0;
     const int sms = sm_count();
     const int B = m->B;
+    a.split_top = B > kDirectMaxB || g->max_deg >= 65536;
     if (B >= (1 << 24)) return fail(SBP_ESTATE, "nodal pass: B must be below 2^24");
     // hybrid pass: the sequential part first (full-range passes of a dense model)
     const int64_t h = std::min<int64_t>(m->p.hybrid_h, g->n);
@@ -1599,7 +1870,7 @@ int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_en
                        B <= kDirectMaxB && g->max_deg < 65536;
     if (fused && a.vcount[0] + a.vcount[1] + a.vcount[2] <= kSmallPass)
         return m->p.dl_fp32 ? launch_small<true>(m, a, sms) : launch_small<false>(m, a, sms);
-    SBP_CUDA(cudaMemsetAsync(m->mcount, 0, 4 * sizeof(unsigned), m->stream));
+    SBP_CUDA(cudaMemsetAsync(m->mcount, 0, kMoverLists * sizeof(unsigned), m->stream));
     if (!fused) {
         int64_t blocks = (v_end - v_begin + 255) / 256;
         if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;

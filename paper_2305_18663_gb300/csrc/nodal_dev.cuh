@@ -42,10 +42,12 @@ struct DecideArgs {
     GraphDev g;
     ModelDev md;
     int64_t v_begin, v_end;
-    Mover *movers;           // four lists: k <= 32, 33..128, > 128, and the movers
-                             // the FP32 test left to the exact evaluation
+    Mover *movers;           // the lists: k <= 32, 33..128, > 128 (split_top: up to kMidDeg,
+                             // up to kWideDeg, more), and the movers the FP32 test left to
+                             // the exact evaluation
     unsigned *mcount;        // their lengths (device counters)
-    int64_t mbase[4];        // their offsets in movers
+    int64_t mbase[kMoverLists];  // their offsets in movers
+    int split_top;
     int force_exact;         // 1: decide every mover by the exact evaluation
     uint64_t seed, sweep_id;
     double beta;
@@ -86,12 +88,12 @@ struct Counts {
 // a mover the FP32 test could not settle (or any mover when a trace is
 // asked for), for the exact evaluation that follows the pass
 __device__ __forceinline__ void push_recheck(const DecideArgs &a, int v, int s, uint64_t w2) {
-    const unsigned i = atomicAdd(&a.mcount[3], 1u);
+    const unsigned i = atomicAdd(&a.mcount[kRecheck], 1u);
     Mover m;
     m.v = v;
     m.s = s;
     m.w2 = w2;
-    a.movers[a.mbase[3] + i] = m;
+    a.movers[a.mbase[kRecheck] + i] = m;
 }
 
 
@@ -442,7 +444,7 @@ __device__ __forceinline__ void count_exact(Counts &c, bool accept, bool margin,
 
 __device__ __forceinline__ void flush_counts(const ModelDev &md, const Counts &c) {
     typedef unsigned long long u64;
-    if (c.proposed | c.moves) {
+    if (c.proposed | c.moves | c.entries) {  // (a warp may have left all its movers to the recheck)
         atomicAdd(&md.counters->proposed, (u64)c.proposed);
         atomicAdd(&md.counters->moves, (u64)c.moves);
         atomicAdd(&md.counters->accepted, (u64)c.accepted);
