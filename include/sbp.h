@@ -149,7 +149,7 @@ void sbp_free_graph(sbp_graph_t *g);
 /* Creates a blockmodel handle for assignment b (n labels in [0, B), host or
  * device) and builds M, block degrees and DL (Eq. 1-2, Section II-A).
  * stream: a cudaStream_t (may be NULL) that every later call on this model
- * orders its work on (the decision pass of a graph with 2^22 edges or more
+ * orders its work on (the decision pass of a graph with 2^19 edges or more
  * runs part of its kernels on two side streams of the model, forked from and
  * joined back into this stream within the call).  p may be NULL
  * (defaults).  The graph must outlive the model.

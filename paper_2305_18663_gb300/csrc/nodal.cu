@@ -1604,9 +1604,14 @@ int cta_table(sbp_model *m, int cap, int sms, int *grid, size_t *smem, unsigned 
     return SBP_OK;
 }
 
-// graphs with at least this many edges run the three degree groups'
-// kernels on three streams
-constexpr int64_t kSideStreamEdges = int64_t(1) << 22;
+// Graphs with at least this many edges run the three degree groups' kernels
+// on three streams: none of them fills the chip (13 to 35% of the warps
+// active at 200k vertices), and each ends in a tail.  One stream and three, a
+// decision pass: 200k vertices, 4M edges at B = 223 223 and 200 us, at 4096
+// 507 and 426, at 65,536 1231 and 903; 100k vertices, 1.6M edges 126 and 99.
+// At 2^18 edges (10,000 vertices, exact form) the fork costs what it gains:
+// 118 and 120 us.
+constexpr int64_t kSideStreamEdges = int64_t(1) << 19;
 
 // streams of the three groups: the model's own one for the movers above 128
 // edges (launched first: the longest tail), side streams for the others
