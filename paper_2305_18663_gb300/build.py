@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libsbp.so")
-SOURCES = ["api.cu", "graph.cu", "blockmodel.cu", "nodal.cu", "merge.cu", "xlogx_table.cu", "sort.cu", "sparse.cu",
+SOURCES = ["api.cu", "graph.cu", "blockmodel.cu", "nodal.cu", "merge.cu", "xlogx_table.cu", "sort.cu", "sparse.cu", "sparse_rows.cu",
            "noalloc.cu", "batch.cu", "engine.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]

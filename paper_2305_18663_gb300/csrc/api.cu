@@ -342,7 +342,7 @@ extern "C" int sbp_build_blockmodel(const sbp_graph_t *g, int32_t B, const int32
     m->g = g;
     m->p = prm;
     m->stream = static_cast<cudaStream_t>(stream);
-    m->npartials = 1024;
+    m->npartials = kPartials;
     const size_t n = (size_t)g->n;
     cudaStream_t st = m->stream;
     m->pinned = pinned_get();
@@ -722,16 +722,19 @@ extern "C" int sbp_get_blockmodel_coo(const sbp_model_t *m, int64_t capacity, in
                 c.push_back(M[(size_t)i]);
             }
     } else {
-        const int64_t z = sparse_nnz(const_cast<sbp_model *>(m));
-        std::vector<uint32_t> rp((size_t)B + 1);
-        std::vector<int32_t> rc((size_t)z), rv((size_t)z);
+        // row r's nonzeros lie at rp[r] .. its end (re, or the next row's begin)
+        std::vector<uint32_t> rp((size_t)B + 1), re((size_t)B);
         SBP_CUDA(cudaMemcpy(rp.data(), m->sp.rp, rp.size() * 4, cudaMemcpyDeviceToHost));
+        if (m->sp.slack) SBP_CUDA(cudaMemcpy(re.data(), m->sp.re, re.size() * 4, cudaMemcpyDeviceToHost));
+        else std::copy(rp.begin() + 1, rp.end(), re.begin());
+        const uint32_t z = re[(size_t)B - 1];
+        std::vector<int32_t> rc((size_t)z), rv((size_t)z);
         if (z > 0) {
             SBP_CUDA(cudaMemcpy(rc.data(), m->sp.rc, (size_t)z * 4, cudaMemcpyDeviceToHost));
             SBP_CUDA(cudaMemcpy(rv.data(), m->sp.rv, (size_t)z * 4, cudaMemcpyDeviceToHost));
         }
         for (int64_t r = 0; r < B; ++r)
-            for (uint32_t i = rp[(size_t)r]; i < rp[(size_t)r + 1]; ++i) {
+            for (uint32_t i = rp[(size_t)r]; i < re[(size_t)r]; ++i) {
                 k.push_back(r * B + rc[i]);
                 c.push_back(rv[i]);
             }

@@ -124,28 +124,31 @@ __global__ void __launch_bounds__(kThreads) k_dl_partial(const int32_t *__restri
 // Eq. 2: DL = E h(B^2/E) + N ln B - L, h(x) = (1+x) ln(1+x) - x ln x.  The
 // partials are summed in a fixed order (strided per thread, then a fixed
 // tree), so the result is reproducible bit for bit.
-__global__ void __launch_bounds__(kThreads) k_dl_final(const DlPartial *__restrict__ partials, int np, int64_t E,
-                                                       int64_t N, int B, double *__restrict__ dl) {
-    __shared__ __int128 sfix[kThreads];
-    __shared__ double sfb[kThreads];
+constexpr int kFinalThreads = 1024;
+__global__ void __launch_bounds__(kFinalThreads) k_dl_final(const DlPartial *__restrict__ partials, int np, int64_t E,
+                                                            int64_t N, int B, double *__restrict__ dl) {
+    __shared__ __int128 sfix[kFinalThreads / 32];
+    __shared__ double sfb[kFinalThreads / 32];
+    __shared__ double model;
+    // the part without the counts (a chain of FP64 logarithms) on a thread of its own
+    if (threadIdx.x == kFinalThreads - 1) model = dl_eq2(E, N, B, 0.0);
     __int128 f = 0;
     double d = 0.0;
-    for (int i = threadIdx.x; i < np; i += blockDim.x) {
+    for (int i = threadIdx.x; i < np; i += kFinalThreads) {
         f += partials[i].fix;
         d += partials[i].fb;
     }
-    sfix[threadIdx.x] = f;
-    sfb[threadIdx.x] = d;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) {
-            sfix[threadIdx.x] += sfix[threadIdx.x + o];
-            sfb[threadIdx.x] += sfb[threadIdx.x + o];
-        }
-        __syncthreads();
+    f = warp_sum_128(f);
+    d = warp_sum(d);
+    if ((threadIdx.x & 31) == 0) {
+        sfix[threadIdx.x >> 5] = f;
+        sfb[threadIdx.x >> 5] = d;
     }
-    if (threadIdx.x == 0) {
-        dl[0] = dl_eq2(E, N, B, fix_to_double(sfix[0]) + sfb[0]);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        f = warp_sum_128(sfix[threadIdx.x]);
+        d = warp_sum(sfb[threadIdx.x]);
+        if (threadIdx.x == 0) dl[0] = model - (fix_to_double(f) + d);
     }
 }
 
@@ -577,8 +580,8 @@ int build_blockmodel(sbp_model *m, bool after_pass) {
     const sbp_graph *g = m->g;
     const int B = m->B;
     SBP_TRY(xlogx_table(g->m + 1, &m->T, &m->XT));
-    const int32_t *vals;
-    int64_t nvals;
+    DlPartial *parts = reinterpret_cast<DlPartial *>(m->partials);
+    int np = 0;
     if (m->dense) {
         const int64_t BB = (int64_t)B * B;
         if (after_pass)
@@ -588,24 +591,19 @@ int build_blockmodel(sbp_model *m, bool after_pass) {
         k_prefix_dense<<<grid_for((int64_t)B * 32, kThreads, 1 << 30), kThreads, 0, m->stream>>>(
             m->M, B, m->P, m->dout, m->din, m->rcp, m->rcp32, m->dsum, m->Pc, (2 * B + 31) / 32);
         SBP_LAUNCHED();
-        vals = m->M;
-        nvals = BB;
+        np = grid_for(BB > B ? BB : B, kThreads * 4, 1024);  // (of kPartials)
+        k_dl_partial<<<np, kThreads, 0, m->stream>>>(m->M, BB, m->dout, m->din, B, m->T, m->XT, parts);
+        SBP_LAUNCHED();
+        k_dl_final<<<1, kFinalThreads, 0, m->stream>>>(parts, np, g->m, g->n, B, m->dl);
+        SBP_LAUNCHED();
     } else {
         bool dl_done = false;
-        SBP_TRY(rebuild_sparse(m, after_pass, &dl_done));
-        if (dl_done) {
-            SBP_CUDA(cudaMemcpyAsync(m->bnew, m->b, (size_t)g->n * 4, cudaMemcpyDeviceToDevice, m->stream));
-            return SBP_OK;
+        SBP_TRY(rebuild_sparse(m, after_pass, &dl_done, &np));
+        if (!dl_done) {
+            k_dl_final<<<1, kFinalThreads, 0, m->stream>>>(parts, np, g->m, g->n, B, m->dl);
+            SBP_LAUNCHED();
         }
-        vals = m->sp.rv;
-        nvals = m->sp.nnz;
     }
-    const int np = grid_for(nvals > B ? nvals : B, kThreads * 4, m->npartials);
-    DlPartial *parts = reinterpret_cast<DlPartial *>(m->partials);
-    k_dl_partial<<<np, kThreads, 0, m->stream>>>(vals, nvals, m->dout, m->din, B, m->T, m->XT, parts);
-    SBP_LAUNCHED();
-    k_dl_final<<<1, kThreads, 0, m->stream>>>(parts, np, g->m, g->n, B, m->dl);
-    SBP_LAUNCHED();
     SBP_CUDA(cudaMemcpyAsync(m->bnew, m->b, (size_t)g->n * 4, cudaMemcpyDeviceToDevice, m->stream));
     return SBP_OK;
 }

@@ -67,6 +67,7 @@ constexpr int kSmallDeg = 32;     // k <= 32: one neighbour per lane, no table
 constexpr int kWarpDeg = 128;     // k <= 128: one warp per vertex, per-warp table
 constexpr int kMidDeg = 512;      // at large B, the classes above 128: up to 512, up to 1600, more
 constexpr int kWideDeg = 1600;
+constexpr int kPartials = 4096;   // partial sums of L a model has room for
 constexpr int kMoverLists = 6;    // a pass's mover lists: five degree classes and the recheck list
 constexpr int kRecheck = 5;
 constexpr int kWarpsPerCta = 8;
@@ -75,13 +76,6 @@ constexpr int64_t kMaxTable = int64_t(1) << 22;  // largest x ln x table (entrie
 
 // ---------------------------------------------------------------------------
 // graph and model state
-// keys computed on the fly from the out-edge list: key of out-edge e is
-// b[esrc[e]] * B + b[oc[e]] (row block, column block)
-struct EdgeKeys {
-    const int32_t *esrc = nullptr, *oc = nullptr, *b = nullptr;
-    uint64_t B = 0;
-};
-
 struct GraphDev {
     int32_t n;
     int64_t m;
@@ -99,6 +93,7 @@ struct sbp_graph {
     int device = 0;
     unsigned char *slab = nullptr;  // the one allocation behind the arrays below (but self_in)
     int32_t *op = nullptr, *ip = nullptr, *oc = nullptr, *ic = nullptr, *esrc = nullptr;
+    int32_t *idst = nullptr;  // target vertex of each in-row entry
     int32_t *tw_oi = nullptr, *tw_io = nullptr;  // twin positions of each edge in the other CSR
     int32_t *self_in = nullptr;  // in-row positions of the self-loops
     int64_t n_self = 0;
@@ -154,7 +149,8 @@ struct ModelDev {
     // sparse form (B > dense_max_B): CSR and CSC of M with per-row / per-column
     // inclusive count prefixes, and per-row open-addressing tables
     int sparse;
-    const uint32_t *rp, *cp, *hoff;   // [B+1]
+    const uint32_t *rp, *re, *cp, *ce;  // [B] begin and end of each row, each column
+    const uint32_t *hoff;               // [B+1]
     const int32_t *rc, *cr;           // column of each row entry, row of each column entry
     const int32_t *rv, *cv;           // their counts
     const uint32_t *rpre, *cpre;      // inclusive count prefixes inside each row / column
@@ -176,21 +172,21 @@ constexpr int32_t kNbSelf = INT32_MIN;  // self-loop bit of a block-labelled ent
 
 struct sbp_model {
     struct Sparse {
-        int64_t cap_e = 0, nnz = 0;
+        int64_t cap_e = 0;
         int32_t cap_b = 0;
-        uint64_t *key0 = nullptr, *key1 = nullptr;
-        uint32_t *start = nullptr, *scratch = nullptr;
-        int32_t *rc = nullptr, *rv = nullptr, *rowof = nullptr, *cr = nullptr, *cv = nullptr;
+        uint32_t *vo = nullptr, *vi = nullptr;  // a vertex's slots in its block's row and column
+        int32_t *lo = nullptr, *li = nullptr;   // far-end labels by row, by column
+        uint32_t *scratch = nullptr;            // kSparseScratch words
+        int32_t *rc = nullptr, *rv = nullptr, *cr = nullptr, *cv = nullptr;
         uint32_t *rpre = nullptr, *cpre = nullptr;
-        uint32_t *ckey0 = nullptr, *ckey1 = nullptr;
-        uint64_t *cval0 = nullptr, *cval1 = nullptr;
         int2 *hkv = nullptr;  // per-row open-addressing slots (key, count)
-        uint32_t *rp = nullptr, *cp = nullptr, *hoff = nullptr, *cnt = nullptr;
+        uint32_t *rp = nullptr, *re = nullptr, *cp = nullptr, *ce = nullptr, *hoff = nullptr;
+        bool slack = false;  // rows end at re / ce; else where the next one begins
+        uint32_t *rcur = nullptr, *ccur = nullptr, *lists = nullptr;
         uint32_t *rpc = nullptr, *cpc = nullptr;  // [B * 32] coarse pivots of rpre / cpre per row / column
-        int32_t *cells = nullptr;  // B x B counts of the counting-sort rebuild
+        int32_t *cells = nullptr;  // B x B counts of a small sparse model
         int64_t cap_cells = 0;
         int32_t cells_B = 0;       // B the cells hold the counts of m->bnew for, else 0
-        int64_t *nnz_dev = nullptr;  // the nonzero count when only the device has it (nnz < 0)
     };
     Sparse sp;
     const sbp_graph *g = nullptr;
@@ -589,10 +585,10 @@ __device__ __forceinline__ uint32_t pivot_upper(const uint32_t *pre, const uint3
 // M[c][u]), t < dout_u + din_u: the block at that position.  One lane.
 __device__ __forceinline__ int sparse_cdf_block(const ModelDev &md, int u, uint32_t t, uint32_t dout_u) {
     if (t < dout_u) {
-        const uint32_t i = pivot_upper(md.rpre, md.rpc + (size_t)u * 32, md.rp[u], md.rp[u + 1], t);
+        const uint32_t i = pivot_upper(md.rpre, md.rpc + (size_t)u * 32, md.rp[u], md.re[u], t);
         return md.rc[i];
     }
-    const uint32_t i = pivot_upper(md.cpre, md.cpc + (size_t)u * 32, md.cp[u], md.cp[u + 1], t - dout_u);
+    const uint32_t i = pivot_upper(md.cpre, md.cpc + (size_t)u * 32, md.cp[u], md.ce[u], t - dout_u);
     return md.cr[i];
 }
 
@@ -657,8 +653,9 @@ int ensure_capacity(sbp_model *m, int32_t B);
 int check_status(const sbp_model *m);
 int xlogx_table(int64_t need, const __int128 **table, int64_t *size);
 int ensure_sparse_capacity(sbp_model *m, int32_t B);
-int rebuild_sparse(sbp_model *m, bool after_pass, bool *dl_done);
-int64_t sparse_nnz(sbp_model *m);  // the nonzero count (read back once when only the device has it)
+int rebuild_sparse(sbp_model *m, bool after_pass, bool *dl_done, int *n_parts);
+int build_sparse_rows(sbp_model *m, int *n_parts);  // sparse_rows.cu
+constexpr int64_t kSparseScratch = 20000;  // words: the small rebuild's lengths and sums, or a cluster's exchange
 void free_sparse(sbp_model *m);
 
 // sort.cu: exclusive scan of n uint32 (in may equal out; *total_dev, device,
@@ -667,11 +664,10 @@ int exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *t
                        cudaStream_t st);
 int64_t scan_scratch_words(int64_t n);
 int64_t sort_scratch_words(int64_t n);
-int sort_chunk_count(int64_t n);
-int64_t sort_chunk_length(int64_t n);
 template <class K, class V>
-int radix_sort(K *k0, K *k1, V *v0, V *v1, int64_t n, int bits, uint32_t *scratch, cudaStream_t st, bool *in_first,
-               const EdgeKeys *edges = nullptr);
+int radix_sort(K *k0, K *k1, V *v0, V *v1, int64_t n, int bits, uint32_t *scratch, cudaStream_t st, bool *in_first);
 ModelDev model_dev(sbp_model *m);
+int fork_side(sbp_model *m, cudaStream_t st[3]);
+int join_side(sbp_model *m);
 
 }  // namespace sbp

@@ -91,12 +91,13 @@ __global__ void __launch_bounds__(kT) k_out_rows(const K *__restrict__ keys, int
 // a repeated edge is paired with its k-th copy.
 __global__ void __launch_bounds__(kT) k_in_rows(const uint32_t *__restrict__ ikey, const uint32_t *__restrict__ ival,
                                                 const int32_t *__restrict__ esrc, int64_t m, int32_t *__restrict__ ic,
-                                                int32_t *__restrict__ tw_oi, int32_t *__restrict__ tw_io,
+                                                int32_t *__restrict__ idst, int32_t *__restrict__ tw_oi, int32_t *__restrict__ tw_io,
                                                 Info *__restrict__ info) {
     for (int64_t j = (int64_t)blockIdx.x * kT + threadIdx.x; j < m; j += (int64_t)gridDim.x * kT) {
         const uint32_t e = ival[j];
         const int32_t s = esrc[e];
         ic[j] = s;
+        idst[j] = (int32_t)ikey[j];
         tw_io[j] = (int32_t)e;
         tw_oi[e] = (int32_t)j;
         if ((uint32_t)s == ikey[j]) atomicAdd(&info->n_self, 1ull);
@@ -258,7 +259,8 @@ int build_graph(sbp_graph *g, const int32_t *src, const int32_t *dst, const Scra
         SBP_TRY((radix_sort<uint32_t, uint32_t>(x.i0, x.i1, x.v0, x.v1, m, bits_for((uint64_t)n - 1), x.words, st,
                                                 &first)));
         *ikey = first ? x.i0 : x.i1;
-        k_in_rows<<<grid_of(m), kT, 0, st>>>(*ikey, first ? x.v0 : x.v1, g->esrc, m, g->ic, g->tw_oi, g->tw_io, x.info);
+        k_in_rows<<<grid_of(m), kT, 0, st>>>(*ikey, first ? x.v0 : x.v1, g->esrc, m, g->ic, g->idst,
+                                                  g->tw_oi, g->tw_io, x.info);
         SBP_LAUNCHED();
     }
     k_row_offsets<<<grid_of(n + 1), kT, 0, st>>>(g->esrc, *ikey, m, n, g->op, g->ip);
@@ -302,6 +304,7 @@ void carve_graph(sbp_graph *g, Carver &c) {
     c.take(&g->oc, m);
     c.take(&g->ic, m);
     c.take(&g->esrc, m);
+    c.take(&g->idst, m);
     c.take(&g->tw_oi, m);
     c.take(&g->tw_io, m);
     c.take(&g->order, n);

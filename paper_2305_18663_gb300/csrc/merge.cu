@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge_proposals(ModelDev md, 
         bool mine = at < count;
         const int r = mine ? (long_pass ? longs[at] : (int)at) : 0;
         if (mine && !long_pass && longs) {
-            const uint32_t len = md.rp[r + 1] - md.rp[r] + md.cp[r + 1] - md.cp[r];
+            const uint32_t len = md.re[r] - md.rp[r] + md.ce[r] - md.cp[r];
             if (len > kMergeLong) {
                 if (lane == 0) longs[atomicAdd(n_long, 1u)] = r;  // parts == 1 here
                 mine = false;

@@ -73,7 +73,7 @@ __device__ __forceinline__ int merge_propose(const ModelDev &md, int r, uint64_t
         // the same walks over the nonzeros of row u / column u, entry r left
         // out (where it is zero there is nothing to step over)
         if (t < row_w) {
-            const uint32_t a = md.rp[u], z = md.rp[u + 1];
+            const uint32_t a = md.rp[u], z = md.re[u];
             int64_t tt = t;
             if (Mur != 0) {
                 const uint32_t pos = lane_lower_i32(md.rc, a, z, r);
@@ -82,7 +82,7 @@ __device__ __forceinline__ int merge_propose(const ModelDev &md, int r, uint64_t
             }
             return md.rc[pivot_upper(md.rpre, md.rpc + (size_t)u * 32, a, z, (uint32_t)tt)];
         }
-        const uint32_t a = md.cp[u], z = md.cp[u + 1];
+        const uint32_t a = md.cp[u], z = md.ce[u];
         int64_t tt = t - row_w;
         if (Mru != 0) {
             const uint32_t pos = lane_lower_i32(md.cr, a, z, r);
@@ -222,7 +222,7 @@ __device__ __forceinline__ void merge_rows(const ModelDev &md, int r, int part, 
     const int lane = threadIdx.x & 31, B = md.B;
     int nq = 0;
     if (md.sparse) {
-        const uint32_t r0 = md.rp[r], rlen = md.rp[r + 1] - r0, c0 = md.cp[r], clen = md.cp[r + 1] - c0;
+        const uint32_t r0 = md.rp[r], rlen = md.re[r] - r0, c0 = md.cp[r], clen = md.ce[r] - c0;
         for (uint32_t b0 = 32u * part; b0 < rlen; b0 += 32u * parts) {
             const uint32_t i = b0 + lane;
             const int t = i < rlen ? md.rc[r0 + i] : r;

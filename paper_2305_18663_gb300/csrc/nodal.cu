@@ -241,8 +241,8 @@ __device__ __forceinline__ void table_move_sparse(const DecideArgs &a, const Tab
     const ModelDev &md = a.md;
     const int r = x.r, s = x.s;
     // segments: row r, row s, column r, column s
-    const uint32_t r0 = md.rp[r], r1 = md.rp[r + 1], s0 = md.rp[s], s1 = md.rp[s + 1];
-    const uint32_t cr0 = md.cp[r], cr1 = md.cp[r + 1], cs0 = md.cp[s], cs1 = md.cp[s + 1];
+    const uint32_t r0 = md.rp[r], r1 = md.re[r], s0 = md.rp[s], s1 = md.re[s];
+    const uint32_t cr0 = md.cp[r], cr1 = md.ce[r], cs0 = md.cp[s], cs1 = md.ce[s];
     const uint32_t most = (uint32_t)(kStreamRatio * nl + 32);
     const bool st_r = r1 - r0 <= most, st_s = s1 - s0 <= most, st_cr = cr1 - cr0 <= most, st_cs = cs1 - cs0 <= most;
     const uint32_t e0 = st_r ? r1 - r0 : 0u, e1 = e0 + (st_s ? s1 - s0 : 0u), e2 = e1 + (st_cr ? cr1 - cr0 : 0u),
@@ -1535,6 +1535,44 @@ int sm_count() {
 
 }  // namespace
 
+// Graphs with at least this many edges run the three degree groups' kernels
+// on three streams: none of them fills the chip (13 to 35% of the warps
+// active at 200k vertices), and each ends in a tail.  One stream and three, a
+// decision pass: 200k vertices, 4M edges at B = 223 223 and 200 us, at 4096
+// 507 and 426, at 65,536 1231 and 903; 100k vertices, 1.6M edges 126 and 99.
+// At 2^18 edges (10,000 vertices, exact form) the fork costs what it gains:
+// 118 and 120 us.
+static constexpr int64_t kSideStreamEdges = int64_t(1) << 19;
+
+// three streams for kernels that may run together: the model's own one (for
+// the longest) and its side streams, forked here and joined by join_side (all
+// the model's own on smaller graphs)
+int fork_side(sbp_model *m, cudaStream_t st[3]) {
+    st[0] = st[1] = st[2] = m->stream;
+    if (m->g->m < kSideStreamEdges) return SBP_OK;
+    if (!m->fork_ev) {
+        for (int i = 0; i < 2; ++i) {
+            SBP_CUDA(cudaStreamCreateWithFlags(&m->side[i], cudaStreamNonBlocking));
+            SBP_CUDA(cudaEventCreateWithFlags(&m->join_ev[i], cudaEventDisableTiming));
+        }
+        SBP_CUDA(cudaEventCreateWithFlags(&m->fork_ev, cudaEventDisableTiming));
+    }
+    SBP_CUDA(cudaEventRecord(m->fork_ev, m->stream));
+    for (int i = 0; i < 2; ++i) SBP_CUDA(cudaStreamWaitEvent(m->side[i], m->fork_ev, 0));
+    st[0] = m->side[1];
+    st[1] = m->side[0];
+    return SBP_OK;
+}
+
+int join_side(sbp_model *m) {
+    if (m->g->m < kSideStreamEdges || !m->fork_ev) return SBP_OK;
+    for (int i = 0; i < 2; ++i) {
+        SBP_CUDA(cudaEventRecord(m->join_ev[i], m->side[i]));
+        SBP_CUDA(cudaStreamWaitEvent(m->stream, m->join_ev[i], 0));
+    }
+    return SBP_OK;
+}
+
 ModelDev model_dev(sbp_model *m) {
     ModelDev d;
     d.B = m->B;
@@ -1555,7 +1593,9 @@ ModelDev model_dev(sbp_model *m) {
     d.XT = m->XT;
     d.sparse = m->dense ? 0 : 1;
     d.rp = m->sp.rp;
+    d.re = m->sp.slack ? m->sp.re : m->sp.rp + 1;
     d.cp = m->sp.cp;
+    d.ce = m->sp.slack ? m->sp.ce : m->sp.cp + 1;
     d.hoff = m->sp.hoff;
     d.rc = m->sp.rc;
     d.cr = m->sp.cr;
@@ -1601,44 +1641,6 @@ int cta_table(sbp_model *m, int cap, int sms, int *grid, size_t *smem, unsigned 
         m->cta_tab_bytes = need;
     }
     *gtab = m->cta_tab;
-    return SBP_OK;
-}
-
-// Graphs with at least this many edges run the three degree groups' kernels
-// on three streams: none of them fills the chip (13 to 35% of the warps
-// active at 200k vertices), and each ends in a tail.  One stream and three, a
-// decision pass: 200k vertices, 4M edges at B = 223 223 and 200 us, at 4096
-// 507 and 426, at 65,536 1231 and 903; 100k vertices, 1.6M edges 126 and 99.
-// At 2^18 edges (10,000 vertices, exact form) the fork costs what it gains:
-// 118 and 120 us.
-constexpr int64_t kSideStreamEdges = int64_t(1) << 19;
-
-// streams of the three groups: the model's own one for the movers above 128
-// edges (launched first: the longest tail), side streams for the others
-// (forked after k_propose, joined back by join_evals)
-int fork_evals(sbp_model *m, cudaStream_t st[3]) {
-    st[0] = st[1] = st[2] = m->stream;
-    if (m->g->m < kSideStreamEdges) return SBP_OK;
-    if (!m->fork_ev) {
-        for (int i = 0; i < 2; ++i) {
-            SBP_CUDA(cudaStreamCreateWithFlags(&m->side[i], cudaStreamNonBlocking));
-            SBP_CUDA(cudaEventCreateWithFlags(&m->join_ev[i], cudaEventDisableTiming));
-        }
-        SBP_CUDA(cudaEventCreateWithFlags(&m->fork_ev, cudaEventDisableTiming));
-    }
-    SBP_CUDA(cudaEventRecord(m->fork_ev, m->stream));
-    for (int i = 0; i < 2; ++i) SBP_CUDA(cudaStreamWaitEvent(m->side[i], m->fork_ev, 0));
-    st[0] = m->side[1];
-    st[1] = m->side[0];
-    return SBP_OK;
-}
-
-int join_evals(sbp_model *m) {
-    if (m->g->m < kSideStreamEdges || !m->fork_ev) return SBP_OK;
-    for (int i = 0; i < 2; ++i) {
-        SBP_CUDA(cudaEventRecord(m->join_ev[i], m->side[i]));
-        SBP_CUDA(cudaStreamWaitEvent(m->stream, m->join_ev[i], 0));
-    }
     return SBP_OK;
 }
 
@@ -1762,9 +1764,9 @@ int launch_small(sbp_model *m, const DecideArgs &a, int sms) {
 template <bool DL32>
 int launch_evals(sbp_model *m, const DecideArgs &a, int sms, bool fused) {
     cudaStream_t st[3];
-    SBP_TRY(fork_evals(m, st));
+    SBP_TRY(fork_side(m, st));
     const int rc = fused ? launch_groups<DL32, true>(m, a, sms, st) : launch_groups<DL32, false>(m, a, sms, st);
-    const int rj = join_evals(m);  // joined on every path
+    const int rj = join_side(m);  // joined on every path
     if (rc != SBP_OK) return rc;
     if (rj != SBP_OK) return rj;
     return launch_recheck<DL32>(m, a, sms);

@@ -1,7 +1,7 @@
 // sort.cu -- device-wide exclusive scan and LSD radix sort.
 //
-// Used by the sparse blockmodel rebuild: the (b[src], b[dst]) keys of all
-// edges are sorted, then run-length encoded into the nonzeros of M.
+// Used when a graph is loaded: the (source, target) keys of all edges, the
+// out-rows' positions by target, and the vertex orders by degree.
 // Stable by construction: each pass keeps the order of equal digits, so the
 // passes compose into a sort on the whole key.
 #include "common.cuh"
@@ -133,8 +133,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const uint32_t *__re
 // in both kernels of a pass:
 //   k_rs_count: per chunk, a histogram of the pass's digit, stored
 //     digit-major (hist[d * G + chunk]); an exclusive scan of it gives every
-//     (digit, chunk) its first output position.  For the first pass of the
-//     edge sort it also makes the keys (b[src] * B + b[dst]) and writes them;
+//     (digit, chunk) its first output position;
 //   k_rs_scatter: the chunk is walked in rounds of 4096 keys.  A key's rank
 //     among the earlier keys of its digit in the round comes from warp
 //     match/popc (per item) and per-warp digit counts; the round is
@@ -150,18 +149,9 @@ constexpr int kRsRound = kRsThreads * kRsItems;    // keys per round
 constexpr int kRsMaxBins = 512;
 constexpr int64_t kRsMaxChunks = 2048;
 
-template <class K, bool EDGES>
-__device__ __forceinline__ K rs_key(const K *__restrict__ keys, const EdgeKeys &ek, int64_t i) {
-    if constexpr (EDGES)
-        return (K)((uint64_t)ek.b[ek.esrc[i]] * ek.B + (uint64_t)ek.b[ek.oc[i]]);
-    else
-        return keys[i];
-}
-
-template <class K, bool EDGES>
-__global__ void __launch_bounds__(kRsThreads) k_rs_count(const K *__restrict__ keys, EdgeKeys ek, int64_t n,
-                                                         int64_t chunk, int shift, int nbins, int G,
-                                                         uint32_t *__restrict__ hist, K *__restrict__ kout) {
+template <class K>
+__global__ void __launch_bounds__(kRsThreads) k_rs_count(const K *__restrict__ keys, int64_t n, int64_t chunk, int shift,
+                                                         int nbins, int G, uint32_t *__restrict__ hist) {
     __shared__ uint32_t h[kRsMaxBins];
     for (int d = threadIdx.x; d < nbins; d += kRsThreads) h[d] = 0;
     __syncthreads();
@@ -175,14 +165,11 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_count(const K *__restrict__ k
         for (int j = 0; j < 4; ++j) {
             const int64_t i = base + j * kRsThreads + threadIdx.x;
             ok[j] = i < end;
-            k[j] = ok[j] ? rs_key<K, EDGES>(keys, ek, i) : (K)0;
+            k[j] = ok[j] ? keys[i] : (K)0;
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (ok[j]) {
-                if (EDGES) kout[base + j * kRsThreads + threadIdx.x] = k[j];
-                atomicAdd(&h[(int)(((uint64_t)k[j] >> shift) & mask)], 1u);
-            }
+            if (ok[j]) atomicAdd(&h[(int)(((uint64_t)k[j] >> shift) & mask)], 1u);
         }
     }
     __syncthreads();
@@ -335,23 +322,17 @@ size_t rs_stage_bytes(bool with_vals) {
     return (size_t)kRsRound * (sizeof(K) + (with_vals ? sizeof(V) : 0));
 }
 
-// one pass: keys from ks (or, with ek.b set, made from the edge list and
-// written to kmade first), digits [shift, shift + nbits)
+// one pass over digits [shift, shift + nbits)
 template <class K, class V>
-int rs_pass(const K *ks, const V *vs, const EdgeKeys &ek, K *kmade, int64_t n, int shift, int nbits, K *kd, V *vd,
-            uint32_t *scratch, cudaStream_t st) {
+int rs_pass(const K *ks, const V *vs, int64_t n, int shift, int nbits, K *kd, V *vd, uint32_t *scratch,
+            cudaStream_t st) {
     int64_t chunk;
     int G;
     rs_chunks(n, &chunk, &G);
     const int nbins = 1 << nbits;
     uint32_t *hist = scratch;
     uint32_t *sscr = scratch + (int64_t)kRsMaxBins * kRsMaxChunks;
-    if (ek.b) {
-        k_rs_count<K, true><<<G, kRsThreads, 0, st>>>(nullptr, ek, n, chunk, shift, nbins, G, hist, kmade);
-        ks = kmade;
-    } else {
-        k_rs_count<K, false><<<G, kRsThreads, 0, st>>>(ks, ek, n, chunk, shift, nbins, G, hist, nullptr);
-    }
+    k_rs_count<K><<<G, kRsThreads, 0, st>>>(ks, n, chunk, shift, nbins, G, hist);
     SBP_LAUNCHED();
     SBP_TRY(exclusive_scan_u32(hist, hist, (int64_t)nbins * G, nullptr, sscr, st));
     const size_t smem = rs_stage_bytes<K, V>(vs != nullptr);
@@ -368,39 +349,20 @@ int64_t sort_scratch_words(int64_t) {
     return (int64_t)kRsMaxBins * kRsMaxChunks + scan_scratch_words((int64_t)kRsMaxBins * kRsMaxChunks);
 }
 
-int sort_chunk_count(int64_t n) {
-    int64_t chunk;
-    int G;
-    rs_chunks(n, &chunk, &G);
-    return G;
-}
-
-int64_t sort_chunk_length(int64_t n) {
-    int64_t chunk;
-    int G;
-    rs_chunks(n, &chunk, &G);
-    return chunk;
-}
-
 // Stable LSD radix sort on the low `bits` bits of the keys, ceil(bits / 9)
 // passes.  The result lands in k0/v0 or k1/v1 according to the parity of the
-// pass count; *in_first tells which.  vals may be NULL.  With `edges`, the
-// first pass makes the keys from the edge list and writes them to k0 (whose
-// contents on entry are ignored).
+// pass count; *in_first tells which.  vals may be NULL.
 template <class K, class V>
-int radix_sort(K *k0, K *k1, V *v0, V *v1, int64_t n, int bits, uint32_t *scratch, cudaStream_t st, bool *in_first,
-               const EdgeKeys *edges) {
+int radix_sort(K *k0, K *k1, V *v0, V *v1, int64_t n, int bits, uint32_t *scratch, cudaStream_t st, bool *in_first) {
     const int passes = (bits + 8) / 9;
     const int width = (bits + passes - 1) / passes;
     K *ks = k0, *kd = k1;
     V *vs = v0, *vd = v1;
-    const EdgeKeys none{};
     if (n > 0) {
         for (int p = 0; p < passes; ++p) {
             const int shift = p * width;
             const int nbits = bits - shift < width ? bits - shift : width;
-            // the first pass of the edge sort makes the keys into k0 (= ks)
-            SBP_TRY((rs_pass<K, V>(ks, vs, (p == 0 && edges) ? *edges : none, ks, n, shift, nbits, kd, vd, scratch, st)));
+            SBP_TRY((rs_pass<K, V>(ks, vs, n, shift, nbits, kd, vd, scratch, st)));
             std::swap(ks, kd);
             std::swap(vs, vd);
         }
@@ -409,12 +371,9 @@ int radix_sort(K *k0, K *k1, V *v0, V *v1, int64_t n, int bits, uint32_t *scratc
     return SBP_OK;
 }
 
-#define SBP_RS_INST(K, V) \
-    template int radix_sort<K, V>(K *, K *, V *, V *, int64_t, int, uint32_t *, cudaStream_t, bool *, const EdgeKeys *);
-SBP_RS_INST(uint64_t, uint64_t)
-SBP_RS_INST(uint64_t, uint32_t)
-SBP_RS_INST(uint32_t, uint64_t)
-SBP_RS_INST(uint32_t, uint32_t)
-#undef SBP_RS_INST
+template int radix_sort<uint64_t, uint32_t>(uint64_t *, uint64_t *, uint32_t *, uint32_t *, int64_t, int, uint32_t *,
+                                            cudaStream_t, bool *);
+template int radix_sort<uint32_t, uint32_t>(uint32_t *, uint32_t *, uint32_t *, uint32_t *, int64_t, int, uint32_t *,
+                                            cudaStream_t, bool *);
 
 }  // namespace sbp
