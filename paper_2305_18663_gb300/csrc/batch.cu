@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                     for (int r = wid; r < B; r += kBatchWarps) {
                         int bs;
                         double bd;
-                        merge_best(md, sa.seed, rid, J.merge_x, r, 0, 1, mqueue[wid], [](MergeSum &) {}, bs, bd);
+                        merge_best<false>(md, sa.seed, rid, J.merge_x, r, 0, 1, mqueue[wid], [](MergeSum &) {}, bs, bd);
                         if (lane == 0) {
                             J.best_s[r] = bs;
                             J.best_d[r] = bd;

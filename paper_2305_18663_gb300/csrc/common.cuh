@@ -584,12 +584,10 @@ __device__ __forceinline__ uint32_t pivot_upper(const uint32_t *pre, const uint3
 // Sparse inverse CDF over row u then column u of M (weights M[u][c], then
 // M[c][u]), t < dout_u + din_u: the block at that position.  One lane.
 __device__ __forceinline__ int sparse_cdf_block(const ModelDev &md, int u, uint32_t t, uint32_t dout_u) {
-    if (t < dout_u) {
-        const uint32_t i = pivot_upper(md.rpre, md.rpc + (size_t)u * 32, md.rp[u], md.re[u], t);
-        return md.rc[i];
-    }
-    const uint32_t i = pivot_upper(md.cpre, md.cpc + (size_t)u * 32, md.cp[u], md.ce[u], t - dout_u);
-    return md.cr[i];
+    const bool row = t < dout_u;  // (one search for both: half the code)
+    const uint32_t i = pivot_upper(row ? md.rpre : md.cpre, (row ? md.rpc : md.cpc) + (size_t)u * 32,
+                                   (row ? md.rp : md.cp)[u], (row ? md.re : md.ce)[u], row ? t : t - dout_u);
+    return (row ? md.rc : md.cr)[i];
 }
 
 // ---------------------------------------------------------------------------

@@ -16,6 +16,7 @@ constexpr uint32_t kMergeLong = 512;
 // Teams of `parts` warps (1, 2, 4 or 8) take the blocks in turn.  long_pass
 // 0: the blocks 0 .. B-1; with `longs`, blocks of more than kMergeLong
 // entries are only listed there.  long_pass 1: the listed blocks.
+template <bool SPARSE>
 __global__ void __launch_bounds__(kMergeThreads) k_merge_proposals(ModelDev md, uint64_t seed, uint64_t round_id, int x,
                                                                    int parts, int32_t *__restrict__ longs,
                                                                    unsigned *__restrict__ n_long, int long_pass,
@@ -43,7 +44,7 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge_proposals(ModelDev md, 
         // block works on block 0 and drops the result)
         int bs;
         double bd;
-        merge_best(md, seed, round_id, x, r, part, parts, queue[wid], [&](MergeSum &sum) {
+        merge_best<SPARSE>(md, seed, round_id, x, r, part, parts, queue[wid], [&](MergeSum &sum) {
             if (parts == 1) return;
             s_fix[wid][lane] = sum.fix;
             s_fb[wid][lane] = sum.fb;
@@ -165,11 +166,12 @@ int launch_merge_proposals(sbp_model *m, uint64_t round_id) {
     const int teams = kMergeWarps / parts;
     const int64_t blocks = ((int64_t)m->B + teams - 1) / teams;
     const int grid = (int)(blocks < (int64_t)sms * 8 ? blocks : (int64_t)sms * 8);
-    k_merge_proposals<<<grid, kMergeThreads, 0, m->stream>>>(md, m->p.seed, round_id, x, parts, longs, n_long, 0,
+    const auto kern = md.sparse ? k_merge_proposals<true> : k_merge_proposals<false>;
+    kern<<<grid, kMergeThreads, 0, m->stream>>>(md, m->p.seed, round_id, x, parts, longs, n_long, 0,
                                                              m->best_s, m->best_d);
     SBP_LAUNCHED();
     if (longs) {
-        k_merge_proposals<<<sms * 4, kMergeThreads, 0, m->stream>>>(md, m->p.seed, round_id, x, kMergeWarps, longs,
+        kern<<<sms * 4, kMergeThreads, 0, m->stream>>>(md, m->p.seed, round_id, x, kMergeWarps, longs,
                                                                     n_long, 1, m->best_s, m->best_d);
         SBP_LAUNCHED();
     }

@@ -30,8 +30,8 @@
 // Before, one warp walked the row once per proposal with FP64 log1p terms
 // (1/64 rate: a term of 2 log1p and 2 divisions took some 1500 cycles of the
 // SM).  Merge proposals of a 200k-vertex, 4M-edge graph, x = 10, before and
-// after: B = 200,000 9.0 -> 2.8 ms, 25,000 10.4 -> 2.0 ms (sparse), 3125 dense
-// 41.4 -> 0.44 ms, 1000 5.7 -> 0.15 ms.  What bounds it now is the latency of
+// after: B = 200,000 9.0 -> 2.2 ms, 25,000 10.4 -> 1.8 ms (sparse), 3125 dense
+// 41.4 -> 0.39 ms, 1000 5.7 -> 0.14 ms.  What bounds it now is the latency of
 // the dependent lookups (row offset, table slot, term).
 #pragma once
 
@@ -43,10 +43,11 @@
 namespace sbp {
 namespace {
 
-constexpr int kMergeQueue = 64;  // entries queued per warp (processed from 32 on)
+constexpr int kMergeQueue = 160;  // entries queued per warp (worked off from 32 on, up to 128 join at a time)
 
 // Proposal of block r on one lane (every search a single-lane one, so the
 // lanes of a warp can draw different proposals of r at once).
+template <bool SPARSE>
 __device__ __forceinline__ int merge_propose(const ModelDev &md, int r, uint64_t w0, uint64_t w1) {
     const int B = md.B;
     const int64_t dr = (int64_t)md.dout[r] + md.din[r];
@@ -56,7 +57,7 @@ __device__ __forceinline__ int merge_propose(const ModelDev &md, int r, uint64_t
     }
     const int64_t t0 = draw_below(w0, (uint64_t)dr);
     int u;
-    if (md.sparse) {
+    if (SPARSE) {
         u = sparse_cdf_block(md, r, (uint32_t)t0, (uint32_t)md.dout[r]);
     } else {
         u = (int)pivot_upper(md.P + (size_t)r * 2 * B, md.Pc + (size_t)r * 32, 0, 2 * B, (uint32_t)t0);
@@ -69,40 +70,29 @@ __device__ __forceinline__ int merge_propose(const ModelDev &md, int r, uint64_t
     if (y < B - 1) return (int)(y + (y >= r));
     const int64_t t = y - (B - 1);
     const int64_t row_w = du_out - Mur;
-    if (md.sparse) {
-        // the same walks over the nonzeros of row u / column u, entry r left
+    if (SPARSE) {
+        // the same walk over the nonzeros of row u or column u, entry r left
         // out (where it is zero there is nothing to step over)
-        if (t < row_w) {
-            const uint32_t a = md.rp[u], z = md.re[u];
-            int64_t tt = t;
-            if (Mur != 0) {
-                const uint32_t pos = lane_lower_i32(md.rc, a, z, r);
-                const int64_t pre = pos > a ? (int64_t)md.rpre[pos - 1] : 0;
-                tt = t >= pre ? t + Mur : t;
-            }
-            return md.rc[pivot_upper(md.rpre, md.rpc + (size_t)u * 32, a, z, (uint32_t)tt)];
+        const bool row = t < row_w;
+        const uint32_t a = (row ? md.rp : md.cp)[u], z = (row ? md.re : md.ce)[u];
+        const uint32_t *prefix = row ? md.rpre : md.cpre;
+        const int64_t own = row ? Mur : Mru;
+        int64_t tt = row ? t : t - row_w;
+        if (own != 0) {
+            const uint32_t pos = lane_lower_i32(row ? md.rc : md.cr, a, z, r);
+            const int64_t pre = pos > a ? (int64_t)prefix[pos - 1] : 0;
+            if (tt >= pre) tt += own;
         }
-        const uint32_t a = md.cp[u], z = md.ce[u];
-        int64_t tt = t - row_w;
-        if (Mru != 0) {
-            const uint32_t pos = lane_lower_i32(md.cr, a, z, r);
-            const int64_t pre = pos > a ? (int64_t)md.cpre[pos - 1] : 0;
-            if (tt >= pre) tt += Mru;
-        }
-        return md.cr[pivot_upper(md.cpre, md.cpc + (size_t)u * 32, a, z, (uint32_t)tt)];
+        return (row ? md.rc : md.cr)[pivot_upper(prefix, (row ? md.rpc : md.cpc) + (size_t)u * 32, a, z, (uint32_t)tt)];
     }
-    const uint32_t *Pu = md.P + (size_t)u * 2 * B, *Pcu = md.Pc + (size_t)u * 32;
-    if (t < row_w) {
-        // row u with column r left out
-        const int64_t pre = r > 0 ? (int64_t)Pu[r - 1] : 0;
-        const int64_t tt = t >= pre ? t + Mur : t;
-        return (int)pivot_upper(Pu, Pcu, 0, 2 * B, (uint32_t)tt);
-    }
-    // column u with row r left out; Pu[B + c] = dout_u + column prefix
-    const int64_t pre = r > 0 ? (int64_t)Pu[B + r - 1] : du_out;
-    int64_t target = du_out + (t - row_w);
-    if (target >= pre) target += Mru;
-    return (int)pivot_upper(Pu, Pcu, 0, 2 * B, (uint32_t)target) - B;
+    // dense: row u with column r left out, then column u with row r left out;
+    // Pu[B + c] = dout_u + column prefix
+    const uint32_t *Pu = md.P + (size_t)u * 2 * B;
+    const bool row = t < row_w;
+    const int64_t pre = row ? (r > 0 ? (int64_t)Pu[r - 1] : 0) : (r > 0 ? (int64_t)Pu[B + r - 1] : du_out);
+    int64_t target = row ? t : du_out + (t - row_w);
+    if (target >= pre) target += row ? Mur : Mru;
+    return (int)pivot_upper(Pu, md.Pc + (size_t)u * 32, 0, 2 * B, (uint32_t)target) - (row ? 0 : B);
 }
 
 // a sum of terms: exact inside the table, FP64 beyond it
@@ -149,12 +139,13 @@ struct MergeLane {
 
 // n queued entries (t, count; bit 31 of t set for a column entry M[t][r])
 // against the lane's proposal
+template <bool SPARSE>
 __device__ __forceinline__ void merge_entries(const ModelDev &md, const int2 *queue, int n, const MergeLane &L,
                                               MergeSum &sum) {
     constexpr int kU = 4;
     for (int i0 = L.g; i0 < n; i0 += kU * L.G) {
         int a[kU], v[kU];
-        if (md.sparse) {
+        if (SPARSE) {
             uint32_t off[kU], cap[kU], h[kU];
             int key[kU];
             int2 kv[kU];
@@ -199,65 +190,65 @@ __device__ __forceinline__ void merge_entries(const ModelDev &md, const int2 *qu
     }
 }
 
-// one entry per lane (count 0: none) joins the warp's queue, which is
-// worked off once it holds 32
-__device__ __forceinline__ void merge_push(const ModelDev &md, int2 *queue, int &nq, int2 e, const MergeLane &L,
-                                           MergeSum &sum) {
-    const int lane = threadIdx.x & 31;
-    const unsigned nz = __ballot_sync(0xffffffffu, e.y != 0);
-    if (e.y != 0) queue[nq + __popc(nz & ((1u << lane) - 1u))] = e;
-    nq += __popc(nz);
-    if (nq >= 32) {
-        __syncwarp();
-        merge_entries(md, queue, nq, L, sum);
-        __syncwarp();
-        nq = 0;
-    }
-}
-
-// Entries of row and column r other than M[r][r], part `part` of `parts`
-// (32 at a time in turn), against the lane's proposal.
+// Entries of row and column r other than M[r][r], part `part` of `parts`,
+// against the lane's proposal: 128 at a time (zeros dropped) join the warp's
+// queue, which is worked off from 32 on.  (One call of merge_entries: at
+// every place that found entries, its unrolled lookups filled the
+// instruction cache, 7.5 of 21 cycles between two issues.)
+template <bool SPARSE>
 __device__ __forceinline__ void merge_rows(const ModelDev &md, int r, int part, int parts, int2 *queue,
                                            const MergeLane &L, MergeSum &sum) {
-    const int lane = threadIdx.x & 31, B = md.B;
-    int nq = 0;
-    if (md.sparse) {
-        const uint32_t r0 = md.rp[r], rlen = md.re[r] - r0, c0 = md.cp[r], clen = md.ce[r] - c0;
-        for (uint32_t b0 = 32u * part; b0 < rlen; b0 += 32u * parts) {
-            const uint32_t i = b0 + lane;
-            const int t = i < rlen ? md.rc[r0 + i] : r;
-            merge_push(md, queue, nq, make_int2(t, t != r ? md.rv[r0 + i] : 0), L, sum);
-        }
-        for (uint32_t b0 = 32u * part; b0 < clen; b0 += 32u * parts) {
-            const uint32_t i = b0 + lane;
-            const int t = i < clen ? md.cr[c0 + i] : r;
-            merge_push(md, queue, nq, make_int2(t | INT32_MIN, t != r ? md.cv[c0 + i] : 0), L, sum);
-        }
+    const int lane = threadIdx.x & 31;
+    uint32_t r0 = 0, c0 = 0, rlen = 0, total = (uint32_t)md.B;
+    const int32_t *row = nullptr;
+    const uint32_t *pre = nullptr;
+    if (SPARSE) {
+        r0 = md.rp[r];
+        rlen = md.re[r] - r0;
+        c0 = md.cp[r] - rlen;  // the column follows the row
+        total = rlen + (md.ce[r] - md.cp[r]);
     } else {
-        // the column's counts as differences of its prefix in P (coalesced)
-        const int32_t *row = md.M + (size_t)r * B;
-        const uint32_t *pre = md.P + (size_t)r * 2 * B + B;
-        for (int b0 = 64 * part; b0 < B; b0 += 64 * parts) {
-            int v[2], c[2];
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int t = b0 + 32 * u + lane;
-                const bool ok = t < B && t != r;
-                v[u] = ok ? row[t] : 0;
-                c[u] = ok ? (int)(pre[t] - pre[t - 1]) : 0;  // pre[-1]: the end of the row's prefix, dout_r
-            }
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int t = b0 + 32 * u + lane;
-                merge_push(md, queue, nq, make_int2(t, v[u]), L, sum);
-                merge_push(md, queue, nq, make_int2(t | INT32_MIN, c[u]), L, sum);
-            }
-        }
+        // the column's counts as differences of its prefix in P (coalesced;
+        // pre[-1] is the end of the row's prefix, dout_r)
+        row = md.M + (size_t)r * md.B;
+        pre = md.P + (size_t)r * 2 * md.B + md.B;
     }
-    if (nq > 0) {
-        __syncwarp();
-        merge_entries(md, queue, nq, L, sum);
-        __syncwarp();
+    int nq = 0;
+    // the team's warps take chunks of 32 in turn, four (dense: two of the row
+    // and two of the column) in flight
+    const uint32_t next = 32u * parts, step = next * (SPARSE ? 4 : 2);
+    for (uint32_t b0 = 32u * part;; b0 += step) {
+        int2 e[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            int t, v = 0;
+            if (SPARSE) {
+                const uint32_t i = b0 + next * u + lane;
+                const bool col = i >= rlen;
+                t = i < total ? (col ? md.cr[c0 + i] : md.rc[r0 + i]) : r;
+                if (t != r) v = col ? md.cv[c0 + i] : md.rv[r0 + i];
+                t |= col ? INT32_MIN : 0;
+            } else {
+                t = (int)(b0 + next * (u >> 1) + lane);
+                if (t < md.B && t != r) v = (u & 1) ? (int)(pre[t] - pre[t - 1]) : row[t];
+                t |= (u & 1) ? INT32_MIN : 0;
+            }
+            e[u] = make_int2(t, v);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const unsigned nz = __ballot_sync(0xffffffffu, e[u].y != 0);
+            if (e[u].y != 0) queue[nq + __popc(nz & ((1u << lane) - 1u))] = e[u];
+            nq += __popc(nz);
+        }
+        const bool last = b0 >= total || total - b0 <= step;
+        if (nq >= 32 || last) {
+            __syncwarp();
+            merge_entries<SPARSE>(md, queue, nq, L, sum);
+            __syncwarp();
+            nq = 0;
+        }
+        if (last) break;
     }
 }
 
@@ -280,7 +271,7 @@ __device__ __forceinline__ void merge_fold(int nq, int G, MergeSum &sum) {
 // `part`).  team_sum(sum) adds the other warps' sums on lane q of warp 0 (a
 // no-op for one warp); every warp of the team calls it the same number of
 // times.  The result is valid in warp 0 (bs = -1 when x = 0).
-template <class TeamSum>
+template <bool SPARSE, class TeamSum>
 __device__ __forceinline__ void merge_best(const ModelDev &md, uint64_t seed, uint64_t round_id, int x, int r,
                                            int part, int parts, int2 *queue, TeamSum team_sum, int &bs_out,
                                            double &bd_out) {
@@ -294,7 +285,7 @@ __device__ __forceinline__ void merge_best(const ModelDev &md, uint64_t seed, ui
         MergeSum corner;
         if (lane < nq) {
             const U64x4 w = philox4x64_10(round_id, (uint64_t)r, (uint64_t)(i0 + lane), 0, seed, 1);
-            si = merge_propose(md, r, w.x, w.y);
+            si = merge_propose<SPARSE>(md, r, w.x, w.y);
             if (part == 0) merge_corner(md, r, si, corner);
         }
         MergeLane L;
@@ -303,12 +294,12 @@ __device__ __forceinline__ void merge_best(const ModelDev &md, uint64_t seed, ui
         L.on = L.g < L.G;
         L.s = __shfl_sync(0xffffffffu, si, lane - L.g * nq);
         L.off = L.cap = 0;
-        if (md.sparse) {
+        if (SPARSE) {
             L.off = md.hoff[L.s];
             L.cap = md.hoff[L.s + 1] - L.off;
         }
         MergeSum sum;
-        merge_rows(md, r, part, parts, queue, L, sum);
+        merge_rows<SPARSE>(md, r, part, parts, queue, L, sum);
         merge_fold(nq, L.G, sum);
         sum.fix += corner.fix;
         sum.fb += corner.fb;
