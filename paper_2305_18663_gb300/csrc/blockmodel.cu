@@ -14,6 +14,7 @@
 // holds, per block u, the inclusive prefix of row u followed by dout_u plus
 // the inclusive prefix of column u; the nodal and merge proposals search it.
 // DL (Eq. 2) is reduced in a fixed order so it is reproducible bit for bit.
+#include <algorithm>
 #include <cmath>
 
 #include "apply.cuh"
@@ -221,61 +222,67 @@ __device__ __forceinline__ void warp_cell_add(int32_t *cells, int key, int d) {
 }
 
 // One item of the accepted-move list, on a warp: a kMoveChunk-edge slice of
-// the concatenated (out, in) row of a moved vertex.  Lane j takes edges j,
-// j + 32, ... of the slice, all loads in flight together.  counts: the cells
-// are updated; nbo (not NULL): the block-labelled rows too (the twin of each
-// edge takes v's new label).
+// the concatenated (out, in) row of a moved vertex, kItemIn chunks of 32
+// edges in flight.  counts: the cells are updated; nbo (not NULL): the
+// block-labelled rows too (the twin of each edge takes v's new label).
+// Bound by the latency of its four dependent rounds of scattered loads: most
+// items are the 40-odd edges of one vertex, so what counts is how many warps
+// are in flight, not how many loads each has: 8 loads a lane at 48 registers
+// and 4 blocks an SM against 2 at 32 and 8, three sweeps of a 1M-vertex graph
+// took 3770 and 3670 us (4 loads, 6 blocks: 3677).
+constexpr int kItemIn = 2;
+
 __device__ __forceinline__ void delta_item(const GraphDev &g, int2 it, const int32_t *__restrict__ bnew,
                                            const int32_t *__restrict__ bold, int32_t *__restrict__ M, int B,
                                            bool counts, int32_t *__restrict__ nbo, int32_t *__restrict__ nbi) {
     const int lane = threadIdx.x & 31;
-    constexpr int kPer = kMoveChunk / 32;
     const int v = it.x;
-    const int r = bold[v], s = bnew[v];
-    if (r == s) return;
+    const int r = counts ? bold[v] : -1, s = bnew[v];
     const int o0 = g.op[v], kout = g.op[v + 1] - o0;
     const int i0 = g.ip[v], k = kout + (g.ip[v + 1] - i0);
-    const int lo = it.y * kMoveChunk;
-    int nb[kPer], t[kPer], u[kPer];
+    if (r == s) return;
+    const int hi = min(k, (it.y + 1) * kMoveChunk);
+    for (int lo = it.y * kMoveChunk; lo < hi; lo += 32 * kItemIn) {
+        int nb[kItemIn], tw[kItemIn], t[kItemIn], u[kItemIn];
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-        const int idx = lo + j * 32 + lane;
-        nb[j] = idx < k ? (idx < kout ? g.oc[o0 + idx] : g.ic[i0 + idx - kout]) : -1;
-    }
-    if (nbo) {
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
+        for (int j = 0; j < kItemIn; ++j) {
             const int idx = lo + j * 32 + lane;
-            if (nb[j] < 0) continue;
-            const int32_t x = s | (nb[j] == v ? kNbSelf : 0);
-            if (idx < kout) nbi[g.tw_oi[o0 + idx]] = x;  // v -> w: in w's in-row
-            else nbo[g.tw_io[i0 + idx - kout]] = x;     // w -> v: in w's out-row
+            const bool out = idx < kout;
+            const int at = out ? o0 + idx : i0 + idx - kout;
+            nb[j] = idx < hi ? (out ? g.oc : g.ic)[at] : -1;
+            tw[j] = nbo && idx < hi ? (out ? g.tw_oi : g.tw_io)[at] : 0;
         }
-    }
-    if (!counts) return;
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-        t[j] = nb[j] >= 0 ? bold[nb[j]] : 0;
-        u[j] = nb[j] >= 0 ? bnew[nb[j]] : 0;
-    }
+        for (int j = 0; j < kItemIn; ++j) {
+            t[j] = counts && nb[j] >= 0 ? bold[nb[j]] : 0;
+            u[j] = counts && nb[j] >= 0 ? bnew[nb[j]] : 0;
+        }
+        if (nbo) {
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-        const int idx = lo + j * 32 + lane;
-        int leave = -1, enter = -1;  // cells (B * B <= 2^26) the edge leaves and enters
-        if (nb[j] >= 0) {
-            if (idx < kout) {
-                // out-edge v -> w: leaves (r, t), enters (s, u)
-                leave = r * B + t[j];
-                enter = s * B + u[j];
-            } else if (u[j] == t[j]) {
-                // in-edge w -> v from a vertex that stayed (a moved
-                // source applies it through its own out-row)
-                leave = t[j] * B + r;
-                enter = t[j] * B + s;
+            for (int j = 0; j < kItemIn; ++j) {
+                // v -> w: in w's in-row; w -> v: in w's out-row
+                if (nb[j] >= 0) (lo + j * 32 + lane < kout ? nbi : nbo)[tw[j]] = s | (nb[j] == v ? kNbSelf : 0);
             }
         }
-        warp_cell_add(M, leave, -1);
-        warp_cell_add(M, enter, 1);
+        if (!counts) continue;
+#pragma unroll
+        for (int j = 0; j < kItemIn; ++j) {
+            int leave = -1, enter = -1;  // cells (B * B <= 2^26) the edge leaves and enters
+            if (nb[j] >= 0) {
+                if (lo + j * 32 + lane < kout) {
+                    // out-edge v -> w: leaves (r, t), enters (s, u)
+                    leave = r * B + t[j];
+                    enter = s * B + u[j];
+                } else if (u[j] == t[j]) {
+                    // in-edge w -> v from a vertex that stayed (a moved
+                    // source applies it through its own out-row)
+                    leave = t[j] * B + r;
+                    enter = t[j] * B + s;
+                }
+            }
+            warp_cell_add(M, leave, -1);
+            warp_cell_add(M, enter, 1);
+        }
     }
 }
 
@@ -284,7 +291,9 @@ __device__ __forceinline__ void delta_item(const GraphDev &g, int2 it, const int
 // so hubs are spread over many warps and no warp scans unmoved vertices.
 // The block-labelled rows (nbo not NULL) follow whatever the plan; the count
 // update runs only when the plan chose it.
-__global__ void __launch_bounds__(kThreads) k_delta_items(GraphDev g, const int2 *__restrict__ items,
+constexpr int kItemCtas = 8;  // per SM
+
+__global__ void __launch_bounds__(kThreads, kItemCtas) k_delta_items(GraphDev g, const int2 *__restrict__ items,
                                                           const DevCounters *__restrict__ c, int64_t cap,
                                                           const int32_t *__restrict__ bnew,
                                                           const int32_t *__restrict__ bold, int32_t *__restrict__ M,
@@ -320,38 +329,14 @@ __global__ void k_nb_self(const int32_t *__restrict__ self_in, int64_t n_self, i
 // the entries that name a moved vertex, after a pass: for every item of
 // the accepted-move list (a 256-edge slice of moved vertex v's rows), the
 // twin of each of v's edges takes v's new label
-__global__ void __launch_bounds__(kThreads) k_nb_items(GraphDev g, const int2 *__restrict__ items,
-                                                       const DevCounters *__restrict__ c, int64_t cap,
-                                                       const int32_t *__restrict__ b, int32_t *__restrict__ nbo,
-                                                       int32_t *__restrict__ nbi) {
-    const int lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(kThreads, kItemCtas) k_nb_items(GraphDev g, const int2 *__restrict__ items,
+                                                                  const DevCounters *__restrict__ c, int64_t cap,
+                                                                  const int32_t *__restrict__ b,
+                                                                  int32_t *__restrict__ nbo, int32_t *__restrict__ nbi) {
     const int64_t total = (int64_t)(c->items < (unsigned long long)cap ? c->items : (unsigned long long)cap);
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    constexpr int kPer = kMoveChunk / 32;
-    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += nw) {
-        const int2 it = items[w];
-        const int v = it.x;
-        const int s = b[v];
-        const int o0 = g.op[v], kout = g.op[v + 1] - o0;
-        const int i0 = g.ip[v], k = kout + (g.ip[v + 1] - i0);
-        const int lo = it.y * kMoveChunk;
-        int nb[kPer], tw[kPer];
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const int idx = lo + j * 32 + lane;
-            const bool ok = idx < k, out = idx < kout;
-            nb[j] = ok ? (out ? g.oc[o0 + idx] : g.ic[i0 + idx - kout]) : -1;
-            tw[j] = ok ? (out ? g.tw_oi[o0 + idx] : g.tw_io[i0 + idx - kout]) : 0;
-        }
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const int idx = lo + j * 32 + lane;
-            if (nb[j] < 0) continue;
-            const int32_t x = s | (nb[j] == v ? kNbSelf : 0);
-            if (idx < kout) nbi[tw[j]] = x;  // v -> w: in w's in-row
-            else nbo[tw[j]] = x;             // w -> v: in w's out-row
-        }
-    }
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += nw)
+        delta_item(g, items[w], b, nullptr, nullptr, 0, false, nbo, nbi);
 }
 
 // ---------------------------------------------------------------------------
@@ -555,7 +540,7 @@ int update_cells(sbp_model *m, int32_t *cells) {
         if (m->list_ok && m->items) {
             // the block-labelled rows follow in the same pass
             const bool nb = m->nb_ok && m->nbo;
-            k_delta_items<<<sms * 4, kThreads, 0, m->stream>>>(g->dev(), m->items, m->counters, m->cap_items, m->b,
+            k_delta_items<<<sms * kItemCtas, kThreads, 0, m->stream>>>(g->dev(), m->items, m->counters, m->cap_items, m->b,
                                                                m->bnew, cells, B, flag, nb ? m->nbo : nullptr,
                                                                nb ? m->nbi : nullptr);
             SBP_LAUNCHED();
@@ -588,9 +573,7 @@ int build_blockmodel(sbp_model *m, bool after_pass) {
             SBP_TRY(update_cells(m, m->M));
         else
             SBP_TRY(count_cells(m, m->M));
-        k_prefix_dense<<<grid_for((int64_t)B * 32, kThreads, 1 << 30), kThreads, 0, m->stream>>>(
-            m->M, B, m->P, m->dout, m->din, m->rcp, m->rcp32, m->dsum, m->Pc, (2 * B + 31) / 32);
-        SBP_LAUNCHED();
+        SBP_TRY(launch_prefix(m));
         np = grid_for(BB > B ? BB : B, kThreads * 4, 1024);  // (of kPartials)
         k_dl_partial<<<np, kThreads, 0, m->stream>>>(m->M, BB, m->dout, m->din, B, m->T, m->XT, parts);
         SBP_LAUNCHED();
@@ -713,7 +696,7 @@ int nb_rows_after_commit(sbp_model *m) {
         m->nb_ok = false;
         return SBP_OK;
     }
-    k_nb_items<<<num_sms() * 4, kThreads, 0, m->stream>>>(m->g->dev(), m->items, m->counters, m->cap_items, m->b,
+    k_nb_items<<<num_sms() * kItemCtas, kThreads, 0, m->stream>>>(m->g->dev(), m->items, m->counters, m->cap_items, m->b,
                                                           m->nbo, m->nbi);
     SBP_LAUNCHED();
     return SBP_OK;
