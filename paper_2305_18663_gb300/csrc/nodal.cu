@@ -875,6 +875,13 @@ __global__ void __launch_bounds__(kBigThreads) k_eval_cta(DecideArgs a, int bin,
 #ifndef SBP_BATCH0_MIN_BLOCKS
 #define SBP_BATCH0_MIN_BLOCKS 4
 #endif
+// CTAs per SM (register budgets) of the batch kernels: the exact form, whose
+// 128-bit sums spill at the FP32 form's budgets, does better with one fewer
+// (three sweeps of 200k vertices: 1342 us at 4 and 3, 1294 at 3 and 3, 1172 at
+// 3 and 2)
+constexpr int batch_min_blocks(int mode, bool dl32) {
+    return mode == 0 ? (dl32 ? SBP_BATCH0_MIN_BLOCKS : 3) : (dl32 ? SBP_DECIDE_MIN_BLOCKS : 2);
+}
 constexpr int kBatchEdges = 32 * kSmallDeg;     // edge ends per sub-batch (33..128)
 constexpr int kBatchEdges0 = SBP_BATCH0_EDGES;  // ... for rows of at most 32
 constexpr int kDirectMaxB = 2048;  // direct-mapped per-warp counts up to this B
@@ -1205,8 +1212,7 @@ __device__ __forceinline__ void batch_movers(const DecideArgs &a, BatchWarp<MODE
 // in lane p % 32, slot p / 32) and evaluate them 32 at a time, so that the
 // proposals' load chains overlap other warps' evaluation.
 template <int MODE, bool DL32, bool FUSED>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, MODE == 0 ? SBP_BATCH0_MIN_BLOCKS : SBP_DECIDE_MIN_BLOCKS)
-    k_eval_batch(DecideArgs a, int bin, int warp_bytes) {
+__global__ void __launch_bounds__(kWarpsPerCta * 32, batch_min_blocks(MODE, DL32)) k_eval_batch(DecideArgs a, int bin, int warp_bytes) {
     extern __shared__ __align__(16) unsigned char bsm[];
     using BW = BatchWarp<MODE>;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
@@ -1698,7 +1704,7 @@ int launch_groups(sbp_model *m, const DecideArgs &a, int sms, const cudaStream_t
         const int wb = (int)((sizeof(BatchWarp<0>) + 15) / 16 * 16);
         const size_t smem = (size_t)wb * kWarpsPerCta;
         SBP_TRY(ensure_dyn_smem((const void *)k_eval_batch<0, DL32, FUSED>, smem));
-        k_eval_batch<0, DL32, FUSED><<<sms * SBP_BATCH0_MIN_BLOCKS, kWarpsPerCta * 32, smem, st[0]>>>(a, 0, wb);
+        k_eval_batch<0, DL32, FUSED><<<sms * batch_min_blocks(0, DL32), kWarpsPerCta * 32, smem, st[0]>>>(a, 0, wb);
         SBP_LAUNCHED();
     }
     // movers with 33 <= k <= 128: batches with direct-mapped counts while B is
@@ -1709,7 +1715,7 @@ int launch_groups(sbp_model *m, const DecideArgs &a, int sms, const cudaStream_t
             const int nwarps = wb <= 10 * 1024 ? kWarpsPerCta : kWarpsPerCta / 2;
             const size_t smem = (size_t)wb * nwarps;
             SBP_TRY(ensure_dyn_smem((const void *)k_eval_batch<1, DL32, FUSED>, smem));
-            k_eval_batch<1, DL32, FUSED><<<sms * SBP_DECIDE_MIN_BLOCKS, nwarps * 32, smem, st[1]>>>(a, 1, wb);
+            k_eval_batch<1, DL32, FUSED><<<sms * batch_min_blocks(1, DL32), nwarps * 32, smem, st[1]>>>(a, 1, wb);
             SBP_LAUNCHED();
         } else {
             SBP_TRY(tables(1, 8, st[1]));
