@@ -197,6 +197,7 @@ struct sbp_model {
     int32_t *M = nullptr;
     uint32_t *P = nullptr;
     uint32_t *Pc = nullptr;
+    uint32_t *colsum = nullptr;  // column sums by chunk of rows (dense, many blocks)
     int32_t *dout = nullptr, *din = nullptr;
     double *rcp = nullptr;
     float *rcp32 = nullptr;
