@@ -7,7 +7,8 @@
 // with a host round trip.  Here one persistent launch takes a table of jobs
 // (one phase of one graph each, every graph in its own dense model); a CTA
 // pulls a job from a device queue, runs the whole phase for it and pulls
-// the next, largest jobs first.  A job:
+// the next, largest jobs first; while few searches are left, each gets a
+// cluster of CTAs instead.  A job:
 //   0. (optional) loads the phase's start state, a bracket state the model
 //      no longer holds, and rebuilds the counts from it;
 //   1. (optional) the merge phase: per round, every block's best merge
@@ -52,8 +53,64 @@ namespace sbp {
 namespace {
 
 constexpr int kBatchThreads = 256;
-constexpr int kBatchWarps = kBatchThreads / 32;
 constexpr size_t kBatchSmemCap = 96 * 1024;  // dynamic shared memory of a CTA (two per SM)
+// A search on the CTAs of a cluster, when there are few searches (see
+// batch_cluster): one CTA an SM, with twice the warps
+constexpr int kClusterThreads = 512;
+constexpr size_t kClusterSmemCap = 180 * 1024;
+
+// Threads that run a search: one CTA, or the CTAs of a cluster.  In a
+// cluster every CTA keeps the search's state (the job, the record, the
+// bracket decisions) in its own shared memory and derives it from the same
+// data, the merge application included; the loops over vertices, edges,
+// blocks and cells are split over all threads, and what one CTA wrote to
+// global memory is read by others only after sync().
+template <bool CLUSTER>
+struct Squad {
+    static constexpr int T = CLUSTER ? kClusterThreads : kBatchThreads;
+    static constexpr int W = T / 32;  // warps of a CTA
+    int rank, tid, nt, wid, nw;       // this CTA; this thread and warp among the squad's
+    __int128 *xch;                    // two sets of a cluster's sums, in turn
+    int turn;
+    __device__ __forceinline__ Squad(__int128 *x) : xch(x), turn(0) {
+        rank = CLUSTER ? cluster_rank() : 0;
+        const int size = CLUSTER ? cluster_size() : 1;
+        tid = rank * T + threadIdx.x;
+        nt = size * T;
+        wid = tid >> 5;
+        nw = nt >> 5;
+    }
+    __device__ __forceinline__ void sync() const {
+        if constexpr (CLUSTER) cluster_sync();
+        else __syncthreads();
+    }
+    // the squad's sum of one int128 per thread (every thread gets it; a
+    // barrier of the squad)
+    __device__ __int128 sum(__int128 v, __int128 *sh) {
+        v = warp_sum_128(v);
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+        __syncthreads();
+        __int128 s = 0;
+        for (int q = 0; q < W; ++q) s += sh[q];
+        if constexpr (CLUSTER) {
+            // a set is written again only after the other set's barrier,
+            // which every CTA reaches after it has read the first
+            __int128 *x = xch + 8 * turn;
+            turn ^= 1;
+            if (threadIdx.x == 0) x[rank] = s;
+            cluster_sync();
+            s = 0;
+            for (int q = 0; q < nt / T; ++q) {
+                const unsigned long long *w = reinterpret_cast<const unsigned long long *>(x + q);
+                s += (__int128)(((unsigned __int128)__ldcg(w + 1) << 64) | __ldcg(w));
+            }
+        } else {
+            __syncthreads();
+        }
+        return s;
+    }
+};
 
 // the blockmodel arrays the apply step writes (the decision pass sees them
 // read-only through DecideArgs)
@@ -173,68 +230,59 @@ __device__ void apply_rows(const GraphDev &g, const int32_t *bold, const int32_t
     }
 }
 
-// the CTA's sum of one int128 per thread (every thread gets it)
-__device__ __int128 cta_sum_128(__int128 v, __int128 *sh) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    v = warp_sum_128(v);
-    __syncthreads();
-    if (lane == 0) sh[w] = v;
-    __syncthreads();
-    __int128 s = 0;
-    for (int q = 0; q < kBatchWarps; ++q) s += sh[q];
-    __syncthreads();
-    return s;
-}
-
-// The dense model of B blocks from labels b, CTA-wide (the per-graph
-// rebuild's counts, prefix rows, degrees and reciprocals): M counted from the
-// edge list, then the sums C = sum T[M] and D = sum T[dout] + T[din]
-// (L = C - D exactly).  Every thread gets C and D.
-__device__ void cta_rebuild(const GraphDev &g, const int32_t *b, const ModelOut &w, int B, int pstep,
-                            const __int128 *__restrict__ T, __int128 *red, __int128 &C, __int128 &D) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+// The dense model of B blocks from labels b (the per-graph rebuild's counts,
+// prefix rows, degrees and reciprocals): M counted from the edge list, then
+// the sums C = sum T[M] and D = sum T[dout] + T[din] (L = C - D exactly).
+// Every thread of the squad gets C and D.
+template <class Sq>
+__device__ void squad_rebuild(Sq &sq, const GraphDev &g, const int32_t *b, const ModelOut &w, int B, int pstep,
+                              const __int128 *__restrict__ T, __int128 *red, __int128 &C, __int128 &D) {
+    const int lane = threadIdx.x & 31;
     const int BB = B * B;
-    for (int i = tid; i < BB; i += kBatchThreads) w.M[i] = 0;
-    __syncthreads();
-    for (int64_t e = tid; e < g.m; e += kBatchThreads) atomicAdd(&w.M[b[g.esrc[e]] * B + b[g.oc[e]]], 1);
-    __syncthreads();
+    for (int i = sq.tid; i < BB; i += sq.nt) w.M[i] = 0;
+    sq.sync();
+    for (int64_t e = sq.tid; e < g.m; e += sq.nt) atomicAdd(&w.M[b[g.esrc[e]] * B + b[g.oc[e]]], 1);
+    sq.sync();
     __int128 dd = 0, c = 0;
-    for (int u = wid; u < B; u += kBatchWarps) {
+    for (int u = sq.wid; u < B; u += sq.nw) {
         prefix_block(w.M, B, u, w.P, w.dout, w.din, w.rcp, w.rcp32, w.dsum, w.Pc, pstep);
         if (lane == 0) {
             dd += T[w.dout[u]];
             dd += T[w.din[u]];
         }
     }
-    for (int i = tid; i < BB; i += kBatchThreads) c += T[w.M[i]];
-    D = cta_sum_128(dd, red);
-    C = cta_sum_128(c, red);
+    for (int i = sq.tid; i < BB; i += sq.nt) c += T[w.M[i]];
+    D = sq.sum(dd, red);
+    C = sq.sum(c, red);
 }
 
 // b[v] = bnew[v] = map[b[v]] for every vertex
-__device__ void cta_relabel(int32_t *b, int32_t *bnew, int n, const int *map) {
-    for (int v = threadIdx.x; v < n; v += kBatchThreads) {
+template <class Sq>
+__device__ void squad_relabel(Sq &sq, int32_t *b, int32_t *bnew, int n, const int *map) {
+    for (int v = sq.tid; v < n; v += sq.nt) {
         const int x = map[b[v]];
         b[v] = x;
         bnew[v] = x;
     }
-    __syncthreads();
+    sq.sync();
 }
 
 // G: lanes per mover in the evaluation (32 / G movers per warp at a time);
 // group_words: shared-memory words of one group (counts, then the list);
 // blk_cap: a power of two >= every job's lim_from (the merge rounds' and the
 // compaction's shared arrays)
-template <bool DL32, int G>
-__global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJob *__restrict__ jobs, int njobs,
-                                                                  unsigned *__restrict__ queue, int group_words,
-                                                                  int blk_cap) {
+template <bool DL32, int G, bool CLUSTER>
+__global__ void __launch_bounds__(Squad<CLUSTER>::T, CLUSTER ? 1 : 2)
+    k_batch_search(const BatchJob *__restrict__ jobs, int njobs, unsigned *__restrict__ queue, int group_words,
+                   int blk_cap, __int128 *__restrict__ xch) {
+    using Sq = Squad<CLUSTER>;
+    constexpr int kThreads = Sq::T, kWarps = Sq::W;
     extern __shared__ __align__(16) unsigned char bsm[];
     __shared__ DecideArgs sa;
     __shared__ ModelOut sw;
     __shared__ SearchRec sr;
-    __shared__ __int128 red[kBatchWarps];
-    __shared__ int2 mqueue[kBatchWarps][kMergeQueue];
+    __shared__ __int128 red[kWarps];
+    __shared__ int2 mqueue[kWarps][kMergeQueue];
     __shared__ TeamShared tsh;
     __shared__ unsigned s_job, s_nmov;
     __shared__ int s_stop, s_left, s_rounds, s_done, s_Bn, s_go, s_start, s_target, s_reload, s_slot;
@@ -254,11 +302,16 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
     mw.mark = mw.x1 + blk_cap;
     int *smap = mw.mark + blk_cap;
     int *par = mw.a0;
-    for (;;) {
-        if (tid == 0) s_job = atomicAdd(queue, 1u);
-        __syncthreads();
-        const unsigned j = s_job;
+    // a cluster takes the one search it was launched for, a CTA the next of
+    // the queue
+    for (bool first = true; !CLUSTER || first; first = false) {
+        if (!CLUSTER) {
+            if (tid == 0) s_job = atomicAdd(queue, 1u);
+            __syncthreads();
+        }
+        const unsigned j = CLUSTER ? blockIdx.x / cluster_size() : s_job;
         if (j >= (unsigned)njobs) return;
+        Sq sq(xch + 16 * (size_t)j);
         if (tid == 0) {
             sa = jobs[j].a;
             sw = jobs[j].w;
@@ -272,6 +325,9 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
         const ModelDev &md = sa.md;
         const int n = g.n;
         int B = md.B;
+        const int v_per = (n + sq.nt / kThreads - 1) / (sq.nt / kThreads);
+        const int v_lo = min(n, sq.rank * v_per), v_hi = min(n, v_lo + v_per);
+        Mover *movers = sa.movers + v_lo;
         bool started = sr.started != 0;
         for (;;) {
             __int128 C = 0, D = 0;
@@ -298,7 +354,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                 const SearchState from = sr.s[s_start];
                 if (s_reload) {
                     const int32_t *src = J.slots + (size_t)from.slot * n;
-                    for (int v = tid; v < n; v += kBatchThreads) {
+                    for (int v = sq.tid; v < n; v += sq.nt) {
                         const int x = src[v];
                         sw.b[v] = x;
                         md.bnew[v] = x;
@@ -310,7 +366,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                         ++sr.starts;
                     }
                     __syncthreads();
-                    cta_rebuild(g, sw.b, sw, B, (2 * B + 31) / 32, md.T, red, C, D);
+                    squad_rebuild(sq, g, sw.b, sw, B, (2 * B + 31) / 32, md.T, red, C, D);
                     have_sums = true;
                 }
                 // 1. merge rounds until from.B - target blocks are gone (or a
@@ -324,7 +380,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                 __syncthreads();
                 while (s_left > 0 && B >= 2) {
                     const uint64_t rid = sr.round_id + (uint64_t)s_rounds;
-                    for (int r = wid; r < B; r += kBatchWarps) {
+                    for (int r = sq.wid; r < B; r += sq.nw) {
                         int bs;
                         double bd;
                         merge_best<false>(md, sa.seed, rid, J.merge_x, r, 0, 1, mqueue[wid], [](MergeSum &) {}, bs, bd);
@@ -333,7 +389,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                             J.best_d[r] = bd;
                         }
                     }
-                    __syncthreads();
+                    sq.sync();
                     CtaTeam team{tsh};
                     int Bn;
                     const int done = merge_apply(team, mw, B, J.best_s, J.best_d, s_left, smap, Bn);
@@ -346,9 +402,9 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                         sa.md.pstep = (2 * Bn + 31) / 32;
                     }
                     __syncthreads();
-                    cta_relabel(sw.b, md.bnew, n, smap);
+                    squad_relabel(sq, sw.b, md.bnew, n, smap);
                     B = s_Bn;
-                    cta_rebuild(g, sw.b, sw, B, md.pstep, md.T, red, C, D);
+                    squad_rebuild(sq, g, sw.b, sw, B, md.pstep, md.T, red, C, D);
                     have_sums = true;
                     if (s_done == 0) break;
                 }
@@ -361,10 +417,10 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
             if (!have_sums) {
                 // sum over the cells of T[M] and the degree terms at the phase start (exact)
                 __int128 c = 0, dd = 0;
-                for (int i = tid; i < B * B; i += kBatchThreads) c += md.T[md.M[i]];
-                for (int u = tid; u < B; u += kBatchThreads) dd += md.T[md.dout[u]] + md.T[md.din[u]];
-                C = cta_sum_128(c, red);
-                D = cta_sum_128(dd, red);
+                for (int i = sq.tid; i < B * B; i += sq.nt) c += md.T[md.M[i]];
+                for (int u = sq.tid; u < B; u += sq.nt) dd += md.T[md.dout[u]] + md.T[md.din[u]];
+                C = sq.sum(c, red);
+                D = sq.sum(dd, red);
             }
             int *list = reinterpret_cast<int *>(cnt + B);
             for (int i = gl; i < B; i += G) cnt[i] = 0u;
@@ -380,12 +436,12 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                 const uint64_t sweep_id = sweep0 + (uint64_t)(k - 1);
                 if (tid == 0) s_nmov = 0;
                 __syncthreads();
-                // 1. proposals
-                for (int base = 0; base < n; base += kBatchThreads) {
+                // 1. proposals (a CTA's vertices, whose movers it evaluates too)
+                for (int base = v_lo; base < v_hi; base += kThreads) {
                     const int v = base + tid;
                     bool mv = false;
                     Proposal p;
-                    if (v < n) {
+                    if (v < v_hi) {
                         p = propose_vertex(g, md, sa.seed, sweep_id, v);
                         mv = p.k > 0 && p.s != p.r;
                     }
@@ -400,7 +456,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                         m.v = v;
                         m.s = p.s;
                         m.w2 = p.w2;
-                        sa.movers[pos0 + __popc(msk & ((1u << lane) - 1u))] = m;
+                        movers[pos0 + __popc(msk & ((1u << lane) - 1u))] = m;
                     }
                 }
                 __syncthreads();
@@ -408,8 +464,8 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                 const int nmov = (int)s_nmov;
                 Counts cts;
                 __syncwarp();
-                for (int q = wid * V + gid; q < nmov; q += kBatchWarps * V) {
-                    const Mover mv = sa.movers[q];
+                for (int q = wid * V + gid; q < nmov; q += kWarps * V) {
+                    const Mover mv = movers[q];
                     const int v = mv.v;
                     const int o0 = g.op[v], kout = g.op[v + 1] - o0;
                     const int i0 = g.ip[v], kin = g.ip[v + 1] - i0;
@@ -451,10 +507,10 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                     for (int e = gl; e < nl; e += G) cnt[list[e]] = 0u;
                     __syncwarp(gm);
                 }
-                __syncthreads();
+                sq.sync();
                 // 3. apply: warp per 32 vertex ids, rows of the moved ones
                 __int128 dc = 0;
-                for (int base = wid * 32; base < n; base += kBatchThreads) {
+                for (int base = sq.wid * 32; base < n; base += sq.nt) {
                     const int vv = base + lane;
                     const bool moved = vv < n && md.bnew[vv] != md.b[vv];
                     unsigned mm = __ballot_sync(0xffffffffu, moved);
@@ -464,19 +520,19 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                         apply_rows(g, md.b, md.bnew, sw.M, B, md.T, base + qq, dc);
                     }
                 }
-                C += cta_sum_128(dc, red);  // includes the barrier before the label copy
-                for (int v = tid; v < n; v += kBatchThreads) sw.b[v] = md.bnew[v];
-                __syncthreads();
+                C += sq.sum(dc, red);  // includes the barrier before the label copy
+                for (int v = sq.tid; v < n; v += sq.nt) sw.b[v] = md.bnew[v];
+                sq.sync();
                 // 4. prefix rows, degrees, DL, the stopping rule
                 __int128 dd = 0;
-                for (int u = wid; u < B; u += kBatchWarps) {
+                for (int u = sq.wid; u < B; u += sq.nw) {
                     prefix_block(sw.M, B, u, sw.P, sw.dout, sw.din, sw.rcp, sw.rcp32, sw.dsum, sw.Pc, md.pstep);
                     if (lane == 0) {
                         dd += md.T[sw.dout[u]];
                         dd += md.T[sw.din[u]];
                     }
                 }
-                const __int128 Dk = cta_sum_128(dd, red);
+                const __int128 Dk = sq.sum(dd, red);
                 if (tid == 0) {
                     const double dlk = dl_eq2(g.m, g.n, B, fix_to_double(C - Dk));
                     J.hist[k] = dlk;
@@ -493,10 +549,10 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
             // 3. compaction: blocks left empty by the sweeps are dropped and
             // the others renumbered in order (the counts rebuilt when any was
             // empty)
-            for (int i = tid; i < B; i += kBatchThreads) par[i] = 0;
+            for (int i = tid; i < B; i += kThreads) par[i] = 0;
             __syncthreads();
-            for (int v = tid; v < n; v += kBatchThreads) atomicAdd(&par[sw.b[v]], 1);
-            __syncthreads();
+            for (int v = tid; v < n; v += kThreads) atomicAdd(&par[sw.b[v]], 1);
+            sq.sync();  // (every CTA counts all labels, before any of them changes)
             CtaTeam team{tsh};
             const int left = compact_map(team, B, par, smap);
             if (tid == 0) {
@@ -508,14 +564,14 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
             __syncthreads();
             double dlc = prev;
             if (s_Bn != B) {
-                cta_relabel(sw.b, md.bnew, n, smap);
+                squad_relabel(sq, sw.b, md.bnew, n, smap);
                 B = s_Bn;
-                cta_rebuild(g, sw.b, sw, B, md.pstep, md.T, red, C, D);
+                squad_rebuild(sq, g, sw.b, sw, B, md.pstep, md.T, red, C, D);
                 dlc = dl_eq2(g.m, g.n, B, fix_to_double(C - D));
             }
             // 4. the phase's state joins the bracket; its labels go to the free slot
             int32_t *dst = J.slots + (size_t)s_slot * n;
-            for (int v = tid; v < n; v += kBatchThreads) dst[v] = sw.b[v];
+            for (int v = sq.tid; v < n; v += sq.nt) dst[v] = sw.b[v];
             if (tid == 0) {
                 J.dl[0] = dlc;
                 sr.sweep_id += (uint64_t)k;
@@ -529,14 +585,14 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_search(const BatchJo
                 search_insert(sr, x);
                 ++sr.phases;
             }
-            __syncthreads();
+            sq.sync();
         }
         // the search goes back (ended, or its next phase is not one for this
         // kernel): the labels, then the record, then its ok word, each
         // visible to the host before the next
         __threadfence_system();
-        __syncthreads();
-        if (tid == 0) {
+        sq.sync();
+        if (sq.tid == 0) {
             sr.B_model = B;
             sr.started = 0;
             const int ok = 2 * B + 4 > group_words ? -1 : 1;
@@ -581,7 +637,20 @@ bool batch_phase_eligible(const sbp_model *m, int32_t B_from, int32_t target, in
            target <= kBatchMaxB && batch_graph_ok(m, max_n);
 }
 
-int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, const BatchTuning &tune,
+// CTAs (one an SM) for each search of a launch while `active` searches are
+// unfinished and may use `sms` of the SMs: 8, 4 or 2; 1: the queue of
+// one-CTA searches, which a GPU's worth of searches fills.  A search of 5000
+// vertices is a chain of a few hundred sweeps that one CTA of eight warps
+// runs alone on its SM: 32 graphs of 500 to 5000 vertices took 327 ms so, and
+// take 117 ms on clusters (4 CTAs each, 8 once half of them are done); 1200
+// of them take 1.7 s either way.
+int batch_cluster(int64_t active, int sms) {
+    for (int c = 8; c > 1; c /= 2)
+        if (active * c <= sms) return c;
+    return 1;
+}
+
+int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, const BatchTuning &tune, int cluster,
                   cudaStream_t st) {
     const int nj = (int)specs.size();
     if (nj == 0) return SBP_OK;
@@ -599,7 +668,8 @@ int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, cons
     while (blk_cap < blk) blk_cap <<= 1;
     // device scratch: jobs, hist rows, queue
     const size_t hist_stride = (size_t)p.max_sweeps + 1;
-    const size_t bytes = (size_t)nj * sizeof(BatchJob) + (size_t)nj * hist_stride * 8 + 16;
+    const size_t xch_at = ((size_t)nj * sizeof(BatchJob) + (size_t)nj * hist_stride * 8 + 16 + 255) / 256 * 256;
+    const size_t bytes = xch_at + (size_t)nj * 16 * sizeof(__int128);
     unsigned char *buf = nullptr;
     SBP_CUDA(cudaMallocAsync(&buf, bytes, st));
     BatchJob *d_jobs = reinterpret_cast<BatchJob *>(buf);
@@ -670,24 +740,31 @@ int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, cons
     // per mover group: B counts and a list of up to B blocks; as many movers
     // per warp as asked for while the CTA's share of shared memory holds them
     const int group_words = 2 * max_B + 4;
-    int V = tune.movers_per_warp == 4 ? 4 : tune.movers_per_warp == 2 ? 2 : 1;
-    while (V > 1 && (size_t)kBatchWarps * V * group_words * 4 > kBatchSmemCap) V /= 2;
+    const bool cl = cluster > 1;
+    const int warps = (cl ? kClusterThreads : kBatchThreads) / 32;
+    int V = tune.movers_per_warp == 4 ? (cl ? 2 : 4) : tune.movers_per_warp == 2 ? 2 : 1;
+    while (V > 1 && (size_t)warps * V * group_words * 4 > (cl ? kClusterSmemCap : kBatchSmemCap)) V /= 2;
     // the merge rounds' and the compaction's arrays share that memory
-    const size_t smem = std::max((size_t)kBatchWarps * V * group_words * 4, (size_t)blk_cap * (kMergeApplyBytes + 4));
+    const size_t smem = std::max((size_t)warps * V * group_words * 4, (size_t)blk_cap * (kMergeApplyBytes + 4));
     const int per_sm = tune.ctas_per_sm > 0 ? tune.ctas_per_sm : 2;
     const int grid = std::min(nj, sm_count_b() * per_sm);
+    __int128 *xch = reinterpret_cast<__int128 *>(buf + xch_at);
     auto launch = [&](auto kern) -> int {
         SBP_TRY(ensure_dyn_smem((const void *)kern, smem));
-        kern<<<grid, kBatchThreads, smem, st>>>(d_jobs, nj, d_queue, group_words, blk_cap);
-        SBP_LAUNCHED();
-        return SBP_OK;
+        return launch_cluster(kern, cl ? cluster : 1, warps * 32, smem, st, cl ? nj : grid, (const BatchJob *)d_jobs, nj,
+                              d_queue, group_words, blk_cap, xch);
     };
-    if (p.dl_fp32) {
-        SBP_TRY(V == 4 ? launch(k_batch_search<true, 8>) : V == 2 ? launch(k_batch_search<true, 16>)
-                                                          : launch(k_batch_search<true, 32>));
+    if (cl) {
+        if (p.dl_fp32)
+            SBP_TRY(V == 2 ? launch(k_batch_search<true, 16, true>) : launch(k_batch_search<true, 32, true>));
+        else
+            SBP_TRY(V == 2 ? launch(k_batch_search<false, 16, true>) : launch(k_batch_search<false, 32, true>));
+    } else if (p.dl_fp32) {
+        SBP_TRY(V == 4 ? launch(k_batch_search<true, 8, false>)
+                       : V == 2 ? launch(k_batch_search<true, 16, false>) : launch(k_batch_search<true, 32, false>));
     } else {
-        SBP_TRY(V == 4 ? launch(k_batch_search<false, 8>) : V == 2 ? launch(k_batch_search<false, 16>)
-                                                           : launch(k_batch_search<false, 32>));
+        SBP_TRY(V == 4 ? launch(k_batch_search<false, 8, false>)
+                       : V == 2 ? launch(k_batch_search<false, 16, false>) : launch(k_batch_search<false, 32, false>));
     }
     SBP_CUDA(cudaFreeAsync(buf, st));
     return SBP_OK;

@@ -61,8 +61,10 @@ bool batch_phase_eligible(const sbp_model *m, int32_t B_from, int32_t target, in
 // positions written).  When the stream reaches the end of the launch each
 // model is in the state the per-graph kernels would leave and each record
 // and its slots hold the search as the kernel left it.  The launch's
-// scratch is freed in stream order.
-int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, const BatchTuning &tune,
+// scratch is freed in stream order.  cluster: CTAs per search, from
+// batch_cluster.
+int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, const BatchTuning &tune, int cluster,
                   cudaStream_t st);
+int batch_cluster(int64_t active, int sms);
 
 }  // namespace sbp

@@ -841,7 +841,7 @@ int commit_small(sbp_model *m, SweepReadback *host) {
     a.parts = reinterpret_cast<DlPartial *>(m->partials);
     a.status = m->status;
     a.host = host;
-    return launch_cluster(k_commit_small, kCommitCluster, kCommitThreads, 0, m->stream, a);
+    return launch_cluster(k_commit_small, kCommitCluster, kCommitThreads, 0, m->stream, 1, a);
 }
 
 // block-labelled rows from m->b (allocated on first use).  Without the

@@ -612,11 +612,12 @@ __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// one launch of one cluster of `size` blocks (1: a plain block)
+// one launch of `count` clusters of `size` blocks (size 1: plain blocks)
 template <class... Args>
-int launch_cluster(void (*kern)(Args...), int size, int threads, size_t smem, cudaStream_t st, Args... args) {
+int launch_cluster(void (*kern)(Args...), int size, int threads, size_t smem, cudaStream_t st, int count,
+                   Args... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)size);
+    cfg.gridDim = dim3((unsigned)(size * count));
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;

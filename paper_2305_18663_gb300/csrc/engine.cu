@@ -465,6 +465,9 @@ int Engine::loop() {
             inflight.push_back(slot);
             ended.clear();
             for (int64_t idx : L.take) ended.push_back(items[(size_t)idx].get());
+            // a batch call's searches may take most of the chip, the server
+            // leaves half of it to its large requests' kernels
+            const int cluster = batch_cluster(running + (int64_t)(items.size() - next_admit), oldest_first ? 76 : 136);
             lk.unlock();
             // each graph's search goes to its mapped record and label slots
             std::vector<BatchSpec> specs(L.take.size());
@@ -479,7 +482,7 @@ int Engine::loop() {
                 sp.started = it.job == 1 ? 1 : 0;
             }
             L.t0 = now_s();
-            int r = batch_enqueue(specs, prm, opt.tune, L.st);
+            int r = batch_enqueue(specs, prm, opt.tune, cluster, L.st);
             if (r == SBP_OK && cudaEventRecord(L.ev, L.st) != cudaSuccess) r = cuda_fail(cudaGetLastError(), "cudaEventRecord");
             std::string msg;
             if (r != SBP_OK) {

@@ -185,7 +185,7 @@ int apply_merge_round(sbp_model *m, int32_t want, int32_t *done, int32_t *B_new)
     const MergeWork x = merge_work(m);
     const bool cl = m->B > kOneCtaB;
     SBP_TRY(launch_cluster(cl ? k_merge_apply<true> : k_merge_apply<false>, cl ? kApplyCluster : 1, kApplyThreads, 0,
-                           m->stream, x.w, x.words, (int)m->B,
+                           m->stream, 1, x.w, x.words, (int)m->B,
                         (const int32_t *)m->best_s, (const double *)m->best_d, (int)want, m->map, x.res));
     int32_t *h = static_cast<int32_t *>(m->pinned);
     SBP_CUDA(cudaMemcpyAsync(h, x.res, 8, cudaMemcpyDeviceToHost, m->stream));
@@ -202,7 +202,7 @@ int compact_blocks(sbp_model *m, int32_t *B_new) {
     const MergeWork x = merge_work(m);
     const bool cl = m->B > kOneCtaB;
     SBP_TRY(launch_cluster(cl ? k_compact_map<true> : k_compact_map<false>, cl ? kApplyCluster : 1, kApplyThreads, 0,
-                           m->stream, x.words, (int)m->B,
+                           m->stream, 1, x.words, (int)m->B,
                         (const int32_t *)m->vcount, m->map, x.res));
     int32_t *h = static_cast<int32_t *>(m->pinned);
     SBP_CUDA(cudaMemcpyAsync(h, x.res + 1, 4, cudaMemcpyDeviceToHost, m->stream));

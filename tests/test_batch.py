@@ -125,3 +125,20 @@ def test_autotuner_returns_valid_options_with_unchanged_results():
     for pg, (b, B, dl, ns, ta, td) in zip(pgs, out):
         pb, pB, pdl, pns = _plain(pg, params)
         assert B == pB and dl == pdl and ns == pns and np.array_equal(b, pb)
+
+
+@pytest.mark.parametrize("count", [1, 20, 40, 80])
+def test_searches_on_clusters_and_single_ctas_equal_plain_runs(count):
+    # few searches run on clusters of 8, 4 and 2 CTAs, many on one CTA each;
+    # a run passes from one to the other as its searches end
+    pgs = []
+    for i in range(count):
+        n = 150 + 37 * i % 500
+        g = dcsbm(n, 9 * n, 5, 2.5, 1, 60, 4.0, seed=1000 + i)
+        pgs.append(P.Graph(g.n, g.src, g.dst))
+    for prm in (P.Params.default(seed=3), P.Params.default(seed=3, dl_fp32=0)):
+        for opts in ({}, dict(movers_per_warp=4, max_B=1024)):
+            out = P.partition_batch(pgs, prm, P.BatchOptions.default(**opts))
+            for pg, (b, B, dl, ns, _, _) in zip(pgs, out):
+                pb, pB, pdl, pns = _plain(pg, prm)
+                assert (B, ns, dl) == (pB, pns, pdl) and np.array_equal(b, pb)
