@@ -42,7 +42,7 @@ void *pinned_get() {
         return p;
     }
     void *p = nullptr;
-    if (cudaMallocHost(&p, 4096) != cudaSuccess) {
+    if (cudaMallocHost(&p, kPinnedBytes) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
@@ -82,9 +82,12 @@ int cuda_fail(cudaError_t e, const char *what) {
 }
 
 int check_status(const sbp_model *m) {
-    int32_t st = 0;
-    SBP_CUDA(cudaMemcpyAsync(&st, m->status, 4, cudaMemcpyDeviceToHost, m->stream));
+    // (read back to pinned memory, its last word: a copy to pageable memory
+    // is staged and waited for by itself)
+    volatile int32_t *h = static_cast<int32_t *>(m->pinned) + kPinnedBytes / 4 - 1;
+    SBP_CUDA(cudaMemcpyAsync((void *)h, m->status, 4, cudaMemcpyDeviceToHost, m->stream));
     SBP_CUDA(cudaStreamSynchronize(m->stream));
+    const int32_t st = *h;
     if (st != 0) {
         SBP_CUDA(cudaMemsetAsync(m->status, 0, 4, m->stream));
         return fail(st, "a kernel recorded status " + std::to_string(st) +
@@ -749,9 +752,21 @@ extern "C" int sbp_get_blockmodel_coo(const sbp_model_t *m, int64_t capacity, in
 
 extern "C" int sbp_get_degrees(const sbp_model_t *m, int32_t *dout, int32_t *din) {
     if (!m) return fail(SBP_EINVAL, "sbp_get_degrees: NULL model");
-    if (dout) SBP_CUDA(cudaMemcpyAsync(dout, m->dout, (size_t)m->B * 4, kind_from_dev(dout), m->stream));
-    if (din) SBP_CUDA(cudaMemcpyAsync(din, m->din, (size_t)m->B * 4, kind_from_dev(din), m->stream));
-    return check_status(m);
+    // few blocks to host arrays go through the pinned buffer with the status
+    const size_t bytes = (size_t)m->B * 4;
+    int32_t *user[2] = {dout, din}, *via[2] = {nullptr, nullptr};
+    const int32_t *from[2] = {m->dout, m->din};
+    for (int q = 0; q < 2; ++q) {
+        if (!user[q]) continue;
+        const cudaMemcpyKind kind = kind_from_dev(user[q]);
+        if (kind == cudaMemcpyDeviceToHost && 2 * bytes + 4 <= kPinnedBytes)
+            via[q] = static_cast<int32_t *>(m->pinned) + (size_t)q * m->B;
+        SBP_CUDA(cudaMemcpyAsync(via[q] ? via[q] : user[q], from[q], bytes, kind, m->stream));
+    }
+    SBP_TRY(check_status(m));
+    for (int q = 0; q < 2; ++q)
+        if (via[q]) std::memcpy(user[q], via[q], bytes);
+    return SBP_OK;
 }
 
 // ---------------------------------------------------------------------------

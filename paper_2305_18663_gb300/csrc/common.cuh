@@ -36,6 +36,7 @@ void count_launch();
 // Device memory of a model: stream-ordered allocation on the model's stream
 // (no device-wide synchronisation, so threads driving other models are not
 // stalled), and a pool of small pinned host buffers for read-backs.
+constexpr size_t kPinnedBytes = 4096;  // of a model's pinned buffer
 cudaError_t model_alloc(void **p, size_t bytes, cudaStream_t st);
 void model_free(void *p, cudaStream_t st);
 void *pinned_get();
