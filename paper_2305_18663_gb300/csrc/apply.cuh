@@ -94,21 +94,30 @@ __device__ __forceinline__ void prefix_block(const int32_t *M, int B, int u, uin
                                              int32_t *__restrict__ dsum, uint32_t *__restrict__ Pc, int pstep) {
     const int lane = threadIdx.x & 31;
     uint32_t *row = P + (size_t)u * 2 * B;
-    uint32_t carry = 0;
-    for (int c0 = 0; c0 < B; c0 += 32) {
-        const int c = c0 + lane;
-        uint32_t v = c < B ? (uint32_t)M[(size_t)u * B + c] : 0u;
-        v = warp_incl_scan_u32(v) + carry;
-        if (c < B) row[c] = v;
-        carry = __shfl_sync(0xffffffffu, v, 31);
-    }
-    const uint32_t du_out = carry;
-    for (int c0 = 0; c0 < B; c0 += 32) {
-        const int c = c0 + lane;
-        uint32_t v = c < B ? (uint32_t)M[(size_t)c * B + u] : 0u;
-        v = warp_incl_scan_u32(v) + carry;
-        if (c < B) row[B + c] = v;
-        carry = __shfl_sync(0xffffffffu, v, 31);
+    uint32_t carry = 0, du_out = 0;
+    // the row, then the column: kPrefixIn chunks of 32 counts in flight
+    constexpr int kPrefixIn = 4;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+        const int32_t *from = half ? M + u : M + (size_t)u * B;
+        const size_t step = half ? (size_t)B : 1;
+        uint32_t *to = row + half * B;
+        for (int c0 = 0; c0 < B; c0 += 32 * kPrefixIn) {
+            uint32_t v[kPrefixIn];
+#pragma unroll
+            for (int q = 0; q < kPrefixIn; ++q) {
+                const int c = c0 + 32 * q + lane;
+                v[q] = c < B ? (uint32_t)from[c * step] : 0u;
+            }
+#pragma unroll
+            for (int q = 0; q < kPrefixIn; ++q) {
+                const int c = c0 + 32 * q + lane;
+                const uint32_t x = warp_incl_scan_u32(v[q]) + carry;
+                if (c < B) to[c] = x;
+                carry = __shfl_sync(0xffffffffu, x, 31);
+            }
+        }
+        if (!half) du_out = carry;
     }
     __syncwarp();
     const int pi = (lane + 1) * pstep - 1 < 2 * B - 1 ? (lane + 1) * pstep - 1 : 2 * B - 1;

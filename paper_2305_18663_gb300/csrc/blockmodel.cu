@@ -94,8 +94,10 @@ __global__ void __launch_bounds__(kThreads) k_prefix_dense(const int32_t *__rest
 //      column prefixes from the sums of the chunks above;
 //   4. k_wide_finish: pivots, din, reciprocals, the column degrees' share of L.
 // Prefix rows and DL at B = 4096: 179 -> 94 us (rows 41, sums 15, columns 28,
-// finish 9; 64 MB read twice, 134 MB written).
-constexpr int kWidePrefixB = 1024;
+// finish 9; 64 MB read twice, 134 MB written).  The line: a commit with nothing
+// moved takes, with a warp per block and with these, 55 and 57 us at B = 1024,
+// 60 and 62 at 1300, 70 and 63 at 1600, 66 and 68 at 2047, 106 and 93 at 3000.
+constexpr int kWidePrefixB = 1400;
 constexpr int kColChunk = 256;
 constexpr int kRowIn = 8;  // counts of a row in flight per thread
 
