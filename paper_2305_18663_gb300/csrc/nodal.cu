@@ -882,7 +882,10 @@ __global__ void __launch_bounds__(kBigThreads) k_eval_cta(DecideArgs a, int bin,
 constexpr int batch_min_blocks(int mode, bool dl32) {
     return mode == 0 ? (dl32 ? SBP_BATCH0_MIN_BLOCKS : 3) : (dl32 ? SBP_DECIDE_MIN_BLOCKS : 2);
 }
-constexpr int kBatchEdges = 32 * kSmallDeg;     // edge ends per sub-batch (33..128)
+// edge ends per sub-batch (33..128): 768 keep a CTA at 64 KB at B = 316, so
+// that three fit an SM (three sweeps of the 1M-vertex graph: 3699 us at 1024,
+// 3630 at 768, 3689 at 640 and at 512)
+constexpr int kBatchEdges = 768;
 constexpr int kBatchEdges0 = SBP_BATCH0_EDGES;  // ... for rows of at most 32
 constexpr int kDirectMaxB = 2048;  // direct-mapped per-warp counts up to this B
 
