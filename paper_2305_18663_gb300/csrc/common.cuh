@@ -365,56 +365,6 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-__device__ __forceinline__ int warp_sum_i(int v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// first index i in a[0, len) with a[i] > t (a non-decreasing, a[len-1] > t),
-// warp-cooperative 32-ary search; every lane returns the answer
-__device__ __forceinline__ int warp_upper_bound(const uint32_t *__restrict__ a, int len, uint32_t t) {
-    const int lane = threadIdx.x & 31;
-    int lo = 0;
-    while (len > 32) {
-        const int step = (len + 31) >> 5;
-        int idx = lo + (lane + 1) * step - 1;
-        const int last = lo + len - 1;
-        if (idx > last) idx = last;
-        const uint32_t val = a[idx];
-        const unsigned mask = __ballot_sync(0xffffffffu, val > t);
-        const int first = __ffs(mask) - 1;  // a[last] > t, so mask != 0
-        const int nlo = lo + first * step;
-        const int nhi = (lo + (first + 1) * step - 1 < last) ? lo + (first + 1) * step - 1 : last;
-        lo = nlo;
-        len = nhi - nlo + 1;
-    }
-    const uint32_t val = lane < len ? a[lo + lane] : 0xffffffffu;
-    const unsigned mask = __ballot_sync(0xffffffffu, val > t);
-    return lo + __ffs(mask) - 1;
-}
-
-// first index i in Pu[0, len) with Pu[i] > t, given the 32 pivots
-// Pcu[q] = Pu[min((q+1) step - 1, len - 1)]: the pivots pick a segment of at
-// most `step` entries, searched with one more read while step <= 32
-__device__ __forceinline__ int warp_cdf_search(const uint32_t *__restrict__ Pu, const uint32_t *Pcu, int len, int step,
-                                               uint32_t t) {
-    const int lane = threadIdx.x & 31;
-    if (len <= 32) {
-        const uint32_t val = lane < len ? Pu[lane] : 0xffffffffu;
-        return __ffs(__ballot_sync(0xffffffffu, val > t)) - 1;
-    }
-    const uint32_t pv = Pcu[lane];
-    const int first = __ffs(__ballot_sync(0xffffffffu, pv > t)) - 1;
-    const int lo = first * step;
-    const int seg = step < len - lo ? step : len - lo;
-    if (seg <= 32) {
-        const uint32_t val = lane < seg ? Pu[lo + lane] : 0xffffffffu;
-        return lo + __ffs(__ballot_sync(0xffffffffu, val > t)) - 1;
-    }
-    return lo + warp_upper_bound(Pu + lo, seg, t);
-}
-
 // ---------------------------------------------------------------------------
 // blockmodel access (dense or sparse, a kernel-wide flag)
 

@@ -393,26 +393,6 @@ __device__ __forceinline__ bool table_add(int *keys, unsigned long long *cnt, in
     return false;
 }
 
-// the same with 32-bit counts (ko | ki << 16) and 16-bit list entries
-__device__ __forceinline__ bool table_add32(int *keys, unsigned *cnt, unsigned short *list, int *nlist, int cap,
-                                            int cap_log2, int key, unsigned inc) {
-    unsigned h = hash_slot(key, cap_log2);
-    for (int p = 0; p < cap; ++p) {
-        const int prev = atomicCAS(&keys[h], -1, key);
-        if (prev == -1) {
-            list[atomicAdd(nlist, 1)] = (unsigned short)h;
-            atomicAdd(&cnt[h], inc);
-            return true;
-        }
-        if (prev == key) {
-            atomicAdd(&cnt[h], inc);
-            return true;
-        }
-        h = (h + 1) & (unsigned)(cap - 1);
-    }
-    return false;
-}
-
 // an accepted move v -> s of a vertex with k edges: the pending label and
 // its items in the accepted-move list
 __device__ __forceinline__ void accept_move(const ModelDev &md, int v, int s, int k) {
