@@ -12,7 +12,7 @@
 // The rows used to be built by counting and std::sort on the host cores (a
 // random access per edge and pass, threads started and joined at any size):
 // loading 4M edges of 200k vertices from host memory and scoring a partition
-// of them took 80.8 ms so, and takes 1.62 ms now; a full run of a 10k-edge
+// of them took 80.8 ms so, and takes 1.49 ms now; a full run of a 10k-edge
 // graph lost 2 ms to it.
 #include <algorithm>
 #include <string>
@@ -200,8 +200,7 @@ struct Carver {
 
 struct Scratch {
     int32_t *src = nullptr, *dst = nullptr;  // the edge list, when it has to be copied
-    uint64_t *k0 = nullptr, *k1 = nullptr;   // edge sort keys
-    uint32_t *i0 = nullptr, *i1 = nullptr, *v0 = nullptr, *v1 = nullptr;
+    uint64_t *k0 = nullptr, *k1 = nullptr;   // edge sort keys, then the other sorts' keys and values
     uint32_t *words = nullptr;
     Info *info = nullptr;
     unsigned *count = nullptr;
@@ -217,14 +216,18 @@ int load_edges(int64_t m, const int32_t *from, int32_t *buf, const int32_t **use
 
 template <class K>
 int sort_edges(const int32_t *s, const int32_t *d, int64_t m, int64_t n, const Scratch &x, sbp_graph *g,
-               cudaStream_t st) {
+               uint32_t **spent, uint32_t **unused, cudaStream_t st) {
     K *k0 = reinterpret_cast<K *>(x.k0), *k1 = reinterpret_cast<K *>(x.k1);
     k_edge_keys<K><<<grid_of(m), kT, 0, st>>>(s, d, m, n, k0, x.info);
     SBP_LAUNCHED();
     bool first = true;
     SBP_TRY((radix_sort<K, uint32_t>(k0, k1, nullptr, nullptr, m, bits_for((uint64_t)n * (uint64_t)n - 1), x.words, st,
                                      &first)));
-    k_out_rows<K><<<grid_of(m), kT, 0, st>>>(first ? k0 : k1, m, n, g->oc, g->esrc, x.i0, x.v0);
+    // the in-rows' keys and values go where the sorted keys are not; those are
+    // done with after this
+    *unused = reinterpret_cast<uint32_t *>(first ? x.k1 : x.k0);
+    *spent = reinterpret_cast<uint32_t *>(first ? x.k0 : x.k1);
+    k_out_rows<K><<<grid_of(m), kT, 0, st>>>(first ? k0 : k1, m, n, g->oc, g->esrc, *unused, *unused + m);
     SBP_LAUNCHED();
     return SBP_OK;
 }
@@ -248,19 +251,18 @@ int build_graph(sbp_graph *g, const int32_t *src, const int32_t *dst, const Scra
     const int64_t n = g->n, m = g->m;
     SBP_CUDA(cudaMemsetAsync(x.info, 0, sizeof(Info), st));
     SBP_CUDA(cudaMemsetAsync(&x.info->bad, 0xff, 8, st));
-    *ikey = x.i0;
+    *ikey = nullptr;
     if (m > 0) {
         const int32_t *s, *d;
         SBP_TRY(load_edges(m, src, x.src, &s, st));
         SBP_TRY(load_edges(m, dst, x.dst, &d, st));
-        if ((uint64_t)n * (uint64_t)n <= (uint64_t(1) << 32)) SBP_TRY(sort_edges<uint32_t>(s, d, m, n, x, g, st));
-        else SBP_TRY(sort_edges<uint64_t>(s, d, m, n, x, g, st));
+        uint32_t *a = nullptr, *c = nullptr;  // keys and values, and their second set
+        if ((uint64_t)n * (uint64_t)n <= (uint64_t(1) << 32)) SBP_TRY(sort_edges<uint32_t>(s, d, m, n, x, g, &c, &a, st));
+        else SBP_TRY(sort_edges<uint64_t>(s, d, m, n, x, g, &c, &a, st));
         bool first = true;
-        SBP_TRY((radix_sort<uint32_t, uint32_t>(x.i0, x.i1, x.v0, x.v1, m, bits_for((uint64_t)n - 1), x.words, st,
-                                                &first)));
-        *ikey = first ? x.i0 : x.i1;
-        k_in_rows<<<grid_of(m), kT, 0, st>>>(*ikey, first ? x.v0 : x.v1, g->esrc, m, g->ic, g->idst,
-                                                  g->tw_oi, g->tw_io, x.info);
+        SBP_TRY((radix_sort<uint32_t, uint32_t>(a, c, a + m, c + m, m, bits_for((uint64_t)n - 1), x.words, st, &first)));
+        *ikey = first ? a : c;
+        k_in_rows<<<grid_of(m), kT, 0, st>>>(*ikey, *ikey + m, g->esrc, m, g->ic, g->idst, g->tw_oi, g->tw_io, x.info);
         SBP_LAUNCHED();
     }
     k_row_offsets<<<grid_of(n + 1), kT, 0, st>>>(g->esrc, *ikey, m, n, g->op, g->ip);
@@ -315,12 +317,8 @@ void carve_scratch(Scratch &x, int64_t n, int64_t m, bool copy_src, bool copy_ds
     const size_t mm = (size_t)m, nv = (size_t)std::max(n, m);
     c.take(&x.src, copy_src ? mm : 0);
     c.take(&x.dst, copy_dst ? mm : 0);
-    c.take(&x.k0, nv);  // the vertex orders are sorted here too
+    c.take(&x.k0, nv);
     c.take(&x.k1, nv);
-    c.take(&x.i0, mm);
-    c.take(&x.i1, mm);
-    c.take(&x.v0, mm);
-    c.take(&x.v1, mm);
     c.take(&x.words, (size_t)sort_scratch_words((int64_t)nv));
     c.take(&x.info, 1);
     c.take(&x.count, 1);
