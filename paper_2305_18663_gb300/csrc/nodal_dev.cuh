@@ -557,20 +557,20 @@ __device__ __forceinline__ void evaluate_group(const DecideArgs &a, const ModelD
     const unsigned gm = group_mask<G>();
     const int gl = (threadIdx.x & 31) & (G - 1);
     const int gbase = (threadIdx.x & 31) & ~(G - 1);
-    // neighbours in r and in s (one lane holds each); 16-bit fields when
-    // the degree allows it
+    // neighbours in r and in s (one lane holds each); unsigned 16-bit fields
+    // when the degree allows it
     if (x.k < 65536) {
-        int pr = 0, ps = 0;
+        unsigned pr = 0, ps = 0;
         each_entry([&](int t, int ko, int ki) {
-            if (t == x.r) pr += ko | (ki << 16);
-            else if (t == x.s) ps += ko | (ki << 16);
+            if (t == x.r) pr += (unsigned)ko | ((unsigned)ki << 16);
+            else if (t == x.s) ps += (unsigned)ko | ((unsigned)ki << 16);
         });
         pr = group_sum<G>(pr, gm);
         ps = group_sum<G>(ps, gm);
-        x.ko_r = pr & 0xffff;
-        x.ki_r = pr >> 16;
-        x.ko_s = ps & 0xffff;
-        x.ki_s = ps >> 16;
+        x.ko_r = (int)(pr & 0xffffu);
+        x.ki_r = (int)(pr >> 16);
+        x.ko_s = (int)(ps & 0xffffu);
+        x.ki_s = (int)(ps >> 16);
     } else {
         int a0 = 0, a1 = 0, a2 = 0, a3 = 0;
         each_entry([&](int t, int ko, int ki) {
