@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, SBP_DIRECT_MIN_BLOCKS) k_ev
 // batches of 32 movers a warp (below) give a small graph too few warps, each
 // with a long serial aggregation: the three groups' kernels and the recheck
 // launch took 80 us at 1000 vertices and 107 us at 20,000 (16 edges out of
-// each), this takes 11 and 39 us.  It is bound by the chain of dependent
+// each), this takes 11 and 39 us (where the line lies: small_pass).  It is bound by the chain of dependent
 // loads of a proposal and a move, a few of them per warp.
 template <bool DL32>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 2) k_eval_small(DecideArgs a, int warp_words) {
@@ -1658,6 +1658,10 @@ int cta_table(sbp_model *m, int cap, int sms, int *grid, size_t *smem, unsigned 
 template <bool DL32, bool FUSED>
 int launch_groups(sbp_model *m, const DecideArgs &a, int sms, const cudaStream_t st[3]) {
     const sbp_graph *g = m->g;
+// Warps of a CTA of the kernels with direct-mapped counts: half as many where
+// eight warps' counts would leave one CTA an SM (B > 1022).
+int direct_warps(int B) { return (2 * B + 4) * 4 * kWarpsPerCta <= 64 * 1024 ? kWarpsPerCta : kWarpsPerCta / 2; }
+
     const int B = m->B;
     // one launch of k_eval_table over list `bin`, tables of 2^cap_log2 slots
     auto tables = [&](int bin, int cap_log2, cudaStream_t on) -> int {
@@ -1680,7 +1684,7 @@ int launch_groups(sbp_model *m, const DecideArgs &a, int sms, const cudaStream_t
     // had sent all of it to the CTA kernel.
     if (g->bin[4] > g->bin[3] && !a.split_top) {
         const int warp_words = 2 * B + 4;
-        const int nwarps = warp_words * 4 * kWarpsPerCta <= 64 * 1024 ? kWarpsPerCta : kWarpsPerCta / 2;
+        const int nwarps = direct_warps(B);
         const size_t smem = (size_t)warp_words * 4 * nwarps;
         SBP_TRY(ensure_dyn_smem((const void *)k_eval_warp_direct<DL32, FUSED>, smem));
         k_eval_warp_direct<DL32, FUSED><<<sms * 4, nwarps * 32, smem, st[2]>>>(a, 2, warp_words);
@@ -1750,16 +1754,33 @@ int launch_recheck(sbp_model *m, const DecideArgs &a0, int sms) {
     return SBP_OK;
 }
 
-// Passes of at most this many vertices take k_eval_small.  Both sides, in us
-// (small pass, the groups' kernels; 16 edges out of each vertex / 20 with a
-// heavy tail): 40,000 vertices 64, 113 / 78, 150; 60,000 85, 103 / 106, 146;
-// 100,000 130, 126 / 174, 180; 200,000 246, 157 / 319, 223.
-constexpr int64_t kSmallPass = 60000;
+// Whether a pass over the vertices of `a` takes k_eval_small, which gives
+// every mover a warp: up to the most vertices at which it was nowhere slower
+// than the groups' kernels, by what these have to do.
+//   - Only the group of up to 32 edges: one kernel with 32 movers a warp.
+//   - More groups: a kernel each, one after another (below 2^19 edges) or on
+//     three streams; rows of hundreds of edges have a warp each there too,
+//     with twice the warps, and win from some 2^21 edges on (the line: 3 x 2^19).
+//   - B > 1022: half the warps here, none lost there in the first group.
+// Both sides in us (groups, small; labels near the planted ones, B = 4 / 1000;
+// B = 2048): only the first group, 6000 vertices 27, 28 / 35, 34; 34, 36; at
+// 20,000 42, 40 / 53, 60; 57, 83; at 60,000 50, 77 / 65, 109; 75, 193.  More
+// groups, 6 edges a vertex and three hubs of 300, 20,000 vertices 51, 42 /
+// 66, 56; 58, 83; at 30,000 54, 52 / 70, 69; 74, 112; at 60,000 62, 76 / 81,
+// 107; 87, 187; 32 edges a vertex, 20,000 71, 41 / 111, 52; 114, 75; 40,000
+// (2^19.3 edges) 48, 61 / 68, 75; 81, 120.
+bool small_pass(const sbp_graph *g, const DecideArgs &a, int B) {
+    const int64_t n = a.vcount[0] + a.vcount[1] + a.vcount[2];
+    const bool half = direct_warps(B) < kWarpsPerCta;
+    if (a.vcount[1] + a.vcount[2] == 0) return n <= (half ? 2500 : 5000);
+    if (g->m < kSideStreamEdges) return n <= (half ? 8000 : 22000);
+    return g->m <= 3 * (int64_t(1) << 19) && n <= (half ? 6000 : 20000);
+}
 
 template <bool DL32>
 int launch_small(sbp_model *m, const DecideArgs &a, int sms) {
     const int warp_words = 2 * m->B + 4;
-    const int nwarps = warp_words * 4 * kWarpsPerCta <= 64 * 1024 ? kWarpsPerCta : kWarpsPerCta / 2;
+    const int nwarps = direct_warps(m->B);
     const size_t smem = (size_t)warp_words * 4 * nwarps;
     SBP_TRY(ensure_dyn_smem((const void *)k_eval_small<DL32>, smem));
     const int64_t n = a.vcount[0] + a.vcount[1] + a.vcount[2];
@@ -1884,7 +1905,7 @@ int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_en
     }
     const bool fused = SBP_FUSED_PROPOSALS && v_begin == 0 && v_end == g->n && !a.skip && !a.trace_on &&
                        B <= kDirectMaxB && g->max_deg < 65536;
-    if (fused && a.vcount[0] + a.vcount[1] + a.vcount[2] <= kSmallPass)
+    if (fused && small_pass(g, a, B))
         return m->p.dl_fp32 ? launch_small<true>(m, a, sms) : launch_small<false>(m, a, sms);
     SBP_CUDA(cudaMemsetAsync(m->mcount, 0, kMoverLists * sizeof(unsigned), m->stream));
     if (!fused) {

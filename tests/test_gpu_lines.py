@@ -1,0 +1,57 @@
+"""Where the one-launch pass ends: on both sides of each line a pass takes the
+form it should (seen in the number of kernels it launches) and gives what the
+general kernels give.  Labels, counts, degrees, statistics and DL are compared
+exactly."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_2305_18663_gb300 as P  # noqa: E402
+from synth.dcsbm import random_labels  # noqa: E402
+from test_gpu_small import _same  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def _launches(call):
+    before = P.sbp_kernel_launches()
+    call()
+    return P.sbp_kernel_launches() - before
+
+
+def _graph(n, extra, seed):
+    """every vertex with two edges out and two in; then `extra`: None, "hub"
+    (one vertex with 300 edges more) or a number of random edges in all"""
+    rng = np.random.default_rng(seed)
+    v = np.arange(n)
+    src, dst = [v, v], [(v + 1) % n, (v + n // 3) % n]
+    if extra == "hub":
+        src, dst = src + [np.zeros(300, np.int64)], dst + [rng.integers(0, n, 300)]
+    elif extra:
+        src, dst = src + [rng.integers(0, n, extra - 2 * n)], dst + [rng.integers(0, n, extra - 2 * n)]
+    return P.Graph(n, np.concatenate(src).astype(np.int32), np.concatenate(dst).astype(np.int32))
+
+
+@pytest.mark.parametrize("n,extra,B,one", [
+    (5_000, None, 1022, True), (5_001, None, 100, False), (2_500, None, 1023, True), (2_501, None, 1023, False),
+    (22_000, "hub", 100, True), (22_001, "hub", 100, False), (8_000, "hub", 1023, True), (8_001, "hub", 1023, False),
+    (20_000, 1 << 19, 100, True), (20_001, 1 << 19, 100, False),
+    (6_000, 1 << 19, 1023, True), (6_001, 1 << 19, 1023, False),
+    (2_000, 3 << 19, 100, True), (2_000, (3 << 19) + 1, 100, False),
+])
+def test_pass_form_and_result(n, extra, B, one):
+    pg = _graph(n, extra, seed=n)
+    b = random_labels(n, B, seed=1)
+    for dl_fp32 in (1, 0):
+        prm = P.Params.default(seed=4, dl_fp32=dl_fp32)
+        whole, parts = P.Model(pg, B, b, prm), P.Model(pg, B, b, prm)
+        for sw in range(2):
+            k = _launches(lambda: P.sbp_nodal_decide(whole.h, sw, 0, n))
+            if sw > 0:  # (the first pass also makes the block-labelled rows)
+                assert (k == 1) == one, k
+            for lo, hi in ((0, n // 3), (n // 3, n)):
+                P.sbp_nodal_decide(parts.h, sw, lo, hi)
+            a, c = P.sbp_commit(whole.h), P.sbp_commit(parts.h)
+            assert a.n_moves > 0 and a.as_dict() | {"n_recheck": 0} == c.as_dict() | {"n_recheck": 0}
+        _same(whole, parts)
