@@ -1556,6 +1556,7 @@ static constexpr int64_t kSideStreamEdges = int64_t(1) << 19;
 // three streams for kernels that may run together: the model's own one (for
 // the longest) and its side streams, forked here and joined by join_side (all
 // the model's own on smaller graphs)
+static constexpr int64_t kSideFirstGroup = 8192;
 int fork_side(sbp_model *m, cudaStream_t st[3]) {
     st[0] = st[1] = st[2] = m->stream;
     if (m->g->m < kSideStreamEdges) return SBP_OK;
@@ -1793,10 +1794,19 @@ int launch_small(sbp_model *m, const DecideArgs &a, int sms) {
 
 template <bool DL32>
 int launch_evals(sbp_model *m, const DecideArgs &a, int sms, bool fused) {
-    cudaStream_t st[3];
-    SBP_TRY(fork_side(m, st));
+    cudaStream_t st[3] = {m->stream, m->stream, m->stream};
+    // One group alone has nothing to run beside it (a sweep of 200k vertices of
+    // 10 edges lost 10 us to the fork), and the first group's kernel on few
+    // vertices is over in 7 us (two sweeps of 60,000 vertices of 67 edges, a
+    // handful of them in it, at B = 1000: 611 us forked, 548 not).
+    // (the top group's classes at large B are kernels of their own.)
+    const sbp_graph *g = m->g;
+    const int64_t *vc = a.vcount;
+    const bool several = (vc[1] > 0 && vc[2] > 0) || (vc[0] >= kSideFirstGroup && vc[1] + vc[2] > 0) ||
+                         (a.split_top && (g->n_mid > 0) + (g->n_wide > 0) + (vc[2] > g->n_mid + g->n_wide) > 1);
+    if (several) SBP_TRY(fork_side(m, st));
     const int rc = fused ? launch_groups<DL32, true>(m, a, sms, st) : launch_groups<DL32, false>(m, a, sms, st);
-    const int rj = join_side(m);  // joined on every path
+    const int rj = several ? join_side(m) : SBP_OK;  // joined on every path
     if (rc != SBP_OK) return rc;
     if (rj != SBP_OK) return rj;
     return launch_recheck<DL32>(m, a, sms);
