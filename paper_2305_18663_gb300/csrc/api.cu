@@ -124,10 +124,9 @@ int validate_params(const sbp_params &p) {
     return SBP_OK;
 }
 
-// the host's copy of a pass's report, once the stream has reached it
+// a pass's report, once the stream has reached the host's copy of it
 int finish_stats(sbp_model *m, sbp_sweep_stats *out) {
     const SweepReadback *h = static_cast<const SweepReadback *>(m->pinned);
-    SBP_CUDA(cudaStreamSynchronize(m->stream));
     if (h->status != 0) {
         const int st = h->status;
         SBP_CUDA(cudaMemsetAsync(m->status, 0, 4, m->stream));
@@ -150,6 +149,7 @@ int read_stats(sbp_model *m, sbp_sweep_stats *out) {
     SBP_CUDA(cudaMemcpyAsync(&h->c, m->counters, sizeof(DevCounters), cudaMemcpyDeviceToHost, m->stream));
     SBP_CUDA(cudaMemcpyAsync(h->dl, m->dl, 16, cudaMemcpyDeviceToHost, m->stream));
     SBP_CUDA(cudaMemcpyAsync(&h->status, m->status, 4, cudaMemcpyDeviceToHost, m->stream));
+    SBP_CUDA(cudaStreamSynchronize(m->stream));
     return finish_stats(m, out);
 }
 
@@ -210,27 +210,27 @@ __global__ void k_diff_labels(const int32_t *__restrict__ bnew, const int32_t *_
 // Same counts and DL as a rebuild from scratch.
 int upload_incremental(sbp_model *m, const int32_t *b) {
     const int64_t n = m->g->n;
-    int32_t *slot = m->status + 2;
+    DiffCounters *diff = reinterpret_cast<DiffCounters *>(m->counters);
     SBP_CUDA(cudaMemcpyAsync(m->bnew, b, (size_t)n * 4, cudaMemcpyDefault, m->stream));
-    SBP_CUDA(cudaMemsetAsync(m->counters, 0, sizeof(DevCounters), m->stream));
-    SBP_CUDA(cudaMemsetAsync(slot, 0, 4, m->stream));
+    SBP_CUDA(cudaMemsetAsync(diff, 0, sizeof(DiffCounters), m->stream));
     k_diff_labels<<<(int)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, m->stream>>>(
-        m->bnew, m->b, n, m->B, m->g->op, m->g->ip, m->items, m->cap_items, m->counters, slot);
+        m->bnew, m->b, n, m->B, m->g->op, m->g->ip, m->items, m->cap_items, m->counters, &diff->bad);
     SBP_LAUNCHED();
-    int32_t *h = static_cast<int32_t *>(m->pinned);
-    SBP_CUDA(cudaMemcpyAsync(h, slot, 4, cudaMemcpyDeviceToHost, m->stream));
+    const DiffCounters *h = static_cast<const DiffCounters *>(m->pinned);
+    SBP_CUDA(cudaMemcpyAsync(m->pinned, diff, sizeof(DiffCounters), cudaMemcpyDeviceToHost, m->stream));
     SBP_CUDA(cudaStreamSynchronize(m->stream));
-    if (*h > 0) {
+    if (h->bad > 0) {
         SBP_CUDA(cudaMemcpyAsync(m->bnew, m->b, (size_t)n * 4, cudaMemcpyDeviceToDevice, m->stream));
         SBP_CUDA(cudaMemsetAsync(m->counters, 0, sizeof(DevCounters), m->stream));
-        return fail(SBP_EINVAL, "label out of [0, B) at vertex " + std::to_string((int64_t)INT32_MAX - *h));
+        return fail(SBP_EINVAL, "label out of [0, B) at vertex " + std::to_string((int64_t)INT32_MAX - h->bad));
     }
     std::swap(m->b, m->bnew);
     m->list_ok = true;  // the items list every change, once
     m->decided.clear();
     m->nb_in_commit = false;
-    if (commit_small_ok(m)) {
-        const int rs = commit_small(m, nullptr);
+    m->light = commit_small_load_ok(m, h->c);
+    if (m->light && commit_small_ok(m)) {
+        const int rs = commit_small(m, nullptr, false);
         if (rs != SBP_OK) m->nb_ok = false;
         return rs;
     }
@@ -353,7 +353,7 @@ extern "C" int sbp_build_blockmodel(const sbp_graph_t *g, int32_t B, const int32
     if (model_alloc((void **)&m->b, n * 4, st) != cudaSuccess || model_alloc((void **)&m->bnew, n * 4, st) != cudaSuccess ||
         model_alloc((void **)&m->dl, 16, st) != cudaSuccess ||
         model_alloc((void **)&m->partials, (size_t)m->npartials * 32, st) != cudaSuccess ||
-        model_alloc((void **)&m->counters, sizeof(DevCounters), st) != cudaSuccess ||
+        model_alloc((void **)&m->counters, sizeof(DiffCounters), st) != cudaSuccess ||
         model_alloc((void **)&m->status, 16, st) != cudaSuccess || !m->pinned) {
         cudaGetLastError();
         sbp_free_model(m);
@@ -438,12 +438,20 @@ extern "C" int sbp_set_pending(sbp_model_t *m, int64_t v_begin, int64_t v_end, c
 extern "C" int sbp_commit(sbp_model_t *m, sbp_sweep_stats *stats) {
     if (!m) return fail(SBP_EINVAL, "sbp_commit: NULL model");
     std::swap(m->b, m->bnew);
-    if (commit_small_ok(m)) {
-        const int rs = commit_small(m, stats ? static_cast<SweepReadback *>(m->pinned) : nullptr);
-        m->decided.clear();
+    // (without statistics nothing is waited for, so the kernel's word on the
+    // load could not be read)
+    SweepReadback *h = static_cast<SweepReadback *>(m->pinned);
+    const bool fits = commit_small_fits(m);
+    if (commit_small_ok(m) && (fits || (stats && m->light))) {
+        int rs = commit_small(m, stats ? h : nullptr, !fits);
+        if (rs == SBP_OK && stats && cudaStreamSynchronize(m->stream) != cudaSuccess)
+            rs = cuda_fail(cudaGetLastError(), "sbp_commit");
         if (rs != SBP_OK) m->nb_ok = false;
-        SBP_TRY(rs);
-        return stats ? finish_stats(m, stats) : SBP_OK;
+        if (rs != SBP_OK || fits || h->done) {
+            m->decided.clear();
+            SBP_TRY(rs);
+            return stats ? finish_stats(m, stats) : SBP_OK;
+        }
     }
     SBP_CUDA(cudaMemcpyAsync(m->dl + 1, m->dl, 8, cudaMemcpyDeviceToDevice, m->stream));
     m->nb_in_commit = false;
@@ -453,7 +461,10 @@ extern "C" int sbp_commit(sbp_model_t *m, sbp_sweep_stats *stats) {
     m->list_ok = true;
     m->decided.clear();
     SBP_TRY(rc);
-    if (stats) SBP_TRY(read_stats(m, stats));
+    if (stats) {
+        SBP_TRY(read_stats(m, stats));
+        m->light = commit_small_load_ok(m, h->c);
+    }
     SBP_CUDA(cudaMemsetAsync(m->counters, 0, sizeof(DevCounters), m->stream));
     return SBP_OK;
 }

@@ -513,10 +513,36 @@ __global__ void __launch_bounds__(kThreads, kItemCtas) k_nb_items(GraphDev g, co
 // less than one of work.  With k_eval_small, three sweeps at 1000 vertices
 // and 8 blocks, their labels set before and read back after, took 209 us
 // instead of 526.
+// Its eight SMs are few for much work, so its use has three limits (labels set
+// from outside and committed, the separate kernels and this one, in us):
+//   - blocks, whose prefix rows it builds on 256 warps (2000 vertices, 8000
+//     edges, nothing moved): 66 and 51 at B = 256, 71 and 68 at 384, 74 and 77
+//     at 512;
+//   - moves: an item costs some 6 ns, an edge end of an update 0.15 ns, an edge
+//     of a recount 0.075 ns, against the 20 us it saves.  kCommitMaxLoad is
+//     that budget in items.  B = 128: 8000 vertices, 130,000 edges, load 3270
+//     76 and 70, 6340 82 and 84; 20,000 vertices, 500,000 edges, 2340 80 and
+//     67, 4660 82 and 83, 10,300 83 and 110; 65,000 vertices, 520,000 edges,
+//     1860 83 and 68, 3760 82 and 80, 45,000 91 and 266;
+//   - vertices and edges, up to which these were measured.
+// Where not every commit of the model is within the load, the kernel looks at
+// the moves first and leaves the commit to the separate kernels when there
+// are too many (a launch and a wait lost, once: the next commit is theirs
+// until one is within it).
 constexpr int kCommitThreads = 1024;
 constexpr int kCommitCluster = 8;
-constexpr int kCommitMaxB = 512;
+constexpr int kCommitMaxB = 256;
 constexpr int64_t kCommitMaxEdges = int64_t(1) << 19;
+constexpr int64_t kCommitMaxVertices = int64_t(1) << 16;
+constexpr unsigned long long kCommitMaxLoad = 3300;
+
+__host__ __device__ inline bool commit_counts_moves(const DevCounters &c, int64_t m) {
+    return c.acc_edges * 4ull <= (unsigned long long)m;  // else all edges are counted again
+}
+
+__host__ __device__ inline unsigned long long commit_load(const DevCounters &c, int64_t m) {
+    return c.items + (commit_counts_moves(c, m) ? c.acc_edges / 40 : (unsigned long long)m / 80);
+}
 
 struct SmallCommit {
     GraphDev g;
@@ -537,6 +563,7 @@ struct SmallCommit {
     DlPartial *parts;  // one per block of the cluster
     const int32_t *status;
     SweepReadback *host;  // NULL: not asked for
+    bool checked;         // the load is looked at first (with host)
 };
 
 __global__ void __launch_bounds__(kCommitThreads) k_commit_small(SmallCommit a) {
@@ -546,7 +573,11 @@ __global__ void __launch_bounds__(kCommitThreads) k_commit_small(SmallCommit a) 
     const int B = a.B, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int tid = cluster_rank() * kCommitThreads + threadIdx.x, nt = cluster_size() * kCommitThreads;
     const DevCounters c = *a.counters;
-    const bool counts = c.acc_edges * 4ull <= (unsigned long long)a.g.m;
+    if (a.checked && commit_load(c, a.g.m) > kCommitMaxLoad) {
+        if (tid == 0) a.host->done = 0;
+        return;
+    }
+    const bool counts = commit_counts_moves(c, a.g.m);
     const int64_t items = (int64_t)(c.items < (unsigned long long)a.cap_items ? c.items : (unsigned long long)a.cap_items);
     // the part of DL that does not need the counts (a chain of FP64
     // logarithms) on a thread of its own
@@ -591,6 +622,7 @@ __global__ void __launch_bounds__(kCommitThreads) k_commit_small(SmallCommit a) 
             a.host->dl[0] = after;
             a.host->dl[1] = before;
             a.host->status = *a.status;
+            a.host->done = 1;
         }
         *a.counters = DevCounters{};
     }
@@ -813,10 +845,17 @@ int commit_blockmodel(sbp_model *m) { return build_blockmodel(m, !m->p.full_rebu
 // holds every change
 bool commit_small_ok(const sbp_model *m) {
     return m->dense && !m->p.full_rebuild && m->list_ok && m->items && m->B <= kCommitMaxB &&
-           m->g->m <= kCommitMaxEdges && m->g->n <= (int64_t(1) << 16);
+           m->g->m <= kCommitMaxEdges && m->g->n <= kCommitMaxVertices;
 }
 
-int commit_small(sbp_model *m, SweepReadback *host) {
+// all vertices moved, all edges counted again
+bool commit_small_fits(const sbp_model *m) {
+    return (unsigned long long)(m->g->n + 2 * m->g->m / kMoveChunk + m->g->m / 80) <= kCommitMaxLoad;
+}
+
+bool commit_small_load_ok(const sbp_model *m, const DevCounters &c) { return commit_load(c, m->g->m) <= kCommitMaxLoad; }
+
+int commit_small(sbp_model *m, SweepReadback *host, bool checked) {
     SBP_TRY(xlogx_table(m->g->m + 1, &m->T, &m->XT));
     const bool nb = m->nb_ok && m->nbo;
     SmallCommit a;
@@ -843,6 +882,7 @@ int commit_small(sbp_model *m, SweepReadback *host) {
     a.parts = reinterpret_cast<DlPartial *>(m->partials);
     a.status = m->status;
     a.host = host;
+    a.checked = checked;
     return launch_cluster(k_commit_small, kCommitCluster, kCommitThreads, 0, m->stream, 1, a);
 }
 

@@ -120,11 +120,19 @@ struct DevCounters {
     unsigned long long entries;  // distinct neighbour blocks of the evaluated movers (sum of D_v)
 };
 
+// ... and after labels set from outside: INT32_MAX - the smallest vertex with
+// one out of range (0: none).  A model's counters have room for it.
+struct DiffCounters {
+    DevCounters c;
+    int32_t bad;
+};
+
 // what a pass reports to the host
 struct SweepReadback {
     DevCounters c;
     double dl[2];
     int32_t status;
+    int32_t done;  // the one-launch commit did the commit (0: it left it, see kCommitMaxLoad)
 };
 
 // the accepted-move list: one (vertex, chunk) item per kMoveChunk edges of
@@ -231,6 +239,7 @@ struct sbp_model {
     bool nb_ok = false;
     bool nb_in_commit = false;  // the apply step's kernel updated them in this commit
     bool list_ok = true;
+    bool light = true;  // the last moves known to the host were within the one-launch commit's load
     std::vector<std::pair<int64_t, int64_t>> decided;  // decide ranges since the last commit
     // side streams of the decision pass: the three degree groups' kernels
     // run concurrently so that each one's tail is filled by the others
@@ -589,8 +598,14 @@ int rebuild_blockmodel(sbp_model *m);  // M, P, degrees, rcp, DL from m->b
 int count_cells(sbp_model *m, int32_t *cells);  // cells[r * B + t] = edges r -> t
 int update_cells(sbp_model *m, int32_t *cells);  // counts of m->bnew -> counts of m->b
 int launch_prefix(sbp_model *m);                 // P, Pc, degrees, reciprocals from a dense M
+// the whole commit of a small dense model in one launch: whether the model has
+// the form, whether every commit of it is within the form's load, whether
+// these moves are, and the launch (checked: by the kernel, which leaves the
+// commit and says so in host->done when they are not)
 bool commit_small_ok(const sbp_model *m);
-int commit_small(sbp_model *m, SweepReadback *host);  // the whole commit of a small dense model in one launch
+bool commit_small_fits(const sbp_model *m);
+bool commit_small_load_ok(const sbp_model *m, const DevCounters &c);
+int commit_small(sbp_model *m, SweepReadback *host, bool checked);
 int commit_blockmodel(sbp_model *m);   // the same after a pass: m->b new labels, m->bnew the previous ones
 int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_end, const sbp_vertex_trace *trace);
 int nb_rows_rebuild(sbp_model *m);       // block-labelled rows from m->b (nb_ok when there is memory)

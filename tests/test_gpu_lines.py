@@ -1,7 +1,7 @@
-"""Where the one-launch pass ends: on both sides of each line a pass takes the
-form it should (seen in the number of kernels it launches) and gives what the
-general kernels give.  Labels, counts, degrees, statistics and DL are compared
-exactly."""
+"""Where the one-launch pass and the one-launch commit end: on both sides of
+each line the call takes the form it should (seen in the number of kernels it
+launches) and gives what the general kernels give.  Labels, counts, degrees,
+statistics and DL are compared exactly."""
 import numpy as np
 import pytest
 
@@ -55,3 +55,37 @@ def test_pass_form_and_result(n, extra, B, one):
             a, c = P.sbp_commit(whole.h), P.sbp_commit(parts.h)
             assert a.n_moves > 0 and a.as_dict() | {"n_recheck": 0} == c.as_dict() | {"n_recheck": 0}
         _same(whole, parts)
+
+
+@pytest.mark.parametrize("n,e", [(1_500, 3_000), (65_536, 131_072), (65_537, 131_074), (20_000, 1 << 19),
+                                 (20_000, (1 << 19) + 1)])
+@pytest.mark.parametrize("B", [2, 256, 257])
+def test_commit_form_and_result(n, e, B):
+    pg = _graph(n, None if e == 2 * n else e, seed=n)
+    b = random_labels(n, B, seed=5)
+    one = P.Model(pg, B, b, P.Params.default(seed=6))
+    full = P.Model(pg, B, b, P.Params.default(seed=6, full_rebuild=1))
+    small = n <= 65_536 and e <= 1 << 19 and B <= 256
+    rng = np.random.default_rng(7)
+
+    def sweep(sw, stats=True):
+        a, c = one.sweep(sw, stats=stats), full.sweep(sw)
+        if stats:
+            assert a.as_dict() | {"n_recheck": 0} == c.as_dict() | {"n_recheck": 0}
+        _same(one, full)
+
+    sweep(0)  # random labels: many moves
+    sweep(1)
+    sweep(2, stats=False)
+    # labels set from outside, few of them changed, many, few again; the pass
+    # after each finds the form of the commit before it
+    for sw, frac in ((3, 0.003), (4, 0.9), (5, 0.003)):
+        lab = one.assignment()
+        pick = rng.random(n) < frac
+        lab[pick] = random_labels(n, B, seed=sw)[pick]
+        k = _launches(lambda: P.sbp_set_assignment(one.h, B, lab))
+        # one kernel lists the changes, one commits them
+        assert (k == 2) == (small and (frac < 0.1 or n < 2_000)), k
+        P.sbp_set_assignment(full.h, B, lab)
+        _same(one, full)
+        sweep(sw)
