@@ -63,8 +63,8 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge_proposals(ModelDev md, 
     }
 }
 
-// The application of a merge round: one launch of one block or one cluster,
-// res[0] the links made, res[1] the new block count.
+// The application of a merge round: one launch of one block or one cluster;
+// res (host memory): [0] the links made, [1] the new block count.
 // The line between the two lies where they meet: one merge phase of B blocks
 // (B / 3 merges, 4 B edges) took, with the block and with the cluster, 165
 // and 221 us at 1024, 345 and 384 us at 4096, 420 and 407 us at 8192, 708 and
@@ -115,7 +115,7 @@ int ensure_merge_work(sbp_model *m, int32_t B) {
     model_free(m->merge_work, m->stream);
     m->merge_work = nullptr;
     m->merge_work_B = 0;
-    const size_t bytes = (size_t)B * kMergeApplyBytes + kClusterWords * 4 + 8;
+    const size_t bytes = (size_t)B * kMergeApplyBytes + kClusterWords * 4;
     if (model_alloc((void **)&m->merge_work, bytes, m->stream) != cudaSuccess) {
         cudaGetLastError();
         return fail(SBP_ENOMEM, "device allocation failed for the merge phase");
@@ -127,7 +127,6 @@ int ensure_merge_work(sbp_model *m, int32_t B) {
 struct MergeWork {
     MergeApply w;
     uint32_t *words;
-    int32_t *res;
 };
 
 MergeWork merge_work(const sbp_model *m) {
@@ -141,7 +140,6 @@ MergeWork merge_work(const sbp_model *m) {
     x.w.x1 = p + 3 * B;
     x.w.mark = p + 4 * B;
     x.words = reinterpret_cast<uint32_t *>(p + 5 * B);
-    x.res = reinterpret_cast<int32_t *>(x.words + kClusterWords);
     return x;
 }
 
@@ -184,11 +182,10 @@ int apply_merge_round(sbp_model *m, int32_t want, int32_t *done, int32_t *B_new)
     SBP_TRY(ensure_merge_work(m, m->B));
     const MergeWork x = merge_work(m);
     const bool cl = m->B > kOneCtaB;
+    int32_t *h = static_cast<int32_t *>(m->pinned);  // (written by the kernel)
     SBP_TRY(launch_cluster(cl ? k_merge_apply<true> : k_merge_apply<false>, cl ? kApplyCluster : 1, kApplyThreads, 0,
-                           m->stream, 1, x.w, x.words, (int)m->B,
-                        (const int32_t *)m->best_s, (const double *)m->best_d, (int)want, m->map, x.res));
-    int32_t *h = static_cast<int32_t *>(m->pinned);
-    SBP_CUDA(cudaMemcpyAsync(h, x.res, 8, cudaMemcpyDeviceToHost, m->stream));
+                           m->stream, 1, x.w, x.words, (int)m->B, (const int32_t *)m->best_s,
+                           (const double *)m->best_d, (int)want, m->map, h));
     SBP_CUDA(cudaStreamSynchronize(m->stream));
     *done = h[0];
     *B_new = h[1];
@@ -198,16 +195,14 @@ int apply_merge_round(sbp_model *m, int32_t want, int32_t *done, int32_t *B_new)
 // m->map for dropping the blocks without vertices; *B_new their number left
 int compact_blocks(sbp_model *m, int32_t *B_new) {
     SBP_TRY(launch_vertex_count(m));
-    SBP_TRY(ensure_merge_work(m, m->B));
-    const MergeWork x = merge_work(m);
     const bool cl = m->B > kOneCtaB;
+    if (cl) SBP_TRY(ensure_merge_work(m, m->B));
+    uint32_t *words = cl ? merge_work(m).words : nullptr;  // (a block alone exchanges nothing)
+    int32_t *h = static_cast<int32_t *>(m->pinned);        // (written by the kernel)
     SBP_TRY(launch_cluster(cl ? k_compact_map<true> : k_compact_map<false>, cl ? kApplyCluster : 1, kApplyThreads, 0,
-                           m->stream, 1, x.words, (int)m->B,
-                        (const int32_t *)m->vcount, m->map, x.res));
-    int32_t *h = static_cast<int32_t *>(m->pinned);
-    SBP_CUDA(cudaMemcpyAsync(h, x.res + 1, 4, cudaMemcpyDeviceToHost, m->stream));
+                           m->stream, 1, words, (int)m->B, (const int32_t *)m->vcount, m->map, h));
     SBP_CUDA(cudaStreamSynchronize(m->stream));
-    *B_new = h[0];
+    *B_new = h[1];
     return SBP_OK;
 }
 
