@@ -87,7 +87,13 @@ __device__ __forceinline__ uint32_t warp_incl_scan_u32(uint32_t v) {
 // One warp, block u of a dense M: P[u] = inclusive prefix of row u, then
 // dout_u plus the inclusive prefix of column u (the proposal CDFs); the 32
 // pivots Pc[u]; degrees and the reciprocals of d_u + B.
-// (M through plain loads: the batched MCMC kernel has just updated it)
+// READONLY: the kernel only reads M (its pointer is __restrict__ there), so
+// the compiler moves the next chunks' loads ahead of this one's stores; with
+// the loads of the other form in their place a launch at B = 1000 takes 31 us
+// instead of 12.  Otherwise M has just been updated in the same launch, its
+// loads are plain ones that stay behind the stores, and kPrefixIn chunks of 32
+// counts are in flight by hand.
+template <bool READONLY>
 __device__ __forceinline__ void prefix_block(const int32_t *M, int B, int u, uint32_t *__restrict__ P,
                                              int32_t *__restrict__ dout, int32_t *__restrict__ din,
                                              double *__restrict__ rcp, float *__restrict__ rcp32,
@@ -95,29 +101,45 @@ __device__ __forceinline__ void prefix_block(const int32_t *M, int B, int u, uin
     const int lane = threadIdx.x & 31;
     uint32_t *row = P + (size_t)u * 2 * B;
     uint32_t carry = 0, du_out = 0;
-    // the row, then the column: kPrefixIn chunks of 32 counts in flight
-    constexpr int kPrefixIn = 4;
-#pragma unroll 1
-    for (int half = 0; half < 2; ++half) {
-        const int32_t *from = half ? M + u : M + (size_t)u * B;
-        const size_t step = half ? (size_t)B : 1;
-        uint32_t *to = row + half * B;
-        for (int c0 = 0; c0 < B; c0 += 32 * kPrefixIn) {
-            uint32_t v[kPrefixIn];
-#pragma unroll
-            for (int q = 0; q < kPrefixIn; ++q) {
-                const int c = c0 + 32 * q + lane;
-                v[q] = c < B ? (uint32_t)from[c * step] : 0u;
-            }
-#pragma unroll
-            for (int q = 0; q < kPrefixIn; ++q) {
-                const int c = c0 + 32 * q + lane;
-                const uint32_t x = warp_incl_scan_u32(v[q]) + carry;
-                if (c < B) to[c] = x;
-                carry = __shfl_sync(0xffffffffu, x, 31);
-            }
+    if constexpr (READONLY) {
+        for (int c0 = 0; c0 < B; c0 += 32) {
+            const int c = c0 + lane;
+            const uint32_t x = warp_incl_scan_u32(c < B ? (uint32_t)M[(size_t)u * B + c] : 0u) + carry;
+            if (c < B) row[c] = x;
+            carry = __shfl_sync(0xffffffffu, x, 31);
         }
-        if (!half) du_out = carry;
+        du_out = carry;
+        for (int c0 = 0; c0 < B; c0 += 32) {
+            const int c = c0 + lane;
+            const uint32_t x = warp_incl_scan_u32(c < B ? (uint32_t)M[(size_t)c * B + u] : 0u) + carry;
+            if (c < B) row[B + c] = x;
+            carry = __shfl_sync(0xffffffffu, x, 31);
+        }
+    } else {
+        // the row, then the column
+        constexpr int kPrefixIn = 4;
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            const int32_t *from = half ? M + u : M + (size_t)u * B;
+            const size_t step = half ? (size_t)B : 1;
+            uint32_t *to = row + half * B;
+            for (int c0 = 0; c0 < B; c0 += 32 * kPrefixIn) {
+                uint32_t v[kPrefixIn];
+#pragma unroll
+                for (int q = 0; q < kPrefixIn; ++q) {
+                    const int c = c0 + 32 * q + lane;
+                    v[q] = c < B ? (uint32_t)from[c * step] : 0u;
+                }
+#pragma unroll
+                for (int q = 0; q < kPrefixIn; ++q) {
+                    const int c = c0 + 32 * q + lane;
+                    const uint32_t x = warp_incl_scan_u32(v[q]) + carry;
+                    if (c < B) to[c] = x;
+                    carry = __shfl_sync(0xffffffffu, x, 31);
+                }
+            }
+            if (!half) du_out = carry;
+        }
     }
     __syncwarp();
     const int pi = (lane + 1) * pstep - 1 < 2 * B - 1 ? (lane + 1) * pstep - 1 : 2 * B - 1;

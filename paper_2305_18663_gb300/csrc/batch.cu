@@ -245,7 +245,7 @@ __device__ void squad_rebuild(Sq &sq, const GraphDev &g, const int32_t *b, const
     sq.sync();
     __int128 dd = 0, c = 0;
     for (int u = sq.wid; u < B; u += sq.nw) {
-        prefix_block(w.M, B, u, w.P, w.dout, w.din, w.rcp, w.rcp32, w.dsum, w.Pc, pstep);
+        prefix_block<false>(w.M, B, u, w.P, w.dout, w.din, w.rcp, w.rcp32, w.dsum, w.Pc, pstep);
         if (lane == 0) {
             dd += T[w.dout[u]];
             dd += T[w.din[u]];
@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(Squad<CLUSTER>::T, CLUSTER ? 1 : 2)
                 // 4. prefix rows, degrees, DL, the stopping rule
                 __int128 dd = 0;
                 for (int u = sq.wid; u < B; u += sq.nw) {
-                    prefix_block(sw.M, B, u, sw.P, sw.dout, sw.din, sw.rcp, sw.rcp32, sw.dsum, sw.Pc, md.pstep);
+                    prefix_block<false>(sw.M, B, u, sw.P, sw.dout, sw.din, sw.rcp, sw.rcp32, sw.dsum, sw.Pc, md.pstep);
                     if (lane == 0) {
                         dd += md.T[sw.dout[u]];
                         dd += md.T[sw.din[u]];

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kThreads) k_prefix_dense(const int32_t *__rest
                                                            uint32_t *__restrict__ Pc, int pstep) {
     const int u = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     if (u >= B) return;
-    prefix_block(M, B, u, P, dout, din, rcp, rcp32, dsum, Pc, pstep);
+    prefix_block<true>(M, B, u, P, dout, din, rcp, rcp32, dsum, Pc, pstep);
 }
 
 // The same at many blocks (B >= kWidePrefixB), in four steps that read and
@@ -94,10 +94,12 @@ __global__ void __launch_bounds__(kThreads) k_prefix_dense(const int32_t *__rest
 //      column prefixes from the sums of the chunks above;
 //   4. k_wide_finish: pivots, din, reciprocals, the column degrees' share of L.
 // Prefix rows and DL at B = 4096: 179 -> 94 us (rows 41, sums 15, columns 28,
-// finish 9; 64 MB read twice, 134 MB written).  The line: a commit with nothing
-// moved takes, with a warp per block and with these, 55 and 57 us at B = 1024,
-// 60 and 62 at 1300, 70 and 63 at 1600, 66 and 68 at 2047, 106 and 93 at 3000.
-constexpr int kWidePrefixB = 1400;
+// finish 9; 64 MB read twice, 134 MB written).  The line: labels of a 200k-vertex
+// graph set from outside and committed, few of them changed, take, with a warp
+// per block and with these, 83 and 98 us at B = 1000, 98 and 104 at 1500, 110
+// and 105 at 1600, 104 and 104 at 1800, 111 and 109 at 2000, 125 and 123 at
+// 2500, 150 and 137 at 3000.
+constexpr int kWidePrefixB = 1600;
 constexpr int kColChunk = 256;
 constexpr int kRowIn = 8;  // counts of a row in flight per thread
 
@@ -597,7 +599,7 @@ __global__ void __launch_bounds__(kCommitThreads) k_commit_small(SmallCommit a) 
     cluster_sync();
     __int128 fix = 0;
     for (int u = tid >> 5; u < B; u += nt >> 5) {
-        prefix_block(a.M, B, u, a.P, a.dout, a.din, a.rcp, a.rcp32, a.dsum, a.Pc, a.pstep);
+        prefix_block<false>(a.M, B, u, a.P, a.dout, a.din, a.rcp, a.rcp32, a.dsum, a.Pc, a.pstep);
         if (lane == 0) fix -= a.T[a.dout[u]] + a.T[a.din[u]];
     }
     for (int i = tid; i < B * B; i += nt) fix += a.T[__ldcg(&a.M[i])];

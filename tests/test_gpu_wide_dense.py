@@ -37,3 +37,14 @@ def test_growing_a_dense_model_past_the_line():
         b = (np.arange(g.n) * 7 % B).astype(np.int32)
         P.sbp_set_assignment(m.h, B, b)
         check_blockmodel(m, O.Model(G, B, b))
+
+
+@pytest.mark.parametrize("B", [1599, 1600, 1601])
+def test_both_sides_of_the_line(B):
+    test_wide_prefix_matches_oracle(B)
+    # and the column sums of a model that grows past it
+    g = dcsbm(3000, 30_000, 10, 2.5, 1, 100, 4.0, seed=2)
+    m = P.Model(P.Graph(g.n, g.src, g.dst), 700, (np.arange(g.n) % 700).astype(np.int32))
+    b = (np.arange(g.n) * 7 % B).astype(np.int32)
+    P.sbp_set_assignment(m.h, B, b)
+    check_blockmodel(m, O.Model(O.Graph(g.n, g.src, g.dst), B, b))
