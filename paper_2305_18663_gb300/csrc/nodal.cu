@@ -875,17 +875,24 @@ __global__ void __launch_bounds__(kBigThreads) k_eval_cta(DecideArgs a, int bin,
 #ifndef SBP_BATCH0_MIN_BLOCKS
 #define SBP_BATCH0_MIN_BLOCKS 4
 #endif
-// CTAs per SM (register budgets) of the batch kernels: the exact form, whose
-// 128-bit sums spill at the FP32 form's budgets, does better with one fewer
-// (three sweeps of 200k vertices: 1342 us at 4 and 3, 1294 at 3 and 3, 1172 at
-// 3 and 2)
-constexpr int batch_min_blocks(int mode, bool dl32) {
-    return mode == 0 ? (dl32 ? SBP_BATCH0_MIN_BLOCKS : 3) : (dl32 ? SBP_DECIDE_MIN_BLOCKS : 2);
+// CTAs of eight warps per SM (register budgets) of the batch kernels.  MANY:
+// the FP32 form's budgets also for the exact form, whose 128-bit sums spill
+// there.  Fewer warps without spills are the faster form in a pass of one or
+// two waves, more warps in a long one over the first group (its lines are in
+// launch_groups).
+constexpr int batch_min_blocks(int mode, bool dl32, bool many) {
+    const bool most = dl32 || many;
+    return mode == 0 ? (most ? SBP_BATCH0_MIN_BLOCKS : 3) : (most ? SBP_DECIDE_MIN_BLOCKS : 2);
 }
-// edge ends per sub-batch (33..128): 768 keep a CTA at 64 KB at B = 316, so
-// that three fit an SM (three sweeps of the 1M-vertex graph: 3699 us at 1024,
-// 3630 at 768, 3689 at 640 and at 512)
-constexpr int kBatchEdges = 768;
+// edge ends per sub-batch (33..128).  Fewer (kBatchFewer) leave more shared
+// memory to CTAs and to the L1 cache, which the long chains of the exact form
+// and of sparse rows use; at few blocks there is room anyway, at many the
+// counts take it all the same, and rows of 80 edges need more sub-batches.
+// 1024 and 768 in us, B = 50 / 316 / 1000: 600,000 vertices of 40 edges, sparse
+// 633 and 614 / 711 and 642 / 742 and 792; dense 594 and 581 / 620 and 587 /
+// 677 and 687; of 80 edges, dense 843 and 883 / 919 and 951 / 1061 and 1098;
+// 60,000 vertices of 67 edges, sparse 145 and 144 / 181 and 164 / 184 and 202.
+constexpr int kBatchEdges = 1024, kBatchFewer = 768;
 constexpr int kBatchEdges0 = SBP_BATCH0_EDGES;  // ... for rows of at most 32
 constexpr int kDirectMaxB = 2048;  // direct-mapped per-warp counts up to this B
 
@@ -900,9 +907,6 @@ struct BatchWarpT {
     double fb[32];
 };
 
-template <int MODE>
-using BatchWarp = BatchWarpT<MODE == 0 ? kBatchEdges0 : kBatchEdges>;
-
 
 __device__ __forceinline__ float fix48_to_float(long long v) {
     return fmaf((float)(int)(v >> 32), 0x1p-16f, (float)(unsigned)(v & 0xffffffffu) * 0x1p-48f);
@@ -916,11 +920,10 @@ __device__ __forceinline__ double fix48_to_double(long long v) {
 // whole rows); MODE 1: rows of 33..128 edges (aggregated per mover in a
 // direct-mapped count array of B entries, dcnt, with its touch list dlist,
 // which follow the warp's BatchWarp in shared memory).  Movers are taken in
-// sub-batches of at most kBatchEdges edge ends.
-template <int MODE, bool DL32>
-__device__ __forceinline__ void batch_movers(const DecideArgs &a, BatchWarp<MODE> &W, unsigned *dcnt, int *dlist,
+// sub-batches of at most kEdges edge ends.
+template <int MODE, bool DL32, int kEdges>
+__device__ __forceinline__ void batch_movers(const DecideArgs &a, BatchWarpT<kEdges> &W, unsigned *dcnt, int *dlist,
                                              const int nv, int v, int s, uint64_t w2, Counts &c) {
-    constexpr int kEdges = MODE == 0 ? kBatchEdges0 : kBatchEdges;
     const int lane = threadIdx.x & 31;
     const GraphDev &g = a.g;
     const ModelDev &md = a.md;
@@ -946,7 +949,7 @@ __device__ __forceinline__ void batch_movers(const DecideArgs &a, BatchWarp<MODE
         if (lane >= o) incl += y;
     }
     const int first = incl - k;
-    // sub-batches of whole rows with at most kBatchEdges edge ends
+    // sub-batches of whole rows with at most kEdges edge ends
     for (int sa = 0; sa < nv;) {
     const int fs = __shfl_sync(0xffffffffu, first, sa);
     const unsigned fit = __ballot_sync(0xffffffffu, lane >= sa && lane < nv && incl - fs <= kEdges);
@@ -1214,10 +1217,11 @@ __device__ __forceinline__ void batch_movers(const DecideArgs &a, BatchWarp<MODE
 // per vertex), keep the movers in a queue of two slots per lane (position p
 // in lane p % 32, slot p / 32) and evaluate them 32 at a time, so that the
 // proposals' load chains overlap other warps' evaluation.
-template <int MODE, bool DL32, bool FUSED>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, batch_min_blocks(MODE, DL32)) k_eval_batch(DecideArgs a, int bin, int warp_bytes) {
+template <int MODE, bool DL32, bool FUSED, bool MANY, int EDGES>
+__global__ void __launch_bounds__(kWarpsPerCta * 32, batch_min_blocks(MODE, DL32, MANY))
+    k_eval_batch(DecideArgs a, int bin, int warp_bytes) {
     extern __shared__ __align__(16) unsigned char bsm[];
-    using BW = BatchWarp<MODE>;
+    using BW = BatchWarpT<EDGES>;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
     BW &W = *reinterpret_cast<BW *>(bsm + (size_t)wid * warp_bytes);
     unsigned *dcnt = reinterpret_cast<unsigned *>(bsm + (size_t)wid * warp_bytes + sizeof(BW));
@@ -1239,7 +1243,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, batch_min_blocks(MODE, DL32
             const int nv = (int)(count - first_i < 32 ? count - first_i : 32);
             Mover mv{0, -1, 0ull};
             if (lane < nv) mv = mlist[first_i + lane];
-            batch_movers<MODE, DL32>(a, W, dcnt, dlist, nv, mv.v, mv.s, mv.w2, c);
+            batch_movers<MODE, DL32, EDGES>(a, W, dcnt, dlist, nv, mv.v, mv.s, mv.w2, c);
         }
         flush_counts_warp(md, c, 0ull);
     } else {
@@ -1288,7 +1292,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, batch_min_blocks(MODE, DL32
                 const uint64_t w2 = q0w;
                 q0v = q1v; q0s = q1s; q0w = q1w;
                 nq -= nv;
-                batch_movers<MODE, DL32>(a, W, dcnt, dlist, nv, v, s, w2, c);
+                batch_movers<MODE, DL32, EDGES>(a, W, dcnt, dlist, nv, v, s, w2, c);
             }
             if (!more) break;
         }
@@ -1552,11 +1556,11 @@ int sm_count() {
 // At 2^18 edges (10,000 vertices, exact form) the fork costs what it gains:
 // 118 and 120 us.
 static constexpr int64_t kSideStreamEdges = int64_t(1) << 19;
+static constexpr int64_t kSideFirstGroup = 8192;
 
 // three streams for kernels that may run together: the model's own one (for
 // the longest) and its side streams, forked here and joined by join_side (all
 // the model's own on smaller graphs)
-static constexpr int64_t kSideFirstGroup = 8192;
 int fork_side(sbp_model *m, cudaStream_t st[3]) {
     st[0] = st[1] = st[2] = m->stream;
     if (m->g->m < kSideStreamEdges) return SBP_OK;
@@ -1654,15 +1658,15 @@ int cta_table(sbp_model *m, int cap, int sms, int *grid, size_t *smem, unsigned 
     return SBP_OK;
 }
 
+// Warps of a CTA of the kernels with direct-mapped counts: half as many where
+// eight warps' counts would leave one CTA an SM (B > 1022).
+int direct_warps(int B) { return (2 * B + 4) * 4 * kWarpsPerCta <= 64 * 1024 ? kWarpsPerCta : kWarpsPerCta / 2; }
+
 // the evaluation kernels of the three degree groups: after k_propose, or
 // (FUSED) drawing the proposals themselves
 template <bool DL32, bool FUSED>
 int launch_groups(sbp_model *m, const DecideArgs &a, int sms, const cudaStream_t st[3]) {
     const sbp_graph *g = m->g;
-// Warps of a CTA of the kernels with direct-mapped counts: half as many where
-// eight warps' counts would leave one CTA an SM (B > 1022).
-int direct_warps(int B) { return (2 * B + 4) * 4 * kWarpsPerCta <= 64 * 1024 ? kWarpsPerCta : kWarpsPerCta / 2; }
-
     const int B = m->B;
     // one launch of k_eval_table over list `bin`, tables of 2^cap_log2 slots
     auto tables = [&](int bin, int cap_log2, cudaStream_t on) -> int {
@@ -1707,24 +1711,58 @@ int direct_warps(int B) { return (2 * B + 4) * 4 * kWarpsPerCta <= 64 * 1024 ? k
         if (g->n_wide > 0) SBP_TRY(tables(3, 11, st[2]));
         if (g->n_mid > 0) SBP_TRY(tables(2, 10, st[0]));
     }
+    // The batch kernels, with no more CTAs than the group has batches of 32
+    // vertices.  Up to 10 KB a warp (B = 460), CTAs of eight warps, as many as
+    // registers hold; three where shared memory holds two, the last ones
+    // following and evening out the end (300,000 vertices with a heavy tail, B =
+    // 330, FP32 form: 310 us, with two 355).  Above, as many CTAs of eight warps
+    // as shared memory holds, if two (to B = 1500), else of four: 600,000
+    // vertices of 40 edges, three CTAs of four warps and these, in us: B = 500
+    // 643 and 425, 1000 561 and 422.
+    auto batch = [&](auto kern, int bin, int min_blocks, size_t bytes, cudaStream_t on) -> int {
+        const int wb = (int)((bytes + 15) / 16 * 16);
+        auto held = [&](int nw) { return (int)(size_t(228) * 1024 / ((size_t)wb * nw + 1024)); };
+        const int nw = wb <= 10 * 1024 || held(kWarpsPerCta) >= 2 ? kWarpsPerCta : kWarpsPerCta / 2;
+        int ctas = min_blocks * kWarpsPerCta / nw;
+        if (wb > 10 * 1024) ctas = std::min(ctas, held(nw));
+        else if (held(nw) < 3) ctas = 3;
+        const int64_t per_cta = 32 * nw, want = (g->bin[bin + 2] - g->bin[bin + 1] + per_cta - 1) / per_cta;
+        const size_t smem = (size_t)wb * nw;
+        SBP_TRY(ensure_dyn_smem((const void *)kern, smem));
+        kern<<<(int)std::min<int64_t>(want, (int64_t)sms * ctas), nw * 32, smem, on>>>(a, bin, wb);
+        SBP_LAUNCHED();
+        return SBP_OK;
+    };
+    // The exact form's budgets (FP32 form's, own): a long pass over the first
+    // group wants the warps; so does one over the second at few blocks, in us:
+    // 300,000 vertices with a heavy tail, B = 50 (first group's budget) 194 and
+    // 227, 307 and 349, 200,000 1238 and 1193 (three sweeps); 600,000, B = 50
+    // (second group's) 529 and 656, of 80 edges 511 and 546, of 40 355 and 336.
+    constexpr bool kTwo = !DL32;
+    const bool many0 = g->n >= (int64_t(1) << 18), many1 = B <= 100 && g->m >= 10 * (int64_t(1) << 20);
     // movers with k <= 32: batches of 32 per warp
     if (g->bin[2] > g->bin[1]) {
-        const int wb = (int)((sizeof(BatchWarp<0>) + 15) / 16 * 16);
-        const size_t smem = (size_t)wb * kWarpsPerCta;
-        SBP_TRY(ensure_dyn_smem((const void *)k_eval_batch<0, DL32, FUSED>, smem));
-        k_eval_batch<0, DL32, FUSED><<<sms * batch_min_blocks(0, DL32), kWarpsPerCta * 32, smem, st[0]>>>(a, 0, wb);
-        SBP_LAUNCHED();
+        constexpr int E = kBatchEdges0;
+        const size_t bytes = sizeof(BatchWarpT<E>);
+        if (kTwo && many0)
+            SBP_TRY(batch(k_eval_batch<0, DL32, FUSED, kTwo, E>, 0, batch_min_blocks(0, DL32, true), bytes, st[0]));
+        else
+            SBP_TRY(batch(k_eval_batch<0, DL32, FUSED, false, E>, 0, batch_min_blocks(0, DL32, false), bytes, st[0]));
     }
     // movers with 33 <= k <= 128: batches with direct-mapped counts while B is
     // small, otherwise one warp each with a 256-slot table
     if (g->bin[3] > g->bin[2]) {
         if (B <= kDirectMaxB) {
-            const int wb = (int)((sizeof(BatchWarp<1>) + 4 * (size_t)B + 4 * kWarpDeg + 15) / 16 * 16);
-            const int nwarps = wb <= 10 * 1024 ? kWarpsPerCta : kWarpsPerCta / 2;
-            const size_t smem = (size_t)wb * nwarps;
-            SBP_TRY(ensure_dyn_smem((const void *)k_eval_batch<1, DL32, FUSED>, smem));
-            k_eval_batch<1, DL32, FUSED><<<sms * batch_min_blocks(1, DL32), nwarps * 32, smem, st[1]>>>(a, 1, wb);
-            SBP_LAUNCHED();
+            constexpr int E = kBatchEdges, F = kBatchFewer;
+            const size_t bytes = 4 * (size_t)B + 4 * kWarpDeg;
+            const int few = batch_min_blocks(1, DL32, false);
+            if (kTwo && many1)
+                SBP_TRY(batch(k_eval_batch<1, DL32, FUSED, kTwo, E>, 1, batch_min_blocks(1, DL32, true),
+                              bytes + sizeof(BatchWarpT<E>), st[1]));
+            else if ((kTwo || !m->dense) && B >= 64 && B <= 320)
+                SBP_TRY(batch(k_eval_batch<1, DL32, FUSED, false, F>, 1, few, bytes + sizeof(BatchWarpT<F>), st[1]));
+            else
+                SBP_TRY(batch(k_eval_batch<1, DL32, FUSED, false, E>, 1, few, bytes + sizeof(BatchWarpT<E>), st[1]));
         } else {
             SBP_TRY(tables(1, 8, st[1]));
         }

@@ -1,7 +1,8 @@
 """Where the one-launch pass and the one-launch commit end: on both sides of
 each line the call takes the form it should (seen in the number of kernels it
 launches) and gives what the general kernels give.  Labels, counts, degrees,
-statistics and DL are compared exactly."""
+statistics and DL are compared exactly.  The forms of the batch kernels (CTA
+shapes, register budgets and sub-batches by size) decide alike."""
 import numpy as np
 import pytest
 
@@ -89,3 +90,35 @@ def test_commit_form_and_result(n, e, B):
         P.sbp_set_assignment(full.h, B, lab)
         _same(one, full)
         sweep(sw)
+
+
+def _device_graph(n, e, seed):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    src = torch.randint(0, n, (e,), generator=gen, device="cuda", dtype=torch.int32)
+    return P.Graph(n, src, torch.randint(0, n, (e,), generator=gen, device="cuda", dtype=torch.int32))
+
+
+# rows on both sides of 32 edges; B at the edges of the sub-batches' range, of
+# the CTA shapes and of the kernels; then the exact form's other budgets
+@pytest.mark.parametrize("n,e,Bs", [
+    (30_000, 600_000, (63, 64, 320, 321, 460, 461, 1500, 1550, 2048)),
+    (1 << 18, 4_400_000, (50,)),
+    (300_000, 10 << 20, (100, 101)),
+])
+def test_batch_kernel_forms_decide_alike(n, e, Bs):
+    pg = _device_graph(n, e, seed=n)
+    for B in Bs:
+        b = random_labels(n, B, seed=B)
+        models = [P.Model(pg, B, b, P.Params.default(seed=2, dl_fp32=f, dense_max_B=d)) for f in (1, 0) for d in (4096, 1)]
+        parts = P.Model(pg, B, b, P.Params.default(seed=2))  # its movers come from lists
+        for sw in range(2):
+            stats = [m.sweep(sw) for m in models]
+            for lo, hi in ((0, n // 3), (n // 3, n)):
+                P.sbp_nodal_decide(parts.h, sw, lo, hi)
+            stats.append(P.sbp_commit(parts.h))
+            assert stats[0].n_moves > n // 2 and stats[0].n_accepted > 0
+            for m, st in zip(models[1:] + [parts], stats[1:]):
+                assert np.array_equal(m.assignment(), models[0].assignment())
+                assert (st.n_moves, st.n_accepted, st.n_entries) == \
+                       (stats[0].n_moves, stats[0].n_accepted, stats[0].n_entries)
+                assert st.dl_after == stats[0].dl_after
