@@ -742,14 +742,26 @@ extern "C" int sbp_get_blockmodel_coo(const sbp_model_t *m, int64_t capacity, in
         SBP_CUDA(cudaMemcpy(rp.data(), m->sp.rp, rp.size() * 4, cudaMemcpyDeviceToHost));
         if (m->sp.slack) SBP_CUDA(cudaMemcpy(re.data(), m->sp.re, re.size() * 4, cudaMemcpyDeviceToHost));
         else std::copy(rp.begin() + 1, rp.end(), re.begin());
-        const uint32_t z = re[(size_t)B - 1];
+        std::vector<uint32_t> first((size_t)B);  // of row r among all nonzeros
+        uint32_t z = 0;
+        for (int64_t r = 0; r < B; ++r) {
+            first[(size_t)r] = z;
+            z += re[(size_t)r] - rp[(size_t)r];
+        }
+        *nnz = z;
+        if ((int64_t)z > capacity) return fail(SBP_EINVAL, "sbp_get_blockmodel_coo: capacity too small");
         std::vector<int32_t> rc((size_t)z), rv((size_t)z);
         if (z > 0) {
-            SBP_CUDA(cudaMemcpy(rc.data(), m->sp.rc, (size_t)z * 4, cudaMemcpyDeviceToHost));
-            SBP_CUDA(cudaMemcpy(rv.data(), m->sp.rv, (size_t)z * 4, cudaMemcpyDeviceToHost));
+            // rows with slack between them are packed first: of a graph with
+            // many edges a block, most slots are empty
+            const int32_t *drc = m->sp.rc, *drv = m->sp.rv;
+            if (m->sp.slack) SBP_TRY(pack_sparse_rows(m, first.data(), &drc, &drv));
+            SBP_CUDA(cudaMemcpyAsync(rc.data(), drc, (size_t)z * 4, cudaMemcpyDeviceToHost, m->stream));
+            SBP_CUDA(cudaMemcpyAsync(rv.data(), drv, (size_t)z * 4, cudaMemcpyDeviceToHost, m->stream));
+            SBP_CUDA(cudaStreamSynchronize(m->stream));
         }
         for (int64_t r = 0; r < B; ++r)
-            for (uint32_t i = rp[(size_t)r]; i < re[(size_t)r]; ++i) {
+            for (uint32_t i = first[(size_t)r], e = r + 1 < B ? first[(size_t)r + 1] : z; i < e; ++i) {
                 k.push_back(r * B + rc[i]);
                 c.push_back(rv[i]);
             }

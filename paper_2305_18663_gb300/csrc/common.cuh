@@ -621,6 +621,9 @@ int xlogx_table(int64_t need, const __int128 **table, int64_t *size);
 int ensure_sparse_capacity(sbp_model *m, int32_t B);
 int rebuild_sparse(sbp_model *m, bool after_pass, bool *dl_done, int *n_parts);
 int build_sparse_rows(sbp_model *m, int *n_parts);  // sparse_rows.cu
+// the rows' columns and counts without the slack between them, row r from
+// first[r] (host array), in scratch of the model
+int pack_sparse_rows(const sbp_model *m, const uint32_t *first, const int32_t **rc, const int32_t **rv);
 constexpr int64_t kSparseScratch = 20000;  // words: the small rebuild's lengths and sums, or a cluster's exchange
 void free_sparse(sbp_model *m);
 

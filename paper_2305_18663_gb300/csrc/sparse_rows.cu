@@ -581,6 +581,22 @@ __global__ void __launch_bounds__(kRowBigThreads) k_rows_big(Rows a) {
     row_partial(a.parts + blockIdx.x, fix, fb);
 }
 
+// a warp per row: its nonzeros to where they lie without slack
+__global__ void __launch_bounds__(kT) k_rows_pack(const uint32_t *__restrict__ rp, const uint32_t *__restrict__ re,
+                                                  const uint32_t *__restrict__ first, int B,
+                                                  const int32_t *__restrict__ rc, const int32_t *__restrict__ rv,
+                                                  int32_t *__restrict__ rc_out, int32_t *__restrict__ rv_out) {
+    const int64_t nw = ((int64_t)gridDim.x * kT) >> 5;
+    for (int64_t r = ((int64_t)blockIdx.x * kT + threadIdx.x) >> 5; r < B; r += nw) {
+        const uint32_t from = rp[r], len = re[r] - from, to = first[r];
+#pragma unroll 4
+        for (uint32_t i = threadIdx.x & 31; i < len; i += 32) {
+            rc_out[to + i] = rc[from + i];
+            rv_out[to + i] = rv[from + i];
+        }
+    }
+}
+
 int row_grid(int64_t work, int per_block, int cap) {
     const int64_t g = (work + per_block - 1) / per_block;
     return (int)(g < 1 ? 1 : g > cap ? cap : g);
@@ -694,6 +710,17 @@ int build_sparse_rows(sbp_model *m, int *n_parts) {
     if (rc != SBP_OK) return rc;
     if (rj != SBP_OK) return rj;
     S.slack = true;
+    return SBP_OK;
+}
+
+// (the labels and the slot cursors of the build are done with after it)
+int pack_sparse_rows(const sbp_model *m, const uint32_t *first, const int32_t **rc, const int32_t **rv) {
+    const sbp_model::Sparse &S = m->sp;
+    SBP_CUDA(cudaMemcpyAsync(S.rcur, first, (size_t)m->B * 4, cudaMemcpyHostToDevice, m->stream));
+    k_rows_pack<<<row_grid(m->B, kT / 32, kSms * 8), kT, 0, m->stream>>>(S.rp, S.re, S.rcur, m->B, S.rc, S.rv, S.lo, S.li);
+    SBP_LAUNCHED();
+    *rc = S.lo;
+    *rv = S.li;
     return SBP_OK;
 }
 

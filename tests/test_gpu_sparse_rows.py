@@ -57,3 +57,24 @@ def test_sweeps_and_merges_on_the_rows(n, B):
     assert P.sbp_merge_blocks(m.h, 7, B // 3) == (oB, orounds)
     assert np.array_equal(m.assignment(), om.assignment())
     check_blockmodel(m, om)
+
+
+@pytest.mark.parametrize("n,B", [(1500, 1025), (40_000, 33_000)])
+def test_reading_the_nonzeros_leaves_the_rows_as_they_are(n, B):
+    # many edges a nonzero (repeats), so most slots of the rows are empty; the
+    # packing uses scratch of the build
+    g = _graph(n, False, seed=n)
+    pg, om = P.Graph(g.n, g.src, g.dst), O.Model(O.Graph(g.n, g.src, g.dst), B, (np.arange(n) % B).astype(np.int32))
+    read, not_read = (P.Model(pg, B, om.assignment(), P.Params.default(seed=1, dense_max_B=1)) for _ in range(2))
+    launches = P.sbp_kernel_launches()
+    keys, cnt = read.coo()
+    assert P.sbp_kernel_launches() > launches  # packed on the device, not read with the slack
+    okeys, ocnt = om.coo()
+    assert np.array_equal(keys, okeys) and np.array_equal(cnt, ocnt)
+    for sw in range(2):
+        a, c = read.sweep(sw), not_read.sweep(sw)
+        assert a.as_dict() == c.as_dict()
+        read.coo()
+    om.set_b(B, read.assignment())
+    check_blockmodel(read, om)
+    check_blockmodel(not_read, om)
