@@ -286,11 +286,13 @@ int sbp_philox_check(uint64_t c0, uint64_t c1, uint64_t c2, uint64_t c3, uint64_
  * II-B; Alg. 1, 2) and ends with the same assignment, B, DL and sweep count.
  * A graph whose next phase starts at B <= 1024 on a dense model and merges
  * to B <= max_B hands its search to a persistent launch over all waiting
- * graphs: a CTA runs that graph's phases (start state, merge rounds, sweeps
- * with the convergence test, compaction, bracket update) until the search
- * ends or a phase is out of those bounds.  This overlaps with the
- * per-graph work (set-up, larger-B phases) that `workers` host threads
- * drive on their graphs' streams.  Graphs are admitted in input order
+ * graphs: a CTA, or while few searches are unfinished a cluster of 2, 4 or 8
+ * CTAs, runs that graph's phases (start state, merge rounds, sweeps with the
+ * convergence test, compaction, bracket update) until the search ends or a
+ * phase is out of those bounds.  (Clusters while all unfinished searches fit
+ * nine tenths of the SMs that way, a server's half of them.)  This overlaps
+ * with the per-graph work (set-up, larger-B phases) that `workers` host
+ * threads drive on their graphs' streams.  Graphs are admitted in input order
  * while their estimated device memory fits mem_fraction of the free
  * memory, and each model is freed when its graph finishes.
  *
@@ -298,10 +300,11 @@ int sbp_philox_check(uint64_t c0, uint64_t c1, uint64_t c2, uint64_t c3, uint64_
  * to (1..1024); max_n: largest graph (vertices) whose searches are batched
  * (a CTA runs a whole search, so the biggest graphs can be better served by
  * the per-graph kernels); dense_max_B: dense/sparse switch of the batch's models
- * (max_B..16384); ctas_per_sm: persistent CTAs per SM (1..8);
- * movers_per_warp: movers a warp of the persistent kernel evaluates at once
- * (1, 2 or 4: 32, 16 or 8 lanes each; fewer when their per-mover count rows
- * would not fit shared memory); mem_fraction: (0, 0.95].  No option changes
+ * (max_B..16384); ctas_per_sm: persistent CTAs per SM (1..8) of the form
+ * with a CTA per search (a cluster has one CTA an SM); movers_per_warp:
+ * movers a warp of the persistent kernel evaluates at once (1, 2 or 4: 32, 16
+ * or 8 lanes each; fewer when their per-mover count rows would not fit shared
+ * memory); mem_fraction: (0, 0.95].  No option changes
  * a result. */
 typedef struct sbp_batch_options {
     int32_t workers;
@@ -367,8 +370,9 @@ int sbp_partition_batch(const sbp_graph_t *const *graphs, int32_t count, const s
  * defaults) and tunes one option at a time, in this order:
  * movers_per_warp {1, 2, 4}, ctas_per_sm {1, 2, 3, 4}, max_B {128, 256,
  * 512, 1024}, max_n {1024, 4096, 16384, 65536}, dense_max_B {1024, 4096};
- * workers (the caller's host threads) and mem_fraction are kept.  A
- * sample runs far from the full batch's load (its host workers are mostly
+ * workers (the caller's host threads) and mem_fraction are kept.  The sample's
+ * searches run in the form (a CTA or a cluster each) in which those of all
+ * `count` graphs would start.  A sample runs far from the full batch's load (its host workers are mostly
  * idle), so options that favour per-graph work can win on it and lose on
  * the whole batch.  *graphs_per_s (may be NULL) receives the best rate on
  * the sample, *trials (may be NULL) the number of timed runs.

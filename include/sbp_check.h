@@ -26,6 +26,16 @@ extern "C" {
 int sbp_bracket_check(const int32_t *B, const double *dl, int32_t count, double reduction, int32_t *out,
                       int32_t *n_bad);
 
+/* *ctas: the CTAs per search of a persistent launch of the batching form
+ * while `unfinished` searches are in a batch call (server: in a server), on a
+ * device of `sms` SMs: 8, 4 or 2 (a cluster per search) or 1.  SBP_EINVAL on
+ * a negative count, sms < 1 or a NULL pointer. */
+int sbp_search_form_check(int64_t unfinished, int32_t sms, int32_t server, int32_t *ctas);
+
+/* Persistent launches of the batching form in this process so far, with one
+ * CTA per search and with a cluster per search (either may be NULL). */
+int sbp_search_launches(int64_t *one_cta, int64_t *clusters);
+
 #ifdef __cplusplus
 }
 #endif

@@ -605,6 +605,8 @@ __global__ void __launch_bounds__(Squad<CLUSTER>::T, CLUSTER ? 1 : 2)
     }
 }
 
+std::atomic<int64_t> g_search_launches[2];  // one CTA per search, a cluster per search
+
 int sm_count_b() {
     static int sms = 0;
     if (!sms) {
@@ -637,18 +639,22 @@ bool batch_phase_eligible(const sbp_model *m, int32_t B_from, int32_t target, in
            target <= kBatchMaxB && batch_graph_ok(m, max_n);
 }
 
-// CTAs (one an SM) for each search of a launch while `active` searches are
-// unfinished and may use `sms` of the SMs: 8, 4 or 2; 1: the queue of
-// one-CTA searches, which a GPU's worth of searches fills.  A search of 5000
+// 8, 4 or 2 CTAs (one an SM) for each search while all unfinished searches fit
+// their share of the SMs so; 1: the queue of one-CTA searches, which a GPU's
+// worth of searches fills.  A batch call's searches may take nine tenths of the
+// chip, the server leaves half of it to its large requests' kernels.  A search of 5000
 // vertices is a chain of a few hundred sweeps that one CTA of eight warps
 // runs alone on its SM: 32 graphs of 500 to 5000 vertices took 327 ms so, and
 // take 117 ms on clusters (4 CTAs each, 8 once half of them are done); 1200
 // of them take 1.7 s either way.
-int batch_cluster(int64_t active, int sms) {
+int batch_cluster(int64_t unfinished, int sms, bool server) {
+    const int share = server ? sms / 2 : sms * 9 / 10;
     for (int c = 8; c > 1; c /= 2)
-        if (active * c <= sms) return c;
+        if (unfinished * c <= share) return c;
     return 1;
 }
+
+int batch_sms() { return sm_count_b(); }
 
 int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, const BatchTuning &tune, int cluster,
                   cudaStream_t st) {
@@ -742,7 +748,7 @@ int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, cons
     const int group_words = 2 * max_B + 4;
     const bool cl = cluster > 1;
     const int warps = (cl ? kClusterThreads : kBatchThreads) / 32;
-    int V = tune.movers_per_warp == 4 ? (cl ? 2 : 4) : tune.movers_per_warp == 2 ? 2 : 1;
+    int V = tune.movers_per_warp == 4 ? 4 : tune.movers_per_warp == 2 ? 2 : 1;
     while (V > 1 && (size_t)warps * V * group_words * 4 > (cl ? kClusterSmemCap : kBatchSmemCap)) V /= 2;
     // the merge rounds' and the compaction's arrays share that memory
     const size_t smem = std::max((size_t)warps * V * group_words * 4, (size_t)blk_cap * (kMergeApplyBytes + 4));
@@ -754,11 +760,14 @@ int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, cons
         return launch_cluster(kern, cl ? cluster : 1, warps * 32, smem, st, cl ? nj : grid, (const BatchJob *)d_jobs, nj,
                               d_queue, group_words, blk_cap, xch);
     };
+    g_search_launches[cl ? 1 : 0].fetch_add(1, std::memory_order_relaxed);
     if (cl) {
         if (p.dl_fp32)
-            SBP_TRY(V == 2 ? launch(k_batch_search<true, 16, true>) : launch(k_batch_search<true, 32, true>));
+            SBP_TRY(V == 4 ? launch(k_batch_search<true, 8, true>)
+                           : V == 2 ? launch(k_batch_search<true, 16, true>) : launch(k_batch_search<true, 32, true>));
         else
-            SBP_TRY(V == 2 ? launch(k_batch_search<false, 16, true>) : launch(k_batch_search<false, 32, true>));
+            SBP_TRY(V == 4 ? launch(k_batch_search<false, 8, true>)
+                           : V == 2 ? launch(k_batch_search<false, 16, true>) : launch(k_batch_search<false, 32, true>));
     } else if (p.dl_fp32) {
         SBP_TRY(V == 4 ? launch(k_batch_search<true, 8, false>)
                        : V == 2 ? launch(k_batch_search<true, 16, false>) : launch(k_batch_search<true, 32, false>));
@@ -824,6 +833,18 @@ extern "C" int sbp_bracket_check(const int32_t *B, const double *dl, int32_t cou
         if (!same) ++bad;
     }
     *n_bad = bad;
+    return SBP_OK;
+}
+
+extern "C" int sbp_search_form_check(int64_t unfinished, int32_t sms, int32_t server, int32_t *ctas) {
+    if (!ctas || unfinished < 0 || sms < 1) return sbp::fail(SBP_EINVAL, "sbp_search_form_check: bad argument");
+    *ctas = sbp::batch_cluster(unfinished, sms, server != 0);
+    return SBP_OK;
+}
+
+extern "C" int sbp_search_launches(int64_t *one_cta, int64_t *clusters) {
+    if (one_cta) *one_cta = sbp::g_search_launches[0].load();
+    if (clusters) *clusters = sbp::g_search_launches[1].load();
     return SBP_OK;
 }
 

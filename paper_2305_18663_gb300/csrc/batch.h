@@ -62,9 +62,13 @@ bool batch_phase_eligible(const sbp_model *m, int32_t B_from, int32_t target, in
 // model is in the state the per-graph kernels would leave and each record
 // and its slots hold the search as the kernel left it.  The launch's
 // scratch is freed in stream order.  cluster: CTAs per search, from
-// batch_cluster.
+// batch_cluster (1: the CTAs take searches from a queue).
 int batch_enqueue(const std::vector<BatchSpec> &specs, const sbp_params &p, const BatchTuning &tune, int cluster,
                   cudaStream_t st);
-int batch_cluster(int64_t active, int sms);
+
+// CTAs per search while `unfinished` searches are in the batch (or server), on
+// a device of `sms` SMs
+int batch_cluster(int64_t unfinished, int sms, bool server);
+int batch_sms();
 
 }  // namespace sbp

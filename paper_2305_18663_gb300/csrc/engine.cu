@@ -117,6 +117,9 @@ struct Engine {
     // oldest request (the server: requests finish closer to arrival order,
     // which keeps the median latency down when the device is saturated)
     bool oldest_first = false;
+    // searches that count as unfinished beside the engine's own when the form
+    // of a launch is chosen (the tuner's sample stands for a larger batch)
+    int64_t others = 0;
     // host-mapped search records with their label slots, reused by size once
     // their graph is done
     std::mutex xfer_mu;
@@ -465,9 +468,7 @@ int Engine::loop() {
             inflight.push_back(slot);
             ended.clear();
             for (int64_t idx : L.take) ended.push_back(items[(size_t)idx].get());
-            // a batch call's searches may take most of the chip, the server
-            // leaves half of it to its large requests' kernels
-            const int cluster = batch_cluster(running + (int64_t)(items.size() - next_admit), oldest_first ? 76 : 136);
+            const int cluster = batch_cluster(running + (int64_t)(items.size() - next_admit) + others, batch_sms(), oldest_first);
             lk.unlock();
             // each graph's search goes to its mapped record and label slots
             std::vector<BatchSpec> specs(L.take.size());
@@ -571,9 +572,11 @@ int batch_options(const sbp_batch_options *o, BatchOptions &opt) {
 using sbp::Engine;
 using sbp::fail;
 
-extern "C" int sbp_partition_batch(const sbp_graph_t *const *graphs, int32_t count, const sbp_params *p,
-                                   const sbp_batch_options *o, int32_t *const *b_out, sbp_batch_result *res,
-                                   sbp_batch_stats *stats) {
+namespace sbp {
+namespace {
+
+int partition_batch(const sbp_graph_t *const *graphs, int32_t count, const sbp_params *p, const sbp_batch_options *o,
+                    int32_t *const *b_out, sbp_batch_result *res, sbp_batch_stats *stats, int64_t others) {
     if (count < 0 || (count > 0 && (!graphs || !res))) return fail(SBP_EINVAL, "sbp_partition_batch: NULL argument");
     for (int i = 0; i < count; ++i)
         if (!graphs[i]) return fail(SBP_EINVAL, "sbp_partition_batch: NULL graph " + std::to_string(i));
@@ -584,6 +587,7 @@ extern "C" int sbp_partition_batch(const sbp_graph_t *const *graphs, int32_t cou
     sbp::BatchOptions opt;
     SBP_TRY(sbp::batch_options(o, opt));
     Engine e;
+    e.others = others;
     SBP_TRY(e.init(prm, opt, false));
     for (int i = 0; i < count; ++i) e.submit(graphs[i], b_out ? b_out[i] : nullptr);
     {
@@ -603,9 +607,19 @@ extern "C" int sbp_partition_batch(const sbp_graph_t *const *graphs, int32_t cou
     return SBP_OK;
 }
 
+}  // namespace
+}  // namespace sbp
+
+extern "C" int sbp_partition_batch(const sbp_graph_t *const *graphs, int32_t count, const sbp_params *p,
+                                   const sbp_batch_options *o, int32_t *const *b_out, sbp_batch_result *res,
+                                   sbp_batch_stats *stats) {
+    return sbp::partition_batch(graphs, count, p, o, b_out, res, stats, 0);
+}
+
 // ---------------------------------------------------------------------------
 // autotuner of the batching form: coordinate search over the options, each
-// candidate timed on the same sample of graphs, every result checked equal
+// candidate timed on the same sample of graphs (its launches in the form that
+// the whole batch starts in), every result checked equal
 
 extern "C" int sbp_autotune_batch(const sbp_graph_t *const *graphs, int32_t count, const sbp_params *p,
                                   int32_t sample, int32_t start, sbp_batch_options *best, double *graphs_per_s,
@@ -633,7 +647,7 @@ extern "C" int sbp_autotune_batch(const sbp_graph_t *const *graphs, int32_t coun
     int ntr = 0;
     auto run = [&](const sbp_batch_options &o, double *rate) -> int {
         const auto t0 = std::chrono::steady_clock::now();
-        SBP_TRY(sbp_partition_batch(pick.data(), ns, p, &o, nullptr, res.data(), nullptr));
+        SBP_TRY(sbp::partition_batch(pick.data(), ns, p, &o, nullptr, res.data(), nullptr, count - ns));
         const double s = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         ++ntr;
         if (!have_ref) {
