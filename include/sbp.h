@@ -139,8 +139,10 @@ int sbp_default_params(sbp_params *p);
  * device pointers) onto the current CUDA device: CSR of out-edges and CSR
  * of in-edges, each row ascending by neighbour id, duplicates kept,
  * self-loops kept (listed in both rows of their vertex).  The graph is the
- * "Graph G" input of Alg. 1-2.  Errors: SBP_EINVAL for n < 1, m < 0,
- * m >= 2^30 or an id outside [0, n); SBP_ENOMEM. */
+ * "Graph G" input of Alg. 1-2.  The graph holds 24 bytes of device memory an
+ * edge and 16 a vertex (4 more a self-loop); the load sorts in that memory and
+ * needs another 16 bytes a vertex and 5 MB until it returns.  Errors:
+ * SBP_EINVAL for n < 1, m < 0, m >= 2^30 or an id outside [0, n); SBP_ENOMEM. */
 int sbp_load_graph(int64_t n, int64_t m, const int32_t *src, const int32_t *dst, sbp_graph_t **out);
 
 int sbp_graph_info(const sbp_graph_t *g, int64_t *n, int64_t *m);

@@ -86,19 +86,17 @@ __global__ void __launch_bounds__(kT) k_out_rows(const K *__restrict__ keys, int
     }
 }
 
-// in-row position j holds out-edge e = ival[j].  The sort is stable and the
-// out-rows are ascending, so in-rows are ascending too and the k-th copy of
-// a repeated edge is paired with its k-th copy.
+// in-row position j holds out-edge e = ival[j] (its keys and values are idst
+// and tw_io).  The sort is stable and the out-rows are ascending, so in-rows
+// are ascending too and the k-th copy of a repeated edge is paired with its
+// k-th copy.
 __global__ void __launch_bounds__(kT) k_in_rows(const uint32_t *__restrict__ ikey, const uint32_t *__restrict__ ival,
                                                 const int32_t *__restrict__ esrc, int64_t m, int32_t *__restrict__ ic,
-                                                int32_t *__restrict__ idst, int32_t *__restrict__ tw_oi, int32_t *__restrict__ tw_io,
-                                                Info *__restrict__ info) {
+                                                int32_t *__restrict__ tw_oi, Info *__restrict__ info) {
     for (int64_t j = (int64_t)blockIdx.x * kT + threadIdx.x; j < m; j += (int64_t)gridDim.x * kT) {
         const uint32_t e = ival[j];
         const int32_t s = esrc[e];
         ic[j] = s;
-        idst[j] = (int32_t)ikey[j];
-        tw_io[j] = (int32_t)e;
         tw_oi[e] = (int32_t)j;
         if ((uint32_t)s == ikey[j]) atomicAdd(&info->n_self, 1ull);
     }
@@ -198,9 +196,15 @@ struct Carver {
     }
 };
 
+// The per-edge arrays are carved as three pairs, and the build sorts in them:
+// nothing else of the edges' size is held while a graph is loaded.
+struct Pairs {
+    int32_t *p[3] = {nullptr, nullptr, nullptr};
+    size_t half = 0;  // second array of a pair
+};
+
 struct Scratch {
-    int32_t *src = nullptr, *dst = nullptr;  // the edge list, when it has to be copied
-    uint64_t *k0 = nullptr, *k1 = nullptr;   // edge sort keys, then the other sorts' keys and values
+    uint32_t *k0 = nullptr, *k1 = nullptr;  // keys and values of the vertex sorts
     uint32_t *words = nullptr;
     Info *info = nullptr;
     unsigned *count = nullptr;
@@ -214,10 +218,12 @@ int load_edges(int64_t m, const int32_t *from, int32_t *buf, const int32_t **use
     return SBP_OK;
 }
 
+// sorts the keys in pairs 1 and 2 and makes the out-rows; *at: the pair that
+// then holds the in-rows' keys and values
 template <class K>
-int sort_edges(const int32_t *s, const int32_t *d, int64_t m, int64_t n, const Scratch &x, sbp_graph *g,
-               uint32_t **spent, uint32_t **unused, cudaStream_t st) {
-    K *k0 = reinterpret_cast<K *>(x.k0), *k1 = reinterpret_cast<K *>(x.k1);
+int sort_edges(const int32_t *s, const int32_t *d, int64_t m, int64_t n, const Scratch &x, const Pairs &e, sbp_graph *g,
+               int *at, cudaStream_t st) {
+    K *k0 = reinterpret_cast<K *>(e.p[1]), *k1 = reinterpret_cast<K *>(e.p[2]);
     k_edge_keys<K><<<grid_of(m), kT, 0, st>>>(s, d, m, n, k0, x.info);
     SBP_LAUNCHED();
     bool first = true;
@@ -225,17 +231,17 @@ int sort_edges(const int32_t *s, const int32_t *d, int64_t m, int64_t n, const S
                                      &first)));
     // the in-rows' keys and values go where the sorted keys are not; those are
     // done with after this
-    *unused = reinterpret_cast<uint32_t *>(first ? x.k1 : x.k0);
-    *spent = reinterpret_cast<uint32_t *>(first ? x.k0 : x.k1);
-    k_out_rows<K><<<grid_of(m), kT, 0, st>>>(first ? k0 : k1, m, n, g->oc, g->esrc, *unused, *unused + m);
+    *at = first ? 2 : 1;
+    uint32_t *ikey = reinterpret_cast<uint32_t *>(e.p[*at]);
+    k_out_rows<K><<<grid_of(m), kT, 0, st>>>(first ? k0 : k1, m, n, g->oc, g->esrc, ikey, ikey + e.half);
     SBP_LAUNCHED();
     return SBP_OK;
 }
 
-// one vertex order, sorted in the edge keys' scratch
+// one vertex order
 int sort_vertices(const sbp_graph *g, int32_t maxk, bool groups, const Scratch &x, int32_t *out, cudaStream_t st) {
     const size_t n = (size_t)g->n;
-    uint32_t *k0 = reinterpret_cast<uint32_t *>(x.k0), *k1 = reinterpret_cast<uint32_t *>(x.k1);
+    uint32_t *k0 = x.k0, *k1 = x.k1;
     k_order_keys<<<grid_of(g->n), kT, 0, st>>>(g->op, g->ip, g->n, maxk, groups, k0, k0 + n);
     SBP_LAUNCHED();
     bool first = true;
@@ -246,23 +252,38 @@ int sort_vertices(const sbp_graph *g, int32_t maxk, bool groups, const Scratch &
 }
 
 // everything but the self-loop positions, whose number `info` then holds
-int build_graph(sbp_graph *g, const int32_t *src, const int32_t *dst, const Scratch &x, Info *info, uint32_t **ikey,
-                cudaStream_t st) {
+int build_graph(sbp_graph *g, const int32_t *src, const int32_t *dst, const Scratch &x, const Pairs &e, Info *info,
+                uint32_t **ikey, cudaStream_t st) {
     const int64_t n = g->n, m = g->m;
     SBP_CUDA(cudaMemsetAsync(x.info, 0, sizeof(Info), st));
     SBP_CUDA(cudaMemsetAsync(&x.info->bad, 0xff, 8, st));
     *ikey = nullptr;
+    // pair 0: the edge list, where it has to be copied, until its keys are
+    // made; then the out-rows.  Pairs 1 and 2: the keys of the first sort and
+    // its second buffer; then the in-rows' keys and values and theirs, which
+    // end as idst and tw_io in one pair, with the other free for ic and tw_oi
+    g->oc = e.p[0];
+    g->esrc = e.p[0] + e.half;
+    int at = 1;
     if (m > 0) {
         const int32_t *s, *d;
-        SBP_TRY(load_edges(m, src, x.src, &s, st));
-        SBP_TRY(load_edges(m, dst, x.dst, &d, st));
-        uint32_t *a = nullptr, *c = nullptr;  // keys and values, and their second set
-        if ((uint64_t)n * (uint64_t)n <= (uint64_t(1) << 32)) SBP_TRY(sort_edges<uint32_t>(s, d, m, n, x, g, &c, &a, st));
-        else SBP_TRY(sort_edges<uint64_t>(s, d, m, n, x, g, &c, &a, st));
+        SBP_TRY(load_edges(m, src, e.p[0], &s, st));
+        SBP_TRY(load_edges(m, dst, e.p[0] + e.half, &d, st));
+        if ((uint64_t)n * (uint64_t)n <= (uint64_t(1) << 32)) SBP_TRY(sort_edges<uint32_t>(s, d, m, n, x, e, g, &at, st));
+        else SBP_TRY(sort_edges<uint64_t>(s, d, m, n, x, e, g, &at, st));
+        uint32_t *a = reinterpret_cast<uint32_t *>(e.p[at]), *c = reinterpret_cast<uint32_t *>(e.p[3 - at]);
         bool first = true;
-        SBP_TRY((radix_sort<uint32_t, uint32_t>(a, c, a + m, c + m, m, bits_for((uint64_t)n - 1), x.words, st, &first)));
-        *ikey = first ? a : c;
-        k_in_rows<<<grid_of(m), kT, 0, st>>>(*ikey, *ikey + m, g->esrc, m, g->ic, g->idst, g->tw_oi, g->tw_io, x.info);
+        SBP_TRY((radix_sort<uint32_t, uint32_t>(a, c, a + e.half, c + e.half, m, bits_for((uint64_t)n - 1), x.words, st,
+                                                &first)));
+        if (!first) at = 3 - at;
+    }
+    g->idst = e.p[at];
+    g->tw_io = e.p[at] + e.half;
+    g->ic = e.p[3 - at];
+    g->tw_oi = e.p[3 - at] + e.half;
+    if (m > 0) {
+        *ikey = reinterpret_cast<uint32_t *>(g->idst);
+        k_in_rows<<<grid_of(m), kT, 0, st>>>(*ikey, *ikey + e.half, g->esrc, m, g->ic, g->tw_oi, x.info);
         SBP_LAUNCHED();
     }
     k_row_offsets<<<grid_of(n + 1), kT, 0, st>>>(g->esrc, *ikey, m, n, g->op, g->ip);
@@ -299,27 +320,20 @@ int finish_graph(sbp_graph *g, const Scratch &x, const Info &info, const uint32_
 }
 
 // Arrays of a graph and of its build, in one allocation each
-void carve_graph(sbp_graph *g, Carver &c) {
-    const size_t n = (size_t)g->n, m = (size_t)g->m;
+void carve_graph(sbp_graph *g, Pairs &e, Carver &c) {
+    const size_t n = (size_t)g->n;
+    e.half = ((size_t)std::max<int64_t>(g->m, 1) + 63) / 64 * 64;  // (aligned as an allocation is)
     c.take(&g->op, n + 1);
     c.take(&g->ip, n + 1);
-    c.take(&g->oc, m);
-    c.take(&g->ic, m);
-    c.take(&g->esrc, m);
-    c.take(&g->idst, m);
-    c.take(&g->tw_oi, m);
-    c.take(&g->tw_io, m);
+    for (auto &p : e.p) c.take(&p, 2 * e.half);
     c.take(&g->order, n);
     c.take(&g->by_degree, n);
 }
 
-void carve_scratch(Scratch &x, int64_t n, int64_t m, bool copy_src, bool copy_dst, Carver &c) {
-    const size_t mm = (size_t)m, nv = (size_t)std::max(n, m);
-    c.take(&x.src, copy_src ? mm : 0);
-    c.take(&x.dst, copy_dst ? mm : 0);
-    c.take(&x.k0, nv);
-    c.take(&x.k1, nv);
-    c.take(&x.words, (size_t)sort_scratch_words((int64_t)nv));
+void carve_scratch(Scratch &x, int64_t n, int64_t m, Carver &c) {
+    c.take(&x.k0, 2 * (size_t)n);
+    c.take(&x.k1, 2 * (size_t)n);
+    c.take(&x.words, (size_t)sort_scratch_words(std::max(n, m)));
     c.take(&x.info, 1);
     c.take(&x.count, 1);
 }
@@ -340,11 +354,11 @@ extern "C" int sbp_load_graph(int64_t n, int64_t m, const int32_t *src, const in
     g->n = n;
     g->m = m;
     cudaGetDevice(&g->device);
-    const bool copy_src = m > 0 && !readable_in_place(src), copy_dst = m > 0 && !readable_in_place(dst);
     Scratch x;
+    Pairs e;
     Carver cg, cs;  // first without memory, for the sizes
-    carve_graph(g, cg);
-    carve_scratch(x, n, m, copy_src, copy_dst, cs);
+    carve_graph(g, e, cg);
+    carve_scratch(x, n, m, cs);
     unsigned char *scratch = nullptr;
     int rc = SBP_OK;
     if (cudaMalloc((void **)&g->slab, cg.used) != cudaSuccess ||
@@ -355,11 +369,11 @@ extern "C" int sbp_load_graph(int64_t n, int64_t m, const int32_t *src, const in
     if (rc == SBP_OK) {
         cg = Carver{g->slab, 0};
         cs = Carver{scratch, 0};
-        carve_graph(g, cg);
-        carve_scratch(x, n, m, copy_src, copy_dst, cs);
+        carve_graph(g, e, cg);
+        carve_scratch(x, n, m, cs);
         Info info{};
         uint32_t *ikey = nullptr;
-        rc = build_graph(g, src, dst, x, &info, &ikey, st);
+        rc = build_graph(g, src, dst, x, e, &info, &ikey, st);
         if (rc == SBP_OK && info.bad != ~0ull)
             rc = fail(SBP_EINVAL, "sbp_load_graph: vertex id out of range at edge " + std::to_string(info.bad));
         if (rc == SBP_OK) rc = finish_graph(g, x, info, ikey, st);

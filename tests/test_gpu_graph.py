@@ -72,3 +72,36 @@ def test_first_bad_edge_is_named(device):
         src, dst = torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda()
     with pytest.raises(P.SbpError, match="at edge 3"):
         P.Graph(5, src, dst)
+
+
+def _pool_high(call):
+    """bytes that `call` took from the device's memory pool at the most"""
+    import ctypes
+    import os
+
+    for lib in ("libcudart.so.13", "libcudart.so", "/usr/local/cuda/lib64/libcudart.so"):
+        try:
+            rt = ctypes.CDLL(lib)
+            break
+        except OSError:
+            continue
+    else:
+        pytest.skip("no CUDA runtime library to ask")
+    pool, zero, high, now = ctypes.c_void_p(), ctypes.c_uint64(0), ctypes.c_uint64(0), ctypes.c_uint64(0)
+    dev = torch.cuda.current_device()
+    assert rt.cudaDeviceGetDefaultMemPool(ctypes.byref(pool), dev) == 0
+    torch.cuda.synchronize()
+    assert rt.cudaMemPoolSetAttribute(pool, 8, ctypes.byref(zero)) == 0  # cudaMemPoolAttrUsedMemHigh
+    assert rt.cudaMemPoolGetAttribute(pool, 7, ctypes.byref(now)) == 0  # cudaMemPoolAttrUsedMemCurrent
+    call()
+    torch.cuda.synchronize()
+    assert rt.cudaMemPoolGetAttribute(pool, 8, ctypes.byref(high)) == 0
+    return high.value - now.value
+
+
+@pytest.mark.parametrize("device", [False, True])
+@pytest.mark.parametrize("n,m", [(1_000, 3_000_000), (70_000, 3_000_000), (1_000_000, 100_000)])
+def test_loading_holds_no_scratch_of_the_edges_size(n, m, device):
+    g = _multigraph(n, m, seed=n)
+    src, dst = (torch.from_numpy(x).cuda() if device else x for x in (g.src, g.dst))
+    assert 16 * n < _pool_high(lambda: P.Graph(n, src, dst)) <= 16 * n + (5 << 20)
