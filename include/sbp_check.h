@@ -1,6 +1,7 @@
 /*
- * sbp_check.h -- test entry points of libsbp that need no device: host
- * runs of device-side logic, compared with the host code it must follow.
+ * sbp_check.h -- test entry points of libsbp that launch nothing: host runs
+ * of device-side logic, compared with the host code it must follow, and what
+ * the library chooses by.
  * Conventions as in sbp.h (SBP_OK or a negative SBP_E* code, the message
  * through sbp_last_error, host arrays borrowed for the call).
  */
@@ -8,6 +9,8 @@
 #define SBP_CHECK_H
 
 #include <stdint.h>
+
+#include "sbp.h"
 
 #ifdef __cplusplus
 extern "C" {
@@ -31,6 +34,10 @@ int sbp_bracket_check(const int32_t *B, const double *dl, int32_t count, double 
  * device of `sms` SMs: 8, 4 or 2 (a cluster per search) or 1.  SBP_EINVAL on
  * a negative count, sms < 1 or a NULL pointer. */
 int sbp_search_form_check(int64_t unfinished, int32_t sms, int32_t server, int32_t *ctas);
+
+/* *bytes: the device memory that the batching form counts for a run of g from
+ * one block per vertex down (what its admission adds up), beside the graph. */
+int sbp_model_bytes(const sbp_graph_t *g, int32_t dense_max_B, int64_t *bytes);
 
 /* Persistent launches of the batching form in this process so far, with one
  * CTA per search and with a cluster per search (either may be NULL). */

@@ -27,7 +27,7 @@ __all__ = [
     "sbp_compact", "sbp_partition", "sbp_get_assignment", "sbp_get_pending", "sbp_set_pending", "sbp_get_B", "sbp_get_dl",
     "sbp_get_blockmodel_dense", "sbp_get_degrees", "sbp_get_blockmodel_coo", "sbp_sync", "sbp_free_model", "sbp_philox_check",
     "sbp_dense_dl_noalloc", "sbp_kernel_launches", "sbp_dxlogx32_check", "sbp_bracket_check",
-    "sbp_search_form_check", "sbp_search_launches",
+    "sbp_search_form_check", "sbp_search_launches", "sbp_model_bytes",
     "sbp_default_batch_options", "sbp_partition_batch",
     "BatchOptions", "BatchResult", "BatchStats", "partition_batch", "Server", "sbp_autotune_batch", "autotune_batch",
     "sbp_server_create", "sbp_server_submit", "sbp_server_poll", "sbp_server_wait", "sbp_server_stats",
@@ -185,6 +185,7 @@ def load(path: str | None = None):
         "sbp_kernel_launches": (C.c_int, [P(u64)]),
         "sbp_bracket_check": (C.c_int, [vp, vp, i32, C.c_double, vp, P(i32)]),
         "sbp_search_form_check": (C.c_int, [C.c_int64, i32, i32, P(i32)]),
+        "sbp_model_bytes": (C.c_int, [vp, i32, P(C.c_int64)]),
         "sbp_search_launches": (C.c_int, [P(C.c_int64), P(C.c_int64)]),
         "sbp_default_batch_options": (C.c_int, [P(BatchOptions)]),
         "sbp_dxlogx32_check": (C.c_int, [vp, vp, i32, vp, vp]),
@@ -432,6 +433,13 @@ def sbp_search_form_check(unfinished: int, sms: int, server: bool = False) -> in
     ctas = C.c_int32(0)
     _check(lib().sbp_search_form_check(int(unfinished), int(sms), int(server), C.byref(ctas)))
     return int(ctas.value)
+
+
+def sbp_model_bytes(g: int, dense_max_B: int) -> int:
+    """Device bytes that the batching form counts for a run of graph g."""
+    n = C.c_int64(0)
+    _check(lib().sbp_model_bytes(g, int(dense_max_B), C.byref(n)))
+    return int(n.value)
 
 
 def sbp_search_launches() -> tuple[int, int]:

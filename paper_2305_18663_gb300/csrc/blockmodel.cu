@@ -662,6 +662,16 @@ int num_sms() {
 
 }  // namespace
 
+size_t dense_bytes(int64_t B) {
+    const size_t b = (size_t)B, chunks = (b + kColChunk - 1) / kColChunk;
+    return 12 * b * b + 128 * b + (B >= kWidePrefixB ? 4 * b * chunks : 0);
+}
+
+size_t block_bytes(int64_t B) { return 44 * (size_t)B; }
+
+size_t label_row_bytes(const sbp_graph *g) { return 8 * (size_t)g->m; }
+
+// (dense_bytes and block_bytes say how much this allocates)
 int ensure_capacity(sbp_model *m, int32_t B) {
     m->dense = B <= m->p.dense_max_B;
     if (!m->dense) SBP_TRY(ensure_sparse_capacity(m, B));

@@ -617,6 +617,15 @@ int launch_relabel(sbp_model *m, const int32_t *map_dev);
 int launch_vertex_count(sbp_model *m);
 int ensure_capacity(sbp_model *m, int32_t B);
 int check_status(const sbp_model *m);
+// device bytes of what these functions and the passes allocate, each beside
+// its allocations: of B blocks, of the dense counts, of sparse rows, of the
+// block-labelled rows, of the merge application, of the decision passes
+size_t block_bytes(int64_t B);
+size_t dense_bytes(int64_t B);
+size_t sparse_bytes(const sbp_graph *g, int64_t B);
+size_t label_row_bytes(const sbp_graph *g);
+size_t merge_work_bytes(int64_t B);
+size_t pass_bytes(const sbp_graph *g, int64_t B);
 int xlogx_table(int64_t need, const __int128 **table, int64_t *size);
 int ensure_sparse_capacity(sbp_model *m, int32_t B);
 int rebuild_sparse(sbp_model *m, bool after_pass, bool *dl_done, int *n_parts);

@@ -45,6 +45,7 @@
 #include <vector>
 
 #include "batch.h"
+#include "sbp_check.h"
 #include "driver.h"
 
 namespace sbp {
@@ -54,12 +55,14 @@ double now_s() {
     return std::chrono::duration<double>(std::chrono::steady_clock::now().time_since_epoch()).count();
 }
 
-// device bytes of a graph's model at its largest: sparse rows at B = N, or
-// the dense counts and prefix rows at the first dense B, min(N, dense_max_B)
+// device bytes of a graph's model at its largest, from B = N on: sparse rows
+// where N is above dense_max_B, the dense counts and prefix rows at the first
+// dense B, at most min(N, dense_max_B), the labels, and 1 MB for what has a
+// fixed size and for the allocations' rounding
 size_t model_bytes(const sbp_graph *g, int dense_max_B) {
-    const size_t n = (size_t)g->n, m = (size_t)std::max<int64_t>(g->m, 1);
-    const size_t bd = std::min(n, (size_t)dense_max_B);
-    return 152 * m + 128 * n + 12 * bd * bd + (1u << 20);
+    const int64_t n = g->n, bd = std::min<int64_t>(n, dense_max_B);
+    return (n > dense_max_B ? sparse_bytes(g, n) : 0) + dense_bytes(bd) + block_bytes(n) + label_row_bytes(g) +
+           merge_work_bytes(n) + pass_bytes(g, n) + 8 * (size_t)n + (1u << 20);
 }
 
 }  // namespace
@@ -609,6 +612,12 @@ int partition_batch(const sbp_graph_t *const *graphs, int32_t count, const sbp_p
 
 }  // namespace
 }  // namespace sbp
+
+extern "C" int sbp_model_bytes(const sbp_graph_t *g, int32_t dense_max_B, int64_t *bytes) {
+    if (!g || !bytes || dense_max_B < 1) return fail(SBP_EINVAL, "sbp_model_bytes: bad argument");
+    *bytes = (int64_t)sbp::model_bytes(g, dense_max_B);
+    return SBP_OK;
+}
 
 extern "C" int sbp_partition_batch(const sbp_graph_t *const *graphs, int32_t count, const sbp_params *p,
                                    const sbp_batch_options *o, int32_t *const *b_out, sbp_batch_result *res,

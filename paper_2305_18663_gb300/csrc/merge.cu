@@ -115,8 +115,7 @@ int ensure_merge_work(sbp_model *m, int32_t B) {
     model_free(m->merge_work, m->stream);
     m->merge_work = nullptr;
     m->merge_work_B = 0;
-    const size_t bytes = (size_t)B * kMergeApplyBytes + kClusterWords * 4;
-    if (model_alloc((void **)&m->merge_work, bytes, m->stream) != cudaSuccess) {
+    if (model_alloc((void **)&m->merge_work, merge_work_bytes(B), m->stream) != cudaSuccess) {
         cudaGetLastError();
         return fail(SBP_ENOMEM, "device allocation failed for the merge phase");
     }
@@ -144,6 +143,8 @@ MergeWork merge_work(const sbp_model *m) {
 }
 
 }  // namespace
+
+size_t merge_work_bytes(int64_t B) { return (size_t)B * kMergeApplyBytes + kClusterWords * 4; }
 
 int launch_merge_proposals(sbp_model *m, uint64_t round_id) {
     int sms = 0, dev = 0;

@@ -1634,16 +1634,31 @@ namespace {
 // The CTA kernel's neighbour table (cap slots of 16 bytes): in shared memory
 // while it fits, else a slice per CTA of a global scratch the model keeps
 // (at most 1 GB, fewer CTAs for very large tables).
-int cta_table(sbp_model *m, int cap, int sms, int *grid, size_t *smem, unsigned long long **gtab) {
+size_t cta_table_bytes(int cap, int sms, int *grid) {
     const size_t bytes = (size_t)cap * 16;
     *grid = sms * 4;
-    *gtab = nullptr;
-    *smem = bytes;
-    if (bytes <= 160 * 1024) return SBP_OK;
-    *smem = 0;
+    if (bytes <= 160 * 1024) return 0;
     const size_t per_grid = std::max<size_t>(1, (size_t(1) << 30) / bytes);
     if ((size_t)*grid > per_grid) *grid = (int)per_grid;
-    const size_t need = bytes * (size_t)*grid;
+    return bytes * (size_t)*grid;
+}
+
+// log2 of the slots that hold a hub's distinct neighbour blocks at a load of
+// at most 0.8
+int hub_cap_log2(const sbp_graph *g, int64_t B) {
+    const int64_t dmax = g->max_deg < B ? g->max_deg : B;
+    const int64_t need = dmax + dmax / 4 + 2;
+    int cap_log2 = 6;
+    while ((int64_t(1) << cap_log2) < need) ++cap_log2;
+    return cap_log2;
+}
+
+int cta_table(sbp_model *m, int cap, int sms, int *grid, size_t *smem, unsigned long long **gtab) {
+    const size_t need = cta_table_bytes(cap, sms, grid);
+    *gtab = nullptr;
+    *smem = (size_t)cap * 16;
+    if (need == 0) return SBP_OK;
+    *smem = 0;
     if (m->cta_tab_bytes < need) {
         model_free(m->cta_tab, m->stream);
         m->cta_tab = nullptr;
@@ -1696,10 +1711,7 @@ int launch_groups(sbp_model *m, const DecideArgs &a, int sms, const cudaStream_t
         SBP_LAUNCHED();
     } else if (g->bin[4] > g->bin[3]) {
         if (g->n - g->bin[3] > g->n_mid + g->n_wide) {
-            const int64_t dmax = g->max_deg < B ? g->max_deg : B;
-            const int64_t need = dmax + dmax / 4 + 2;
-            int cap_log2 = 6;
-            while ((int64_t(1) << cap_log2) < need) ++cap_log2;
+            const int cap_log2 = hub_cap_log2(g, B);
             int grid;
             size_t smem;
             unsigned long long *gtab;
@@ -1778,11 +1790,7 @@ int launch_recheck(sbp_model *m, const DecideArgs &a0, int sms) {
     const sbp_graph *g = m->g;
     DecideArgs a = a0;
     a.force_exact = 1;
-    const int64_t dmax = g->max_deg < m->B ? g->max_deg : m->B;
-    const int64_t need = dmax + dmax / 4 + 2;
-    int cap_log2 = 6;
-    while ((int64_t(1) << cap_log2) < need) ++cap_log2;
-    const int cap = 1 << cap_log2;
+    const int cap_log2 = hub_cap_log2(g, m->B), cap = 1 << cap_log2;
     int grid;
     size_t smem;
     unsigned long long *gtab;
@@ -1850,7 +1858,18 @@ int launch_evals(sbp_model *m, const DecideArgs &a, int sms, bool fused) {
     return launch_recheck<DL32>(m, a, sms);
 }
 
+// at most one item per vertex plus one per kMoveChunk edge ends
+int64_t most_items(const sbp_graph *g) { return g->n + (2 * g->m) / kMoveChunk + 1; }
+
 }  // namespace
+
+// the mover lists, the accepted-move list, the hybrid pass's flags, the hubs'
+// tables
+size_t pass_bytes(const sbp_graph *g, int64_t B) {
+    int grid;
+    return 2 * (size_t)g->n * sizeof(Mover) + (size_t)most_items(g) * sizeof(int2) + (size_t)g->n +
+           cta_table_bytes(1 << hub_cap_log2(g, std::min<int64_t>(B, 1 << 24)), sm_count(), &grid);  // (B is below that)
+}
 
 int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_end, const sbp_vertex_trace *trace) {
     const sbp_graph *g = m->g;
@@ -1863,8 +1882,7 @@ int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_en
         }
     }
     if (!m->items) {
-        // at most one item per vertex plus one per kMoveChunk edge ends
-        const int64_t cap = g->n + (2 * g->m) / kMoveChunk + 1;
+        const int64_t cap = most_items(g);
         if (model_alloc((void **)&m->items, (size_t)cap * sizeof(int2), m->stream) != cudaSuccess) {
             cudaGetLastError();
             return fail(SBP_ENOMEM, "cudaMalloc failed for the accepted-move list");

@@ -270,6 +270,15 @@ __global__ void k_sparse_pivots(const uint32_t *__restrict__ rp, const uint32_t 
 
 }  // namespace
 
+size_t sparse_bytes(const sbp_graph *g, int64_t B) {
+    const size_t E = (size_t)std::max<int64_t>(g->m, 1), n = (size_t)g->n, b = (size_t)B;
+    const size_t edges = 8 * 4 * E, tables = 8 * (4 * E + 2 * n), vertices = 8 * n;
+    const size_t rows = 28 * b + 8, lists = 4 * (8 * b + 7 * (b / 1024 + 1)), pivots = 256 * b;
+    const size_t small = std::min(b, (size_t)kSmallRowsB);
+    return edges + tables + vertices + rows + lists + pivots + 4 * small * small + 4 * (size_t)kSparseScratch;
+}
+
+// (sparse_bytes says how much this allocates)
 int ensure_sparse_capacity(sbp_model *m, int32_t B) {
     sbp_model::Sparse &S = m->sp;
     const int64_t E = m->g->m > 0 ? m->g->m : 1, n = m->g->n;
