@@ -633,14 +633,10 @@ int build_sparse_rows(sbp_model *m, int *n_parts);  // sparse_rows.cu
 // the rows' columns and counts without the slack between them, row r from
 // first[r] (host array), in scratch of the model
 int pack_sparse_rows(const sbp_model *m, const uint32_t *first, const int32_t **rc, const int32_t **rv);
-constexpr int64_t kSparseScratch = 20000;  // words: the small rebuild's lengths and sums, or a cluster's exchange
+constexpr int64_t kSparseScratch = 20000;  // words: the small rebuild's lengths and sums, the row lists' lengths
 void free_sparse(sbp_model *m);
 
-// sort.cu: exclusive scan of n uint32 (in may equal out; *total_dev, device,
-// may be NULL) and the stable LSD radix sort with its scratch sizes
-int exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *total_dev, uint32_t *scratch,
-                       cudaStream_t st);
-int64_t scan_scratch_words(int64_t n);
+// sort.cu: the stable LSD radix sort and its scratch size
 int64_t sort_scratch_words(int64_t n);
 template <class K, class V>
 int radix_sort(K *k0, K *k1, V *v0, V *v1, int64_t n, int bits, uint32_t *scratch, cudaStream_t st, bool *in_first);

@@ -59,9 +59,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t *__
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-// one block: exclusive scan of the block sums, in place; grand total to *total
-__global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t *__restrict__ sums, int64_t nb,
-                                                            uint32_t *__restrict__ total_out) {
+// one block: exclusive scan of the block sums, in place
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t *__restrict__ sums, int64_t nb) {
     __shared__ uint32_t sh[33];
     uint32_t carry = 0;
     for (int64_t base = 0; base < nb; base += kScanBlock) {
@@ -81,12 +80,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t *__restrict
         }
         carry += total;
     }
-    if (threadIdx.x == 0 && total_out) *total_out = carry;
 }
 
 // one block for short arrays: exclusive scan of in into out (may alias)
-__global__ void __launch_bounds__(kScanThreads) k_scan_small(const uint32_t *in, int64_t n, uint32_t *out,
-                                                             uint32_t *__restrict__ total_out) {
+__global__ void __launch_bounds__(kScanThreads) k_scan_small(const uint32_t *in, int64_t n, uint32_t *out) {
     __shared__ uint32_t sh[33];
     uint32_t carry = 0;
     for (int64_t base = 0; base < n; base += kScanBlock) {
@@ -106,7 +103,6 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_small(const uint32_t *in,
         }
         carry += total;
     }
-    if (threadIdx.x == 0 && total_out) *total_out = carry;
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_down(const uint32_t *__restrict__ in, int64_t n,
@@ -278,34 +274,26 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const K *__restrict__
     }
 }
 
-}  // namespace
-
 // Exclusive scan of n uint32 values (in may equal out).  scratch needs
-// scan_scratch_words(n) words; *total_dev (device, may be NULL) gets the sum.
+// scan_scratch_words(n) words.
 int64_t scan_scratch_words(int64_t n) { return (n + kScanBlock - 1) / kScanBlock + 1; }
 
-int exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *total_dev, uint32_t *scratch,
-                       cudaStream_t st) {
-    if (n <= 0) {
-        if (total_dev) SBP_CUDA(cudaMemsetAsync(total_dev, 0, 4, st));
-        return SBP_OK;
-    }
+int exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *scratch, cudaStream_t st) {
+    if (n <= 0) return SBP_OK;
     if (n <= 8 * kScanBlock) {
-        k_scan_small<<<1, kScanThreads, 0, st>>>(in, n, out, total_dev);
+        k_scan_small<<<1, kScanThreads, 0, st>>>(in, n, out);
         SBP_LAUNCHED();
         return SBP_OK;
     }
     const int64_t nb = (n + kScanBlock - 1) / kScanBlock;
     k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, scratch);
     SBP_LAUNCHED();
-    k_scan_sums<<<1, kScanThreads, 0, st>>>(scratch, nb, total_dev);
+    k_scan_sums<<<1, kScanThreads, 0, st>>>(scratch, nb);
     SBP_LAUNCHED();
     k_scan_down<<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, scratch, out);
     SBP_LAUNCHED();
     return SBP_OK;
 }
-
-namespace {
 
 // chunk length (a whole number of rounds) and chunk count for n keys
 void rs_chunks(int64_t n, int64_t *chunk, int *G) {
@@ -334,7 +322,7 @@ int rs_pass(const K *ks, const V *vs, int64_t n, int shift, int nbits, K *kd, V 
     uint32_t *sscr = scratch + (int64_t)kRsMaxBins * kRsMaxChunks;
     k_rs_count<K><<<G, kRsThreads, 0, st>>>(ks, n, chunk, shift, nbins, G, hist);
     SBP_LAUNCHED();
-    SBP_TRY(exclusive_scan_u32(hist, hist, (int64_t)nbins * G, nullptr, sscr, st));
+    SBP_TRY(exclusive_scan_u32(hist, hist, (int64_t)nbins * G, sscr, st));
     const size_t smem = rs_stage_bytes<K, V>(vs != nullptr);
     // the staging area plus the static tables pass the default 48 KB limit
     SBP_TRY(ensure_dyn_smem((const void *)k_rs_scatter<K, V>, smem));
