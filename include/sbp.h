@@ -151,10 +151,12 @@ void sbp_free_graph(sbp_graph_t *g);
 /* Creates a blockmodel handle for assignment b (n labels in [0, B), host or
  * device) and builds M, block degrees and DL (Eq. 1-2, Section II-A).
  * stream: a cudaStream_t (may be NULL) that every later call on this model
- * orders its work on (the decision pass of a graph with 2^19 edges or more
- * runs part of its kernels on two side streams of the model, forked from and
- * joined back into this stream within the call).  p may be NULL
- * (defaults).  The graph must outlive the model.
+ * orders its work on.  On a graph with 2^19 edges or more, two steps run part
+ * of their kernels on two side streams of the model, forked from and joined
+ * back into this stream within the call: the decision pass, and the rebuild of
+ * a sparse blockmodel of more than 1024 blocks, which creating a model, setting
+ * its labels, a commit, a merge phase and a compaction can ask for.  p may be
+ * NULL (defaults).  The graph must outlive the model.
  * Errors: SBP_EINVAL for B < 1, B > n or a label outside [0, B);
  * SBP_ENOMEM. */
 int sbp_build_blockmodel(const sbp_graph_t *g, int32_t B, const int32_t *b, const sbp_params *p, void *stream,

@@ -5,7 +5,8 @@
 // per warp; for 33..128 with direct-mapped counts while B is small),
 // k_eval_warp_direct (one warp per mover, direct-mapped counts) or, at
 // larger B, k_eval_table (one warp per mover with a shared-memory table) and
-// k_eval_cta (one CTA per mover, very large tables).  In a pass over all
+// k_eval_cta (one CTA per mover, the largest rows).  A small pass over all
+// vertices is one kernel, k_eval_small, a warp per mover.  In a pass over all
 // vertices without a trace the first two kinds draw the proposals of their
 // group's vertices themselves; otherwise k_propose (one lane per vertex)
 // draws every proposal first and hands the moving ones (s != r) over in
@@ -623,7 +624,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 2) k_eval_small(DecideArgs 
 }
 
 // ---------------------------------------------------------------------------
-// CTA per mover: tables beyond 4096 slots or degree >= 65536
+// CTA per mover: at large B the movers of more than kWideDeg edges, degrees of
+// 65,536 and more at any B, and the recheck
 
 struct CtaScratch {
     __int128 dl[kBigThreads / 32];

@@ -333,7 +333,8 @@ int rebuild_sparse(sbp_model *m, bool after_pass, bool *dl_done, int *n_parts) {
         S.cells_B = 0;
         return build_sparse_rows(m, n_parts);
     }
-    // counting sort over the B x B keys, then everything in one CTA
+    // the B x B counts, then five kernels: lengths, offsets, rows with columns
+    // and tables, scalars with DL, pivots
     if (after_pass && S.cells_B == B)
         SBP_TRY(update_cells(m, S.cells));
     else
