@@ -10,7 +10,13 @@ namespace {
 constexpr int kMergeThreads = 256;
 constexpr int kMergeWarps = kMergeThreads / 32;
 // sparse blocks with more entries than this get a CTA (a hub's block of the
-// first phases has thousands, and one warp on it would be the launch's tail)
+// first phases has thousands, and one warp on it would be the launch's tail).
+// The line, in us, at 128, 512, 2048 and never: 200,000 vertices, 4M edges, heavy
+// tail, one block per vertex 1760 / 1740 / 1733 / 2834, 50,000 blocks 2840 /
+// 1693 / 1881 / 2435; 50,000 vertices, 6000 blocks 537 / 414 / 539 / 614; 1M
+// vertices, 10M edges, 250,000 blocks 5405 / 4201 / 4371 / 6411.  Where all
+// blocks have much the same entries a warp each is better (200,000 vertices,
+// 6000 blocks 1576 / 1579 / 1393 / 1312).
 constexpr uint32_t kMergeLong = 512;
 
 // Teams of `parts` warps (1, 2, 4 or 8) take the blocks in turn.  long_pass
