@@ -1566,13 +1566,12 @@ static constexpr int64_t kSideFirstGroup = 8192;
 int fork_side(sbp_model *m, cudaStream_t st[3]) {
     st[0] = st[1] = st[2] = m->stream;
     if (m->g->m < kSideStreamEdges) return SBP_OK;
-    if (!m->fork_ev) {
-        for (int i = 0; i < 2; ++i) {
-            SBP_CUDA(cudaStreamCreateWithFlags(&m->side[i], cudaStreamNonBlocking));
-            SBP_CUDA(cudaEventCreateWithFlags(&m->join_ev[i], cudaEventDisableTiming));
-        }
-        SBP_CUDA(cudaEventCreateWithFlags(&m->fork_ev, cudaEventDisableTiming));
+    // (a call that failed half way left what it had made)
+    for (int i = 0; i < 2; ++i) {
+        if (!m->side[i]) SBP_CUDA(cudaStreamCreateWithFlags(&m->side[i], cudaStreamNonBlocking));
+        if (!m->join_ev[i]) SBP_CUDA(cudaEventCreateWithFlags(&m->join_ev[i], cudaEventDisableTiming));
     }
+    if (!m->fork_ev) SBP_CUDA(cudaEventCreateWithFlags(&m->fork_ev, cudaEventDisableTiming));
     SBP_CUDA(cudaEventRecord(m->fork_ev, m->stream));
     for (int i = 0; i < 2; ++i) SBP_CUDA(cudaStreamWaitEvent(m->side[i], m->fork_ev, 0));
     st[0] = m->side[1];
@@ -1582,11 +1581,14 @@ int fork_side(sbp_model *m, cudaStream_t st[3]) {
 
 int join_side(sbp_model *m) {
     if (m->g->m < kSideStreamEdges || !m->fork_ev) return SBP_OK;
+    int rc = SBP_OK;  // both are joined, whatever the first gives
     for (int i = 0; i < 2; ++i) {
-        SBP_CUDA(cudaEventRecord(m->join_ev[i], m->side[i]));
-        SBP_CUDA(cudaStreamWaitEvent(m->stream, m->join_ev[i], 0));
+        cudaError_t e = cudaEventRecord(m->join_ev[i], m->side[i]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(m->stream, m->join_ev[i], 0);
+        else cudaStreamSynchronize(m->side[i]);
+        if (e != cudaSuccess) rc = cuda_fail(e, "joining the side streams");
     }
-    return SBP_OK;
+    return rc;
 }
 
 ModelDev model_dev(sbp_model *m) {
