@@ -1809,8 +1809,11 @@ int launch_recheck(sbp_model *m, const DecideArgs &a0, int sms) {
 // every mover a warp: up to the most vertices at which it was nowhere slower
 // than the groups' kernels, by what these have to do.
 //   - Only the group of up to 32 edges: one kernel with 32 movers a warp.
-//   - More groups: a kernel each, one after another (below 2^19 edges) or on
-//     three streams; rows of hundreds of edges have a warp each there too,
+//   - More groups: a kernel each, one after another below 2^19 edges.  The
+//     second group's takes 30 to 70 us as soon as a few warps have a batch of
+//     its movers; three hubs, or hundreds of rows above 128 edges, do not.
+//   - From 2^19 edges they run on three streams, where the top group's rows
+//     are the long ones; rows of hundreds of edges have a warp each there too,
 //     with twice the warps, and win from some 2^21 edges on (the line: 3 x 2^19).
 //   - B > 1022: half the warps here, none lost there in the first group.
 // Both sides in us (groups, small; labels near the planted ones, B = 4 / 1000;
@@ -1818,13 +1821,18 @@ int launch_recheck(sbp_model *m, const DecideArgs &a0, int sms) {
 // 20,000 42, 40 / 53, 60; 57, 83; at 60,000 50, 77 / 65, 109; 75, 193.  More
 // groups, 6 edges a vertex and three hubs of 300, 20,000 vertices 51, 42 /
 // 66, 56; 58, 83; at 30,000 54, 52 / 70, 69; 74, 112; at 60,000 62, 76 / 81,
-// 107; 87, 187; 32 edges a vertex, 20,000 71, 41 / 111, 52; 114, 75; 40,000
-// (2^19.3 edges) 48, 61 / 68, 75; 81, 120.
+// 107; 87, 187; 100 vertices of 40 among them, 40,000 82, 63 / 133, 83; 137,
+// 139; 20 edges a vertex, 20,000 56, 42 / 97, 57; 95, 80, 40,000 71, 62 / 96, 77;
+// 102, 130, 60,000 61, 77 / 96, 103; 98, 168; 32 edges a vertex, 20,000 71, 41 /
+// 111, 52; 114, 75, 40,000 (2^19.3 edges) 48, 61 / 68, 75; 81, 120, with a heavy
+// tail 70, 59 / 129, 80; 128, 124.
 bool small_pass(const sbp_graph *g, const DecideArgs &a, int B) {
     const int64_t n = a.vcount[0] + a.vcount[1] + a.vcount[2];
     const bool half = direct_warps(B) < kWarpsPerCta;
     if (a.vcount[1] + a.vcount[2] == 0) return n <= (half ? 2500 : 5000);
-    if (g->m < kSideStreamEdges) return n <= (half ? 8000 : 22000);
+    if (g->m < kSideStreamEdges && a.vcount[1] >= 64) return n <= (half ? 20000 : 40000);
+    if (g->m < kSideStreamEdges) return n <= (half ? 10000 : 22000);
+    if (!half && a.vcount[2] >= 64 && g->m <= 3 * (int64_t(1) << 18)) return n <= 40000;
     return g->m <= 3 * (int64_t(1) << 19) && n <= (half ? 6000 : 20000);
 }
 

@@ -23,12 +23,15 @@ def _launches(call):
 
 def _graph(n, extra, seed):
     """every vertex with two edges out and two in; then `extra`: None, "hub"
-    (one vertex with 300 edges more) or a number of random edges in all"""
+    (one vertex with 300 edges more), "mid" (64 with 40 more) or a number of
+    random edges in all"""
     rng = np.random.default_rng(seed)
     v = np.arange(n)
     src, dst = [v, v], [(v + 1) % n, (v + n // 3) % n]
     if extra == "hub":
         src, dst = src + [np.zeros(300, np.int64)], dst + [rng.integers(0, n, 300)]
+    elif extra == "mid":
+        src, dst = src + [np.repeat(np.arange(64), 40)], dst + [rng.integers(64, n, 64 * 40)]
     elif extra:
         src, dst = src + [rng.integers(0, n, extra - 2 * n)], dst + [rng.integers(0, n, extra - 2 * n)]
     return P.Graph(n, np.concatenate(src).astype(np.int32), np.concatenate(dst).astype(np.int32))
@@ -36,7 +39,8 @@ def _graph(n, extra, seed):
 
 @pytest.mark.parametrize("n,extra,B,one", [
     (5_000, None, 1022, True), (5_001, None, 100, False), (2_500, None, 1023, True), (2_501, None, 1023, False),
-    (22_000, "hub", 100, True), (22_001, "hub", 100, False), (8_000, "hub", 1023, True), (8_001, "hub", 1023, False),
+    (22_000, "hub", 100, True), (22_001, "hub", 100, False), (10_000, "hub", 1023, True), (10_001, "hub", 1023, False),
+    (40_000, "mid", 100, True), (40_001, "mid", 100, False), (20_000, "mid", 1023, True), (20_001, "mid", 1023, False),
     (20_000, 1 << 19, 100, True), (20_001, 1 << 19, 100, False),
     (6_000, 1 << 19, 1023, True), (6_001, 1 << 19, 1023, False),
     (2_000, 3 << 19, 100, True), (2_000, (3 << 19) + 1, 100, False),
