@@ -463,7 +463,7 @@ extern "C" int sbp_commit(sbp_model_t *m, sbp_sweep_stats *stats) {
     SBP_TRY(rc);
     if (stats) {
         SBP_TRY(read_stats(m, stats));
-        m->light = commit_small_load_ok(m, h->c);
+        m->light = commit_small_try_next(m, h->c);
     }
     SBP_CUDA(cudaMemsetAsync(m->counters, 0, sizeof(DevCounters), m->stream));
     return SBP_OK;

@@ -239,7 +239,7 @@ struct sbp_model {
     bool nb_ok = false;
     bool nb_in_commit = false;  // the apply step's kernel updated them in this commit
     bool list_ok = true;
-    bool light = true;  // the last moves known to the host were within the one-launch commit's load
+    bool light = true;  // after the last moves known to the host, the one-launch commit is asked
     std::vector<std::pair<int64_t, int64_t>> decided;  // decide ranges since the last commit
     // side streams of the decision pass: the three degree groups' kernels
     // run concurrently so that each one's tail is filled by the others
@@ -605,6 +605,7 @@ int launch_prefix(sbp_model *m);                 // P, Pc, degrees, reciprocals 
 bool commit_small_ok(const sbp_model *m);
 bool commit_small_fits(const sbp_model *m);
 bool commit_small_load_ok(const sbp_model *m, const DevCounters &c);
+bool commit_small_try_next(const sbp_model *m, const DevCounters &c);  // worth asking the kernel after these
 int commit_small(sbp_model *m, SweepReadback *host, bool checked);
 int commit_blockmodel(sbp_model *m);   // the same after a pass: m->b new labels, m->bnew the previous ones
 int launch_decide(sbp_model *m, uint64_t sweep_id, int64_t v_begin, int64_t v_end, const sbp_vertex_trace *trace);
