@@ -228,8 +228,8 @@ int upload_incremental(sbp_model *m, const int32_t *b) {
     m->list_ok = true;  // the items list every change, once
     m->decided.clear();
     m->nb_in_commit = false;
-    m->light = commit_small_load_ok(m, h->c);
-    if (m->light && commit_small_ok(m)) {
+    m->light = commit_small_try_next(m, h->c);
+    if (commit_small_ok(m) && commit_small_load_ok(m, h->c)) {
         const int rs = commit_small(m, nullptr, false);
         if (rs != SBP_OK) m->nb_ok = false;
         return rs;

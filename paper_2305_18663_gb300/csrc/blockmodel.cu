@@ -521,24 +521,34 @@ __global__ void __launch_bounds__(kThreads, kItemCtas) k_nb_items(GraphDev g, co
 //     edges, nothing moved): 66 and 51 at B = 256, 71 and 68 at 384, 74 and 77
 //     at 512;
 //   - moves: an item costs some 6 ns, an edge end of an update 0.15 ns, an edge
-//     of a recount 0.075 ns, and the blocks' rows add up, against the 25 to 30
-//     us it saves.  kCommitMaxLoad is that budget in items.  B = 128: 8000
-//     vertices, 130,000 edges, load 3530 76 and 70, 6600 82 and 84; 20,000
-//     vertices, 500,000 edges, 2600 80 and 67, 4920 82 and 83, 10,600 83 and
-//     110; 65,000 vertices, 520,000 edges, 2120 83 and 68, 4760 82 and 80,
-//     45,000 91 and 266; B = 256: 20,000 vertices, 320,000 edges, 4710 80 and 82;
+//     of a recount 0.075 ns, and the blocks' rows add up, against the launches
+//     it saves; commit_max_load is that budget in items.  A pass's commit also
+//     saves the copies that read its statistics back: B = 128, 8000 vertices,
+//     130,000 edges, load 4670 57 and 49; 12,000, 170,000, 6540 57 and 57;
+//     20,000, 130,000, 6080 57 and 53, 9360 58 and 67; 60,000, 500,000, 6850 59
+//     and 63; B = 64: 12,000, 170,000, 6340 57 and 56; B = 256: 5720 57 and 54,
+//     7470 58 and 63.  At few blocks the separate kernels wait for one another
+//     at the counts, B = 8: 20,000 vertices, 520,000 edges, 9790 142 and 129,
+//     12,400 156 and 167; 40,000, 300,000, 10,990 107 and 98, 17,900 120 and
+//     133.  Labels set from outside, nothing read, B = 128: 8000, 130,000, 3530
+//     76 and 70, 6600 82 and 84; 20,000, 500,000, 2600 80 and 67, 4920 82 and
+//     83, 10,600 83 and 110; 65,000, 520,000, 4760 82 and 80, 45,000 91 and 266;
 //   - vertices and edges, up to which these were measured.
 // Where not every commit of the model is within the load, the kernel looks at
 // the moves first and leaves the commit to the separate kernels when there
 // are too many (a launch and a wait lost).  It is not asked after a pass with
-// more than kCommitTryFactor times the load: from one pass to the next the
-// moves rarely fall by more.
+// (or labels set from outside) more than kCommitTryFactor times the load: from
+// one pass to the next the moves rarely fall by more.
 constexpr int kCommitThreads = 1024;
 constexpr int kCommitCluster = 8;
 constexpr int kCommitMaxB = 256;
 constexpr int64_t kCommitMaxEdges = int64_t(1) << 19;
 constexpr int64_t kCommitMaxVertices = int64_t(1) << 16;
-constexpr unsigned long long kCommitMaxLoad = 4800, kCommitTryFactor = 3;
+constexpr unsigned long long kCommitTryFactor = 3;
+
+__host__ __device__ inline unsigned long long commit_max_load(int B) {
+    return 6000 + 32000 / (B > 8 ? B : 8);  // (fewer than 8 blocks were not measured)
+}
 
 __host__ __device__ inline bool commit_counts_moves(const DevCounters &c, int64_t m) {
     return c.acc_edges * 4ull <= (unsigned long long)m;  // else all edges are counted again
@@ -578,7 +588,7 @@ __global__ void __launch_bounds__(kCommitThreads) k_commit_small(SmallCommit a) 
     const int B = a.B, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int tid = cluster_rank() * kCommitThreads + threadIdx.x, nt = cluster_size() * kCommitThreads;
     const DevCounters c = *a.counters;
-    if (a.checked && commit_load(c, a.g.m, B) > kCommitMaxLoad) {
+    if (a.checked && commit_load(c, a.g.m, B) > commit_max_load(B)) {
         if (tid == 0) a.host->done = 0;
         return;
     }
@@ -866,15 +876,16 @@ bool commit_small_ok(const sbp_model *m) {
 // all vertices moved, all edges counted again
 bool commit_small_fits(const sbp_model *m) {
     const sbp_graph *g = m->g;
-    return (unsigned long long)(g->n + 2 * g->m / kMoveChunk + g->m / 80 + (int64_t)m->B * m->B / 64) <= kCommitMaxLoad;
+    return (unsigned long long)(g->n + 2 * g->m / kMoveChunk + g->m / 80 + (int64_t)m->B * m->B / 64) <=
+           commit_max_load(m->B);
 }
 
 bool commit_small_load_ok(const sbp_model *m, const DevCounters &c) {
-    return commit_load(c, m->g->m, m->B) <= kCommitMaxLoad;
+    return commit_load(c, m->g->m, m->B) <= commit_max_load(m->B);
 }
 
 bool commit_small_try_next(const sbp_model *m, const DevCounters &c) {
-    return commit_load(c, m->g->m, m->B) <= kCommitTryFactor * kCommitMaxLoad;
+    return commit_load(c, m->g->m, m->B) <= kCommitTryFactor * commit_max_load(m->B);
 }
 
 int commit_small(sbp_model *m, SweepReadback *host, bool checked) {

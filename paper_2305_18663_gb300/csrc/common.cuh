@@ -132,7 +132,7 @@ struct SweepReadback {
     DevCounters c;
     double dl[2];
     int32_t status;
-    int32_t done;  // the one-launch commit did the commit (0: it left it, see kCommitMaxLoad)
+    int32_t done;  // the one-launch commit did the commit (0: it left it, see commit_max_load)
 };
 
 // the accepted-move list: one (vertex, chunk) item per kMoveChunk edges of

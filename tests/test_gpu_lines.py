@@ -126,3 +126,32 @@ def test_batch_kernel_forms_decide_alike(n, e, Bs):
                 assert (st.n_moves, st.n_accepted, st.n_entries) == \
                        (stats[0].n_moves, stats[0].n_accepted, stats[0].n_entries)
                 assert st.dl_after == stats[0].dl_after
+
+
+# Labels set from outside, more of them changed than one launch commits but
+# less than three times as many: the commit of the pass after is asked about
+# its own moves, and takes the form that they call for.
+@pytest.mark.parametrize("B", [8, 64, 256])
+def test_commit_form_after_labels_set(B):
+    n, m = 20_000, 40_000
+    pg = _graph(n, None, seed=n)  # four edge ends a vertex
+    b = random_labels(n, B, seed=5)
+    one = P.Model(pg, B, b, P.Params.default(seed=6))
+    full = P.Model(pg, B, b, P.Params.default(seed=6, full_rebuild=1))
+    for sw in range(20):
+        one.sweep(sw), full.sweep(sw)
+    lab = one.assignment()
+    pick = np.random.default_rng(7).random(n) < 0.6
+    lab[pick] = random_labels(n, B, seed=8)[pick]
+    assert _launches(lambda: P.sbp_set_assignment(one.h, B, lab)) > 2
+    P.sbp_set_assignment(full.h, B, lab)
+    for sw in range(20, 30):
+        P.sbp_nodal_decide(one.h, sw, 0, n)
+        got = []
+        k = _launches(lambda: got.append(P.sbp_commit(one.h)))
+        c = full.sweep(sw)
+        assert got[0].as_dict() | {"n_recheck": 0} == c.as_dict() | {"n_recheck": 0}
+        acc = got[0].n_accepted
+        load = acc + (acc // 10 if 16 * acc <= m else m // 80) + B * B // 64
+        assert (k == 1) == (load <= 6000 + 32_000 // B), (sw, k, load)
+        _same(one, full)
