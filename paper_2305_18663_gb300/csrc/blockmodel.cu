@@ -519,7 +519,8 @@ __global__ void __launch_bounds__(kThreads, kItemCtas) k_nb_items(GraphDev g, co
 // from outside and committed, the separate kernels and this one, in us):
 //   - blocks, whose prefix rows it builds on 256 warps (2000 vertices, 8000
 //     edges, nothing moved): 66 and 51 at B = 256, 71 and 68 at 384, 74 and 77
-//     at 512;
+//     at 512; with a pass before it and its statistics read (3000 vertices,
+//     40,000 edges), 91 and 67 at 300, 91 and 82 at 500;
 //   - moves: an item costs some 6 ns, an edge end of an update 0.15 ns, an edge
 //     of a recount 0.075 ns, and the blocks' rows add up, against the launches
 //     it saves; commit_max_load is that budget in items.  A pass's commit also
@@ -541,7 +542,7 @@ __global__ void __launch_bounds__(kThreads, kItemCtas) k_nb_items(GraphDev g, co
 // one pass to the next the moves rarely fall by more.
 constexpr int kCommitThreads = 1024;
 constexpr int kCommitCluster = 8;
-constexpr int kCommitMaxB = 256;
+constexpr int kCommitMaxB = 512, kCommitMaxSetB = 256;  // of a pass, of labels set from outside
 constexpr int64_t kCommitMaxEdges = int64_t(1) << 19;
 constexpr int64_t kCommitMaxVertices = int64_t(1) << 16;
 constexpr unsigned long long kCommitTryFactor = 3;
@@ -881,7 +882,7 @@ bool commit_small_fits(const sbp_model *m) {
 }
 
 bool commit_small_load_ok(const sbp_model *m, const DevCounters &c) {
-    return commit_load(c, m->g->m, m->B) <= commit_max_load(m->B);
+    return m->B <= kCommitMaxSetB && commit_load(c, m->g->m, m->B) <= commit_max_load(m->B);
 }
 
 bool commit_small_try_next(const sbp_model *m, const DevCounters &c) {

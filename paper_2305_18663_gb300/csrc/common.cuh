@@ -600,7 +600,7 @@ int update_cells(sbp_model *m, int32_t *cells);  // counts of m->bnew -> counts 
 int launch_prefix(sbp_model *m);                 // P, Pc, degrees, reciprocals from a dense M
 // the whole commit of a small dense model in one launch: whether the model has
 // the form, whether every commit of it is within the form's load, whether
-// these moves are, and the launch (checked: by the kernel, which leaves the
+// these labels set from outside are, and the launch (checked: by the kernel, which leaves the
 // commit and says so in host->done when they are not)
 bool commit_small_ok(const sbp_model *m);
 bool commit_small_fits(const sbp_model *m);

@@ -155,3 +155,20 @@ def test_commit_form_after_labels_set(B):
         load = acc + (acc // 10 if 16 * acc <= m else m // 80) + B * B // 64
         assert (k == 1) == (load <= 6000 + 32_000 // B), (sw, k, load)
         _same(one, full)
+
+
+# the most blocks of the one-launch commit of a pass, few vertices moving
+@pytest.mark.parametrize("B,one_launch", [(257, True), (512, True), (513, False)])
+def test_commit_form_at_many_blocks(B, one_launch):
+    n = 1_500
+    pg = _graph(n, None, seed=n)
+    b = random_labels(n, B, seed=5)
+    one = P.Model(pg, B, b, P.Params.default(seed=6))
+    full = P.Model(pg, B, b, P.Params.default(seed=6, full_rebuild=1))
+    for sw in range(4):
+        P.sbp_nodal_decide(one.h, sw, 0, n)
+        got = []
+        k = _launches(lambda: got.append(P.sbp_commit(one.h)))
+        assert (k == 1) == one_launch, k
+        assert got[0].as_dict() | {"n_recheck": 0} == full.sweep(sw).as_dict() | {"n_recheck": 0}
+        _same(one, full)
