@@ -1815,7 +1815,14 @@ int launch_recheck(sbp_model *m, const DecideArgs &a0, int sms) {
 //   - From 2^19 edges they run on three streams, where the top group's rows
 //     are the long ones; rows of hundreds of edges have a warp each there too,
 //     with twice the warps, and win from some 2^21 edges on (the line: 3 x 2^19).
-//   - B > 1022: half the warps here, none lost there in the first group.
+//   - B > 1022: half the warps here, none lost there in the first group; with a
+//     second and a third group those cost more (B = 1500 and 2048, 100 vertices
+//     of 50 edges and 100 of 300 among 120,000 edges, 30,000 vertices 145, 111,
+//     40,000 162, 147; a heavy tail and 390,000 edges, 25,000 168, 93, 40,000
+//     172, 138; the full run of 20,900 such vertices 58.1 ms, 48.7).
+//   - From 2^19 to 3 x 2^18 edges and beyond 40,000 vertices a heavy tail would
+//     gain (48,395 vertices, 598,074 edges at B = 72, labels set and a sweep 295,
+//     273), a hundred long rows lose more (54,000, 528,000 at B = 72, 59, 95).
 // Both sides in us (groups, small; labels near the planted ones, B = 4 / 1000;
 // B = 2048): only the first group, 6000 vertices 27, 28 / 35, 34; 34, 36; at
 // 20,000 42, 40 / 53, 60; 57, 83; at 60,000 50, 77 / 65, 109; 75, 193.  More
@@ -1830,7 +1837,7 @@ bool small_pass(const sbp_graph *g, const DecideArgs &a, int B) {
     const int64_t n = a.vcount[0] + a.vcount[1] + a.vcount[2];
     const bool half = direct_warps(B) < kWarpsPerCta;
     if (a.vcount[1] + a.vcount[2] == 0) return n <= (half ? 2500 : 5000);
-    if (g->m < kSideStreamEdges && a.vcount[1] >= 64) return n <= (half ? 20000 : 40000);
+    if (g->m < kSideStreamEdges && a.vcount[1] >= 64) return n <= (half && a.vcount[2] < 64 ? 20000 : 40000);
     if (g->m < kSideStreamEdges) return n <= (half ? 10000 : 22000);
     if (!half && a.vcount[2] >= 64 && g->m <= 3 * (int64_t(1) << 18)) return n <= 40000;
     return g->m <= 3 * (int64_t(1) << 19) && n <= (half ? 6000 : 20000);

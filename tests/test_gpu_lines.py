@@ -172,3 +172,26 @@ def test_commit_form_at_many_blocks(B, one_launch):
         assert (k == 1) == one_launch, k
         assert got[0].as_dict() | {"n_recheck": 0} == full.sweep(sw).as_dict() | {"n_recheck": 0}
         _same(one, full)
+
+
+# more than 1022 blocks, rows in the second and in the third group
+@pytest.mark.parametrize("n,one", [(20_001, True), (40_000, True), (40_001, False)])
+def test_pass_form_with_all_groups(n, one):
+    rng = np.random.default_rng(n)
+    v = np.arange(n)
+    mid, far = np.repeat(np.arange(64), 40), np.repeat(np.arange(64, 128), 200)
+    src = np.concatenate([v, v, mid, far])
+    dst = np.concatenate([(v + 1) % n, (v + n // 3) % n, rng.integers(128, n, mid.size + far.size)])
+    pg = P.Graph(n, src.astype(np.int32), dst.astype(np.int32))
+    b = random_labels(n, 1_023, seed=1)
+    prm = P.Params.default(seed=4)
+    whole, parts = P.Model(pg, 1_023, b, prm), P.Model(pg, 1_023, b, prm)
+    for sw in range(2):
+        k = _launches(lambda: P.sbp_nodal_decide(whole.h, sw, 0, n))
+        if sw > 0:
+            assert (k == 1) == one, k
+        for lo, hi in ((0, n // 3), (n // 3, n)):
+            P.sbp_nodal_decide(parts.h, sw, lo, hi)
+        a, c = P.sbp_commit(whole.h), P.sbp_commit(parts.h)
+        assert a.n_moves > 0 and a.as_dict() | {"n_recheck": 0} == c.as_dict() | {"n_recheck": 0}
+    _same(whole, parts)
